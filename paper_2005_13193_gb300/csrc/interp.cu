@@ -1450,33 +1450,27 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
   }
   if (!encode) return false;
   const GridArgs& g = a->g;
-  const cuuint32_t unit[4] = {1, 1, 1, 1};
+  const cuuint32_t unit[3] = {1, 1, 1};
   const cuuint64_t m1 = (cuuint64_t)g.m[1], m2 = (cuuint64_t)g.m[2], rx = (cuuint64_t)g.rx;
-  if (coef_t == PS_F32X4) {
-    const cuuint64_t dims[4] = {4, rx, m1, m2};
-    const cuuint64_t strides[3] = {16, rx * 16, rx * m1 * 16};
-    const cuuint32_t box[4] = {4, (cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
-    return encode(&a->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(a->coef),
-                  dims, strides, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-  }
-  // 16-bit nodes: pairs of nodes (16 bytes) are the inner unit; rx is even
-  const cuuint64_t dims[4] = {8, rx / 2, m1, m2};
-  const cuuint64_t strides[3] = {16, rx * 8, rx * m1 * 8};
-  const cuuint32_t box[4] = {8, (cuuint32_t)a->SX / 2, (cuuint32_t)a->S[1],
-                             (cuuint32_t)a->S[2]};
-  const CUtensorMapDataType t =
-      coef_t == PS_BF16X4 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  if (encode(&a->tmap, t, 4, const_cast<void*>(a->coef), dims, strides, box, unit,
+  if (4 * a->SX > 256) return false;  // a box holds at most 256 values per axis
+  const cuuint64_t dims[3] = {4 * rx, m1, m2};
+  const cuuint32_t box[3] = {4 * (cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
+  const cuuint64_t nb = coef_t == PS_F32X4 ? 16 : 8;  // bytes of a node
+  const cuuint64_t strides[2] = {rx * nb, rx * m1 * nb};
+  const CUtensorMapDataType t = coef_t == PS_F32X4    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                : coef_t == PS_BF16X4 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                      : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  if (encode(&a->tmap, t, 3, const_cast<void*>(a->coef), dims, strides, box, unit,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return false;
-  // the rows' scales (s_u, s_v, s_w, 1): [m2][m1][4] floats
-  const cuuint64_t sdims[3] = {4, m1, m2};
-  const cuuint64_t sstrides[2] = {16, m1 * 16};
-  const cuuint32_t sbox[3] = {4, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
-  return encode(&a->tmap2, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(a->scale),
+  if (coef_t == PS_F32X4) return true;
+  // 16-bit nodes: the rows' scales (s_u, s_v, s_w, 1), [m2][m1][4] floats
+  if (4 * a->S[1] > 256) return false;
+  const cuuint64_t sdims[2] = {4 * m1, m2};
+  const cuuint64_t sstrides[1] = {m1 * 16};
+  const cuuint32_t sbox[2] = {4 * (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
+  return encode(&a->tmap2, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(a->scale),
                 sdims, sstrides, sbox, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;

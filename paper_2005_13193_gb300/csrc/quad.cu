@@ -797,7 +797,7 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done) {
   a.wait_probe = tuning().wait_probe;
   a.tma = 0;
   if constexpr (NodeDtype<Tc>::v >= 0)
-    if (a0.tma && SX <= 256) a.tma = encode_node_halo_map(&a, (ps_dtype)NodeDtype<Tc>::v) ? 1 : 0;
+    if (a0.tma) a.tma = encode_node_halo_map(&a, (ps_dtype)NodeDtype<Tc>::v) ? 1 : 0;
   if constexpr (MODE == 4 && std::is_same<Tc, float4>::value) {
     // the later field's node map in tmap2 (tma = 2)
     if (a.tma == 1 && a.coef2) {

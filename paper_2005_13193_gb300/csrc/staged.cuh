@@ -169,9 +169,9 @@ __device__ __forceinline__ void tma_copy_halo(const CUtensorMap* map, float4* ds
                "r"(bytes)
                : "memory");
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<unsigned long long>(map)), "r"(0), "r"(P0[0]), "r"(P0[1]), "r"(P0[2]),
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(4 * P0[0]), "r"(P0[1]), "r"(P0[2]),
       "r"(smem_u32(mbar))
       : "memory");
 }
@@ -184,9 +184,9 @@ __device__ __forceinline__ void tma_issue_halo(const CUtensorMap* map, float4* d
                "r"(bytes)
                : "memory");
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<unsigned long long>(map)), "r"(0), "r"(P0[0]), "r"(P0[1]), "r"(P0[2]),
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(4 * P0[0]), "r"(P0[1]), "r"(P0[2]),
       "r"(smem_u32(mbar))
       : "memory");
 }
@@ -228,17 +228,17 @@ __device__ __forceinline__ void tma_issue_node16(const CUtensorMap* nodes,
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
                "r"(bytes)
                : "memory");
-  // node pairs are the 16-byte inner unit: x coordinate P0[0] / 2
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(raw)),
-      "l"(reinterpret_cast<unsigned long long>(nodes)), "r"(0), "r"(P0[0] >> 1), "r"(P0[1]),
-      "r"(P0[2]), "r"(smem_u32(mbar))
-      : "memory");
+  // (P0[0] is even: the rows start on 16-byte boundaries)
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(sraw)),
-      "l"(reinterpret_cast<unsigned long long>(scales)), "r"(0), "r"(P0[1]), "r"(P0[2]),
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(raw)),
+      "l"(reinterpret_cast<unsigned long long>(nodes)), "r"(4 * P0[0]), "r"(P0[1]), "r"(P0[2]),
+      "r"(smem_u32(mbar))
+      : "memory");
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(sraw)),
+      "l"(reinterpret_cast<unsigned long long>(scales)), "r"(4 * P0[1]), "r"(P0[2]),
       "r"(smem_u32(mbar))
       : "memory");
 }
