@@ -118,11 +118,11 @@ int64_t ps_coef_row_pitch(int nx, ps_dtype coef_t);
 
 /* Launch-shape knobs (not part of the method):
  *  "brick_kernel" (for the brick-staged calls, bins given): -1 = automatic
- *     (default; 5 for the gradient tensor and for 16-bit coefficients, 0
- *     otherwise), 0 = one CTA per brick, 8 lanes per particle, phases
- *     separated by block barriers, 2 = one CTA per brick, one thread per
- *     particle, 5 = one CTA per brick, four lanes per particle, each holding
- *     one z-row of the stencil in registers (the Heun predictor reuses it
+ *     (default; 5 for three components, 0 for one), 0 = one CTA per brick, 8
+ *     lanes per particle, phases separated by block barriers, 2 = one CTA per
+ *     brick, one thread per particle, 5 = one CTA per brick, each warp on its
+ *     own with 32 particles at a time, four lanes per particle holding one
+ *     z-row of the stencil each in registers (the Heun predictor reuses it
  *     when it stays in its cell); 16-bit node halos stay 16-bit in shared
  *     memory.  Forms a case does not support fall back to 0.
  *  "brick_min_stage" in [0, 2^20] (default 8): bricks holding fewer particles

@@ -893,19 +893,19 @@ __device__ __forceinline__ void brick_phased(const StagedArgs& a, int bin, float
   // no barrier here: phase A of the first round does not read the halo, and
   // the barrier that follows it also publishes the staged halo
   if (a.vec && is_cube11(a)) {
-    stage_halo_vec<Tc, NC, 11>(a, coef, P0, halo, false);
+    stage_halo_vec<Tc, NC, 11>(a, coef, P0, halo, false, a.scale);
     process_brick<Tc, NC, MODE, 11>(a, beg, end, P0, halo, R);
     return;
   }
   if (a.vec && is_cube11_rows12(a)) {
-    stage_halo_vec<Tc, NC, 12>(a, coef, P0, halo, false);
+    stage_halo_vec<Tc, NC, 12>(a, coef, P0, halo, false, a.scale);
     process_brick<Tc, NC, MODE, 12>(a, beg, end, P0, halo, R);
     return;
   }
   if (a.vec)
-    stage_halo_vec<Tc, NC>(a, coef, P0, halo, false);
+    stage_halo_vec<Tc, NC>(a, coef, P0, halo, false, a.scale);
   else
-    stage_halo<Tc, NC>(a, coef, P0, halo, false);
+    stage_halo<Tc, NC>(a, coef, P0, halo, false, a.scale);
   process_brick<Tc, NC, MODE>(a, beg, end, P0, halo, R);
 }
 
@@ -1258,9 +1258,9 @@ __global__ void __launch_bounds__(64) interp_thread(StagedArgs a) {
   const Tc* coef = static_cast<const Tc*>(a.coef);
   float4* halo = smem;
   if (a.vec)
-    stage_halo_vec<Tc, NC>(a, coef, P0, halo);
+    stage_halo_vec<Tc, NC>(a, coef, P0, halo, true, a.scale);
   else
-    stage_halo<Tc, NC>(a, coef, P0, halo);
+    stage_halo<Tc, NC>(a, coef, P0, halo, true, a.scale);
   const GridArgs& g = a.g;
   const int64_t np = a.np;
   const float nanf_ = __int_as_float(0x7fc00000);
@@ -1428,8 +1428,9 @@ ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[
 
 }  // namespace
 
-// Tensor map of the node halo box (4 floats x SX nodes x S[1] rows x S[2]
-// planes) over the PS_F32X4 array; the driver's encoder is looked up once.
+// Tensor map of the halo box over the coefficients (nodes: S[1] x S[2] rows of
+// SX nodes; planar FP32: rows of SX floats of the three components); the
+// driver's encoder is looked up once.
 bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   static bool looked = false;
@@ -1452,7 +1453,19 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
   const GridArgs& g = a->g;
   const cuuint32_t unit[3] = {1, 1, 1};
   const cuuint64_t m1 = (cuuint64_t)g.m[1], m2 = (cuuint64_t)g.m[2], rx = (cuuint64_t)g.rx;
-  if (4 * a->SX > 256) return false;  // a box holds at most 256 values per axis
+  // a box holds at most 256 values per axis
+  if (a->S[1] > 256 || a->S[2] > 256 || (coef_t == PS_F32 ? 1 : 4) * a->SX > 256) return false;
+  if (coef_t == PS_F32) {
+    // planar: [3][m2][m1][rx] floats, the box's three components one behind the other
+    const cuuint64_t pd[4] = {rx, m1, m2, 3};
+    const cuuint64_t ps[3] = {rx * 4, rx * m1 * 4, rx * m1 * m2 * 4};
+    const cuuint32_t pb[4] = {(cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2], 3};
+    const cuuint32_t pu[4] = {1, 1, 1, 1};
+    return encode(&a->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(a->coef), pd, ps,
+                  pb, pu, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  }
   const cuuint64_t dims[3] = {4 * rx, m1, m2};
   const cuuint32_t box[3] = {4 * (cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
   const cuuint64_t nb = coef_t == PS_F32X4 ? 16 : 8;  // bytes of a node
@@ -1502,12 +1515,10 @@ template <> struct DtypeOf<f16x4> { static constexpr int v = PS_F16X4; };
 
 template <typename Tc, int NC, int MODE>
 ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st) {
-  // brick_kernel -1 (default): the measured-faster form per case, the quad
-  // kernel for the gradient tensor and for 16-bit coefficients (planar ones
-  // too, so that both storages of the same values give the same bits), the
-  // phased kernel otherwise
+  // brick_kernel -1 (default): the quad form for three components, the phased
+  // kernel for one
   int k = tuning().brick_kernel;
-  if (k < 0) k = (MODE == 1 || IsQuant<Tc>::value) ? 5 : 0;
+  if (k < 0) k = 5;
   if constexpr (NC == 3 && DtypeOf<Tc>::v >= 0) {
     if (k == 5) {
       bool done = false;

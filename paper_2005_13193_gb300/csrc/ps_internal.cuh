@@ -173,6 +173,25 @@ __device__ __forceinline__ void flag_status(int32_t* st, int code, int64_t idx) 
 __device__ __forceinline__ bool locate(double x, double inv_h, int n, int& cell, float& t) {
   const double s = __dmul_rn(x, inv_h);
   const long long bits = __double_as_longlong(s);
+  {
+    // 0 < s < 2^20 inside the box, the usual case, in 32-bit operations: the
+    // mantissa left-justified in (vh, lo << 12), the integer part in its top
+    // e bits, the next 32 bits the fraction (24 of them kept)
+    const int shi = (int)(bits >> 32);
+    const unsigned lo = (unsigned)bits;
+    const int e = (shi >> 20) - 1023;  // below -1023 for s < 0
+    const unsigned vh = __funnelshift_l(lo, (unsigned)shi, 12);
+    if (e >= -31 && e < 20) {
+      const int ip = e < 0 ? 0 : (int)((((unsigned)shi & 0xfffffu) | 0x100000u) >> (20 - e));
+      const unsigned fr = e < 0 ? ((0x80000000u | (vh >> 1)) >> (-1 - e))
+                                : __funnelshift_l(lo << 12, vh, e);
+      if (ip < n) {
+        cell = ip;
+        t = (float)(fr >> 8) * __int_as_float(0x33800000);
+        return true;
+      }
+    }
+  }
   const int bexp = (int)((bits >> 52) & 0x7ff);
   cell = 0;
   t = 0.f;

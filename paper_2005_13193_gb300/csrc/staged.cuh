@@ -21,6 +21,8 @@ struct StagedArgs {
   int vec;      // 1: halo rows are whole 16-byte vectors inside the array
   int min_stage;  // bricks with fewer particles gather from global memory
   int tma;        // 1: the node halo is one tensor copy described by tmap
+                  // (2: the second field's too, by tmap2)
+  int two;        // 1: the second field's halo is staged beside the first
   int chunked;    // 1: bins are runs of particles (sparse field): no halo
   int wait_probe; // > 0: test knob, a wait on a barrier nothing completes
                   // (this many clocks) follows the halo's own wait
@@ -38,6 +40,8 @@ struct StagedArgs {
   const int64_t* ids_in;
   int64_t* ids_out;
   double dt;
+  double half_dt;
+  double ih32[3];  // 2^32 n/L per axis
   float dtih[3];  // dt * n/L per axis
   int32_t* status;
   // counting pass of the next step's bin sort (NULL = off): each particle's
@@ -219,12 +223,10 @@ __host__ __device__ constexpr bool node16_in_place_ok(int Sz, int PS, int Sy, in
 }
 static_assert(node16_in_place_ok(11, 132, 11, 12), "16-bit node halo cannot widen in place");
 
-__device__ __forceinline__ void tma_issue_node16(const CUtensorMap* nodes,
-                                                 const CUtensorMap* scales, void* raw,
-                                                 void* sraw, unsigned long long* mbar,
-                                                 const int P0[3], unsigned bytes) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)) : "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+__device__ __forceinline__ void tma_copy_node16(const CUtensorMap* nodes,
+                                                const CUtensorMap* scales, void* raw,
+                                                void* sraw, unsigned long long* mbar,
+                                                const int P0[3], unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
                "r"(bytes)
                : "memory");
@@ -241,6 +243,35 @@ __device__ __forceinline__ void tma_issue_node16(const CUtensorMap* nodes,
       "l"(reinterpret_cast<unsigned long long>(scales)), "r"(4 * P0[1]), "r"(P0[2]),
       "r"(smem_u32(mbar))
       : "memory");
+}
+
+__device__ __forceinline__ void tma_issue_node16(const CUtensorMap* nodes,
+                                                 const CUtensorMap* scales, void* raw,
+                                                 void* sraw, unsigned long long* mbar,
+                                                 const int P0[3], unsigned bytes) {
+  tma_init_barrier(mbar);
+  tma_copy_node16(nodes, scales, raw, sraw, mbar, P0, bytes);
+}
+
+// A planar halo (rows of floats, three components; P0[0] is a
+// multiple of 4) or a float4 node halo, on an initialised barrier.
+template <bool PLANAR>
+__device__ __forceinline__ void tma_copy(const CUtensorMap* map, void* dst,
+                                         unsigned long long* mbar, const int P0[3],
+                                         unsigned bytes) {
+  if constexpr (!PLANAR) {
+    tma_copy_halo(map, static_cast<float4*>(dst), mbar, P0, bytes);
+  } else {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
+                 "r"(bytes)
+                 : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<unsigned long long>(map)), "r"(P0[0]), "r"(P0[1]), "r"(P0[2]),
+        "r"(0), "r"(smem_u32(mbar))
+        : "memory");
+  }
 }
 
 // Waits for the barrier's phase of the given parity, giving up after `limit`
@@ -278,7 +309,8 @@ __device__ __forceinline__ int wrap_row(int P, int n) {
 // before storing them so that the loads overlap.
 template <typename Tc, int NC>
 __device__ __forceinline__ void stage_halo(const StagedArgs& a, const Tc* __restrict__ coef,
-                                           const int P0[3], float4* halo, bool sync = true) {
+                                           const int P0[3], float4* halo, bool sync,
+                                           const float* __restrict__ scale) {
   const GridArgs& g = a.g;
   const int Sx = a.S[0], Sy = a.S[1], Sz = a.S[2];
   const bool narrow = Sx <= 16;
@@ -307,12 +339,12 @@ __device__ __forceinline__ void stage_halo(const StagedArgs& a, const Tc* __rest
         float x = 0.f;
         if (act[u]) {
           if constexpr (IsNode16<Tc>::value) {
-            x = node16_value(coef[row * m0 + Px].v[c]) * __ldg(a.scale + row * 4 + c);
+            x = node16_value(coef[row * m0 + Px].v[c]) * __ldg(scale + row * 4 + c);
           } else if constexpr (IsNode4<Tc>::value) {
             x = __ldg(reinterpret_cast<const float*>(coef + row * m0 + Px) + c);
           } else {
             x = (float)CoefLoad<Tc>::ld(coef + c * cs + row * m0 + Px);
-            if (IsQuant<Tc>::value) x *= __ldg(a.scale + c * m2 * m1 + row);
+            if (IsQuant<Tc>::value) x *= __ldg(scale + c * m2 * m1 + row);
           }
         }
         v[u][c] = x;
@@ -365,13 +397,15 @@ template <> struct Vec16<__half> : Vec16Half<__half> {};
 template <typename Tc, int NC, int KS>
 __device__ __forceinline__ void stage_halo_vec_planar(const StagedArgs& a,
                                                       const Tc* __restrict__ coef,
-                                                      const int P0[3], float4* halo, bool sync);
+                                                      const int P0[3], float4* halo, bool sync,
+                                                      const float* __restrict__ scale);
 
 // Node coefficients: one 16-byte load and store per halo point, consecutive
 // threads along the rows.
 template <typename Tc, int KS>
 __device__ __forceinline__ void stage_nodes(const StagedArgs& a, const Tc* __restrict__ coef,
-                                            const int P0[3], float4* halo) {
+                                            const int P0[3], float4* halo,
+                                            const float* __restrict__ scale) {
   const HaloGeo<KS> hg(a);
   const int64_t rx = a.g.rx, m1 = a.g.m[1];
   const Tc* b0 = coef + ((int64_t)P0[2] * m1 + P0[1]) * rx + P0[0];
@@ -382,7 +416,7 @@ __device__ __forceinline__ void stage_nodes(const StagedArgs& a, const Tc* __res
     const int64_t roff = (int64_t)lz * m1 + ly;
     if constexpr (IsNode16<Tc>::value) {
       const Tc n = b0[roff * rx + x];
-      const float4 sc = __ldg(reinterpret_cast<const float4*>(a.scale) +
+      const float4 sc = __ldg(reinterpret_cast<const float4*>(scale) +
                               ((int64_t)P0[2] * m1 + P0[1]) + roff);
       halo[lz * hg.PS + ly * hg.SX + x] =
           make_float4(node16_value(n.v[0]) * sc.x, node16_value(n.v[1]) * sc.y,
@@ -395,19 +429,21 @@ __device__ __forceinline__ void stage_nodes(const StagedArgs& a, const Tc* __res
 
 template <typename Tc, int NC, int KS = 0>
 __device__ __forceinline__ void stage_halo_vec(const StagedArgs& a, const Tc* __restrict__ coef,
-                                               const int P0[3], float4* halo, bool sync = true) {
+                                               const int P0[3], float4* halo, bool sync,
+                                               const float* __restrict__ scale) {
   if constexpr (IsNode4<Tc>::value) {
-    stage_nodes<Tc, KS>(a, coef, P0, halo);
+    stage_nodes<Tc, KS>(a, coef, P0, halo, scale);
     if (sync) __syncthreads();
   } else {
-    stage_halo_vec_planar<Tc, NC, KS>(a, coef, P0, halo, sync);
+    stage_halo_vec_planar<Tc, NC, KS>(a, coef, P0, halo, sync, scale);
   }
 }
 
 template <typename Tc, int NC, int KS>
 __device__ __forceinline__ void stage_halo_vec_planar(const StagedArgs& a,
                                                       const Tc* __restrict__ coef,
-                                                      const int P0[3], float4* halo, bool sync) {
+                                                      const int P0[3], float4* halo, bool sync,
+                                                      const float* __restrict__ scale) {
   constexpr int V = Vec16<Tc>::V;
   constexpr int U = 8 / V;               // rows in flight per thread
   const GridArgs& g = a.g;
@@ -439,7 +475,7 @@ __device__ __forceinline__ void stage_halo_vec_planar(const StagedArgs& a,
       for (int c = 0; c < NC; ++c) {
         float sc = 1.f;
         if (IsQuant<Tc>::value)
-          sc = __ldg(a.scale + ((int64_t)c * m2 + P0[2] + lz) * m1 + P0[1] + ly);
+          sc = __ldg(scale + ((int64_t)c * m2 + P0[2] + lz) * m1 + P0[1] + ly);
         Vec16<Tc>::load(b0 + c * cs + roff, sc, v[c]);
       }
       const int h0 = lz * hg.PS + ly * hg.SX + q * 4;
@@ -469,7 +505,7 @@ __device__ __forceinline__ void stage_halo_vec_planar(const StagedArgs& a,
         if (act[u]) {
           float s = 1.f;
           if (IsQuant<Tc>::value)
-            s = __ldg(a.scale + ((int64_t)c * m2 + P0[2] + lz) * m1 + P0[1] + ly);
+            s = __ldg(scale + ((int64_t)c * m2 + P0[2] + lz) * m1 + P0[1] + ly);
           Vec16<Tc>::load(base + c * cs + roff, s, v[u][c]);
         }
       }

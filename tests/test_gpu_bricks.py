@@ -1,0 +1,82 @@
+"""The quad brick form where its work splits: bricks holding every number of
+particles around a warp's 32 and a block's trip, long bricks, the last bricks of an axis that hold fewer cells, positions on both
+sides of the halo's edge.  Bars as in test_gpu_parity (FP32 interpolation
+1e-5 of the rms velocity, a Heun step dt times that)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2005_13193_gb300 as ps
+from paper_2005_13193_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+TWO_PI = 2 * math.pi
+DEV = "cuda"
+
+
+def _counted_positions(n, brick, counts, seed):
+    """Brick b (x fastest) holds counts[b % len(counts)] particles, the first one
+    of each on the brick's low corner and the second just below its high one."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    nb = [-(-n[d] // brick[d]) for d in range(3)]
+    cols = []
+    for b in range(nb[0] * nb[1] * nb[2]):
+        m = counts[b % len(counts)]
+        o = (b % nb[0], b // nb[0] % nb[1], b // (nb[0] * nb[1]))
+        lo = np.array([o[d] * brick[d] for d in range(3)], dtype=np.float64)[:, None]
+        hi = np.array([min(n[d], (o[d] + 1) * brick[d]) for d in range(3)],
+                      dtype=np.float64)[:, None]
+        u = rng.random((3, m))
+        if m > 0:
+            u[:, 0] = 0.0
+        if m > 1:
+            u[:, 1] = 1.0 - 1e-9
+        cols.append((lo + u * (hi - lo)) * (TWO_PI / np.array(n, dtype=np.float64)[:, None]))
+    return np.concatenate(cols, axis=1)
+
+
+@pytest.mark.parametrize("n,brick", [((32, 16, 24), (8, 8, 8)), ((30, 21, 18), (8, 8, 8)),
+                                     ((16, 130, 8), (2, 60, 2)), ((24, 20, 16), (12, 5, 8))])
+@pytest.mark.parametrize("dtype,bar", [(ps.F32X4, 1e-5), (torch.float32, 1e-5),
+                                       (ps.F16X4, 4e-3)])
+def test_bricks_of_every_fill(n, brick, dtype, bar):
+    counts = [0, 1, 7, 8, 9, 31, 32, 33, 63, 64, 65, 71, 72, 96, 97, 127, 128, 129, 200]
+    field = synth.random_field(n, ncomp=3, seed=5).astype(np.float32)
+    cref = oracle.spline_coeffs(field.astype(np.float64))
+    pos = _counted_positions(n, brick, counts, seed=6)
+    pos = np.ascontiguousarray(
+        pos[:, np.random.Generator(np.random.PCG64(7)).permutation(pos.shape[1])])
+    sf = ps.SplineField.from_field(torch.from_numpy(field).to(DEV), dtype)
+    pg = torch.from_numpy(pos).to(DEV)
+    bins = ps.bin_particles(n, brick, pg)
+    ref, gref = oracle.interp(cref, pos, grad=True)
+    rms, cmax = np.sqrt((ref ** 2).mean()), np.abs(cref).max()
+    st = torch.zeros(4, dtype=torch.int32, device=DEV)
+    vel = sf.interp(pg, bins=bins, status=st)
+    velg, grad = sf.interp(pg, grad=True, bins=bins, status=st)
+    # 16-bit values: half a unit of 2^-11 of the line's scale (below 2 max|c|)
+    # per coefficient, the weights (their derivatives) summing to 1 (2 per axis)
+    q = 0.0 if bar < 1e-4 else 2.0 ** -11 * cmax
+    for v in (vel, velg):
+        assert np.abs(v.cpu().numpy() - ref).max() <= 1e-5 * rms + q
+    for d in range(3):
+        tol = (1e-5 * 3 * cmax + 2 * q) * n[d] / TWO_PI
+        assert np.abs(grad[:, d].cpu().numpy() - gref[:, d]).max() <= tol
+    dt = 0.3 * TWO_PI / max(n)
+    new_ref, u1 = oracle.rk2_step(cref, pos, dt)
+    tr = ps.Tracker(sf, pg.clone(), brick=brick)
+    tr.step(dt)
+    ids = tr.ids.cpu().numpy()
+    if q == 0.0:
+        assert np.abs(tr.pos.cpu().numpy() - new_ref[:, ids]).max() <= dt * 1e-5 * rms + 1e-14
+    # the counts the step took are those of the positions it wrote
+    x1 = tr.pos.clone()
+    off = torch.empty_like(tr.offsets)
+    xs = torch.empty_like(x1)
+    ps.ps_rk2_sort(n, brick, x1, xs, off, tr.ws, counted=True, status=st)
+    np.testing.assert_array_equal(off.cpu().numpy(),
+                                  oracle.bin_particles(n, brick, x1.cpu().numpy())[1])
+    assert ps.ps_status_read(st)[0] == 0
