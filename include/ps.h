@@ -329,6 +329,39 @@ ps_status ps_lagrangian_accel(const ps_grid* grid, ps_dtype coef_t,
                               int32_t* status, void* stream);
 
 /* ------------------------------------------------------------------------ */
+/* ps_interp, ps_interp_hessian and ps_lagrangian_accel with a workspace for */
+/* the results of a permuted call (bin_offsets and perm given).  Storing     */
+/* every particle's values at its own place writes one DRAM sector per value */
+/* once the result rows outgrow the L2; with ws the values are stored in bin */
+/* order and the rows put in place a few at a time.  The same results.       */
+/*   ws: ps_unsort_workspace_size(np, rows) bytes, 256-byte aligned, rows =  */
+/*   3 (vel), 12 (vel and grad), 18 (hess), 3 or 6 (acc, acc and vel); NULL  */
+/*   or too small, or without perm: as the calls above.                      */
+/* ------------------------------------------------------------------------ */
+size_t ps_unsort_workspace_size(int64_t np, int rows);
+ps_status ps_interp_ws(const ps_grid* grid, int ncomp, ps_dtype coef_t,
+                       const void* coef, const float* scale, int64_t np,
+                       const double* pos, const int64_t* perm,
+                       const int32_t* bin_offsets, const int32_t brick[3],
+                       float* vel, float* grad, void* ws, size_t ws_bytes,
+                       int32_t* status, void* stream);
+ps_status ps_interp_hessian_ws(const ps_grid* grid, int ncomp, ps_dtype coef_t,
+                               const void* coef, const float* scale, int64_t np,
+                               const double* pos, const int64_t* perm,
+                               const int32_t* bin_offsets,
+                               const int32_t brick[3], float* hess, void* ws,
+                               size_t ws_bytes, int32_t* status, void* stream);
+ps_status ps_lagrangian_accel_ws(const ps_grid* grid, ps_dtype coef_t,
+                                 const void* coef_n, const float* scale_n,
+                                 const void* coef_np1, const float* scale_np1,
+                                 double dt_field, int64_t np,
+                                 const double* pos, const int64_t* perm,
+                                 const int32_t* bin_offsets,
+                                 const int32_t brick[3], float* acc, float* vel,
+                                 void* ws, size_t ws_bytes, int32_t* status,
+                                 void* stream);
+
+/* ------------------------------------------------------------------------ */
 /* One second-order Runge-Kutta step (Sec. 2.1; Sec. 4.3), Heun's form:     */
 /*   u1 = u(x^n; coef_n);  x* = x^n + dt u1;  u2 = u(x*; coef_np1);         */
 /*   x^{n+1} = x^n + (dt/2)(u1 + u2)                                        */

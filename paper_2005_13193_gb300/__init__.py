@@ -86,6 +86,10 @@ def _ptr(t: Optional[torch.Tensor]):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _nbytes(t: Optional[torch.Tensor]) -> int:
+    return t.numel() * t.element_size() if t is not None else 0
+
+
 def _dev(t: Optional[torch.Tensor], name: str, dtype=None, numel=None):
     if t is None:
         return
@@ -273,9 +277,10 @@ def ps_interp(coef: torch.Tensor, n, pos: torch.Tensor, vel: torch.Tensor,
               scale: Optional[torch.Tensor] = None, perm: Optional[torch.Tensor] = None,
               bin_offsets: Optional[torch.Tensor] = None, brick=None,
               grad: Optional[torch.Tensor] = None, status: Optional[torch.Tensor] = None,
-              L=DEFAULT_L, stream=None):
+              L=DEFAULT_L, stream=None, ws: Optional[torch.Tensor] = None):
     """Operations 2-3 (Sec. 2.2, Eq. (spline)) at positions pos [3][np] -> vel [ncomp][np].
-    n = (nx, ny, nz) of the grid the coefficients belong to."""
+    n = (nx, ny, nz) of the grid the coefficients belong to.  ws (ps_unsort_workspace_size
+    of 3 rows, 12 with grad): with perm, the results go through bin order."""
     _check_coef_shape(coef, n)
     ncomp = _ncomp_of(coef)
     np_ = pos.shape[1]
@@ -287,10 +292,12 @@ def ps_interp(coef: torch.Tensor, n, pos: torch.Tensor, vel: torch.Tensor,
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(grad, "grad", torch.float32, ncomp * 3 * np_)
     _dev(status, "status", torch.int32, 4)
+    _dev(ws, "ws")
     g = make_grid(n, L)
-    _check(_lib().ps_interp(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef), _ptr(scale), np_,
-                            _ptr(pos), _ptr(perm), _ptr(bin_offsets), _brick_arr(brick),
-                            _ptr(vel), _ptr(grad), _ptr(status), _stream(stream)))
+    _check(_lib().ps_interp_ws(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef), _ptr(scale),
+                               np_, _ptr(pos), _ptr(perm), _ptr(bin_offsets), _brick_arr(brick),
+                               _ptr(vel), _ptr(grad), _ptr(ws), _nbytes(ws), _ptr(status),
+                               _stream(stream)))
 
 
 def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Tensor,
@@ -316,10 +323,11 @@ def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Te
 def ps_interp_hessian(coef: torch.Tensor, n, pos: torch.Tensor, hess: torch.Tensor,
                       scale: Optional[torch.Tensor] = None, perm: Optional[torch.Tensor] = None,
                       bin_offsets: Optional[torch.Tensor] = None, brick=None,
-                      status: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None):
+                      status: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None,
+                      ws: Optional[torch.Tensor] = None):
     """Second derivatives of Eq. (spline): hess [ncomp][6][np] (xx, yy, zz, xy, xz, yz).
-    With bin_offsets (and brick, perm as for ps_interp) the stencils come from each
-    brick's staged halo."""
+    With bin_offsets (and brick, perm, ws (18 rows) as for ps_interp) the stencils come
+    from each brick's staged halo."""
     _check_coef_shape(coef, n)
     ncomp = _ncomp_of(coef)
     np_ = pos.shape[1]
@@ -331,10 +339,11 @@ def ps_interp_hessian(coef: torch.Tensor, n, pos: torch.Tensor, hess: torch.Tens
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(status, "status", torch.int32, 4)
     g = make_grid(n, L)
-    _check(_lib().ps_interp_hessian(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef),
-                                    _ptr(scale), np_, _ptr(pos), _ptr(perm), _ptr(bin_offsets),
-                                    _brick_arr(brick), _ptr(hess), _ptr(status),
-                                    _stream(stream)))
+    _dev(ws, "ws")
+    _check(_lib().ps_interp_hessian_ws(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef),
+                                       _ptr(scale), np_, _ptr(pos), _ptr(perm),
+                                       _ptr(bin_offsets), _brick_arr(brick), _ptr(hess), _ptr(ws),
+                                       _nbytes(ws), _ptr(status), _stream(stream)))
 
 
 def ps_lagrangian_accel(coef_n: torch.Tensor, n, pos: torch.Tensor, acc: torch.Tensor,
@@ -343,10 +352,11 @@ def ps_lagrangian_accel(coef_n: torch.Tensor, n, pos: torch.Tensor, acc: torch.T
                         scale_np1: Optional[torch.Tensor] = None,
                         vel: Optional[torch.Tensor] = None, perm: Optional[torch.Tensor] = None,
                         bin_offsets: Optional[torch.Tensor] = None, brick=None,
-                        status: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None):
+                        status: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None,
+                        ws: Optional[torch.Tensor] = None):
     """a = du/dt + (u . grad) u at pos [3][np] -> acc [3][np] (du/dt from two fields).
-    With bin_offsets (and brick, perm as for ps_interp) the stencils of coef_n come from
-    each brick's staged halo."""
+    With bin_offsets (and brick, perm, ws (3 rows, 6 with vel) as for ps_interp) the
+    stencils come from each brick's staged halos."""
     _check_coef_shape(coef_n, n)
     np_ = pos.shape[1]
     _dev(coef_n, "coef_n")
@@ -360,11 +370,13 @@ def ps_lagrangian_accel(coef_n: torch.Tensor, n, pos: torch.Tensor, acc: torch.T
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(status, "status", torch.int32, 4)
     g = make_grid(n, L)
-    _check(_lib().ps_lagrangian_accel(ctypes.byref(g), _coef_type(coef_n), _ptr(coef_n),
-                                      _ptr(scale_n), _ptr(coef_np1), _ptr(scale_np1),
-                                      float(dt_field), np_, _ptr(pos), _ptr(perm),
-                                      _ptr(bin_offsets), _brick_arr(brick), _ptr(acc),
-                                      _ptr(vel), _ptr(status), _stream(stream)))
+    _dev(ws, "ws")
+    _check(_lib().ps_lagrangian_accel_ws(ctypes.byref(g), _coef_type(coef_n), _ptr(coef_n),
+                                         _ptr(scale_n), _ptr(coef_np1), _ptr(scale_np1),
+                                         float(dt_field), np_, _ptr(pos), _ptr(perm),
+                                         _ptr(bin_offsets), _brick_arr(brick), _ptr(acc),
+                                         _ptr(vel), _ptr(ws), _nbytes(ws), _ptr(status),
+                                         _stream(stream)))
 
 
 def ps_rk2_workspace_size(n, brick, np_: int, L=DEFAULT_L) -> int:
@@ -437,6 +449,29 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
     return t
 
 
+# Result rows from this size on go through bin order (see ps_interp_ws): about half
+# the L2, beyond which scattered 4-byte stores reach DRAM one by one.
+_UNSORT_BYTES = 48 << 20
+
+
+def _unsort_ws(bins: Optional["Bins"], np_: int, rows: int, device):
+    """A workspace for the rows of a permuted call, or None where it would not help or
+    does not fit."""
+    if bins is None or bins.perm is None or 4 * rows * np_ < _UNSORT_BYTES:
+        return None
+    try:
+        return workspace(int(_lib().ps_unsort_workspace_size(np_, rows)), device)
+    except torch.cuda.OutOfMemoryError:
+        return None
+
+
+def _on_stream(ws: Optional[torch.Tensor], stream):
+    """Keep a scratch tensor's memory until the work queued on `stream` is done."""
+    if ws is not None and stream is not None:
+        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream)
+                         else torch.cuda.ExternalStream(int(stream)))
+
+
 class SplineField:
     """Padded spline coefficients of a periodic field (Sec. 2.2 Operation 1)."""
 
@@ -479,11 +514,13 @@ class SplineField:
         """Second derivatives at pos: [ncomp][6][np] (xx, yy, zz, xy, xz, yz); with
         `bins` of these positions, from each brick's staged halo."""
         h = torch.empty((self.ncomp, 6, pos.shape[1]), dtype=torch.float32, device=pos.device)
+        ws = _unsort_ws(bins, pos.shape[1], 18, pos.device)
         ps_interp_hessian(self.coef, self.n, pos, h, scale=self.scale,
                           perm=bins.perm if bins is not None else None,
                           bin_offsets=bins.offsets if bins is not None else None,
                           brick=bins.brick if bins is not None else None, status=status,
-                          L=self.L, stream=stream)
+                          L=self.L, stream=stream, ws=ws)
+        _on_stream(ws, stream)
         return h
 
     def acceleration(self, pos: torch.Tensor, later: Optional["SplineField"] = None,
@@ -493,6 +530,7 @@ class SplineField:
         `later` (the field dt_field later) when given; with `bins` of these positions,
         from each brick's staged halo."""
         a = torch.empty((3, pos.shape[1]), dtype=torch.float32, device=pos.device)
+        ws = _unsort_ws(bins, pos.shape[1], 3, pos.device)
         ps_lagrangian_accel(self.coef, self.n, pos, a,
                             coef_np1=later.coef if later is not None else None,
                             dt_field=dt_field, scale_n=self.scale,
@@ -500,7 +538,8 @@ class SplineField:
                             perm=bins.perm if bins is not None else None,
                             bin_offsets=bins.offsets if bins is not None else None,
                             brick=bins.brick if bins is not None else None,
-                            status=status, L=self.L, stream=stream)
+                            status=status, L=self.L, stream=stream, ws=ws)
+        _on_stream(ws, stream)
         return a
 
     def interp(self, pos: torch.Tensor, grad: bool = False, bins: Optional["Bins"] = None,
@@ -509,11 +548,13 @@ class SplineField:
         vel = torch.empty((self.ncomp, np_), dtype=torch.float32, device=pos.device)
         g = (torch.empty((self.ncomp, 3, np_), dtype=torch.float32, device=pos.device)
              if grad else None)
+        ws = _unsort_ws(bins, np_, 12 if grad else 3, pos.device)
         ps_interp(self.coef, self.n, pos, vel, scale=self.scale,
                   perm=bins.perm if bins is not None else None,
                   bin_offsets=bins.offsets if bins is not None else None,
                   brick=bins.brick if bins is not None else None, grad=g, status=status,
-                  L=self.L, stream=stream)
+                  L=self.L, stream=stream, ws=ws)
+        _on_stream(ws, stream)
         return (vel, g) if grad else vel
 
 
@@ -598,7 +639,7 @@ class Tracker:
 class InterpFn(torch.autograd.Function):
     """u = I(pos; spline(field)) with the hand-written adjoint:
     d/dpos via the spline derivative, d/dfield via scatter-add + the transposed
-    (= same, symmetric) periodic solves."""
+    (= same, symmetric) periodic solves.  Enough particles are binned first."""
 
     @staticmethod
     def forward(ctx, pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L):
@@ -612,7 +653,7 @@ class InterpFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g_vel):
         (pos,) = ctx.saved_tensors
-        sf = ctx.sf
+        sf, bins = ctx.sf, ctx.bins
         g_vel = g_vel.contiguous().float()
         want_pos = ctx.needs_input_grad[0]
         want_field = ctx.needs_input_grad[1]

@@ -563,9 +563,9 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
       const int node = WPack<CT>::node(wq, geo) + k * geo.PS;
       const int hrow = IsNode16<Tc>::value ? (WPack<CT>::l2(wq) + k) * geo.Sy + WPack<CT>::l1(wq) : 0;
       float vq[16][3];
+      float out[NOut<MODE>::v];
       if (wq >= 0) fetch_halo<Tc, CT>(vq, halo, node, hrow, geo);
       else fetch_global<Tc>(vq, cq, k, g, coef, a.scale);
-      float out[NOut<MODE>::v];
       if constexpr (MODE == 0) quad_sum<false>(vq, tq, k, out);
       if constexpr (MODE == 1) quad_sum<true>(vq, tq, k, out);
       if constexpr (MODE == 3) quad_sum_hess(vq, tq, k, out);
@@ -634,16 +634,17 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
     // -- 3: lane i finishes particle i
     const float nanf_ = __int_as_float(0x7fc00000);
     if (v && !ok) flag_status(a.status, PS_DEV_NONFINITE_POS, pp);
+    const int oo = a.slot_out ? c0 + lane : pp;  // where the results go
     if constexpr (MODE <= 1) {
       if (v) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) a.vel[c * np + pp] = ok ? res[c] : nanf_;
+        for (int c = 0; c < 3; ++c) a.vel[c * np + oo] = ok ? res[c] : nanf_;
         if (MODE == 1) {
 #pragma unroll
           for (int c = 0; c < 3; ++c)
 #pragma unroll
             for (int d = 0; d < 3; ++d)
-              a.grad[(c * 3 + d) * np + pp] =
+              a.grad[(c * 3 + d) * np + oo] =
                   ok ? __fmul_rn(res[(MODE == 1 ? 3 : 0) * (1 + d) + c], g.inv_hf[d]) : nanf_;
         }
       }
@@ -658,7 +659,7 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
         for (int c = 0; c < 3; ++c)
 #pragma unroll
           for (int e = 0; e < 6; ++e)
-            a.grad[(c * 6 + e) * np + pp] = ok ? __fmul_rn(res[3 * e + c], sc[e]) : nanf_;
+            a.grad[(c * 6 + e) * np + oo] = ok ? __fmul_rn(res[3 * e + c], sc[e]) : nanf_;
       }
     }
     if constexpr (MODE == 4) {
@@ -670,8 +671,8 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
           acc = __fmaf_rn(__fmul_rn(res[6 + c], g.inv_hf[1]), res[1], acc);
           acc = __fmaf_rn(__fmul_rn(res[9 + c], g.inv_hf[2]), res[2], acc);
           if (second) acc = __fmaf_rn(__fsub_rn(res[12 + c], res[c]), (float)a.dt, acc);
-          a.grad[c * np + pp] = ok ? acc : nanf_;
-          if (a.vel) a.vel[c * np + pp] = ok ? res[c] : nanf_;
+          a.grad[c * np + oo] = ok ? acc : nanf_;
+          if (a.vel) a.vel[c * np + oo] = ok ? res[c] : nanf_;
         }
       }
     }

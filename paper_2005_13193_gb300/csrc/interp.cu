@@ -1514,7 +1514,8 @@ template <> struct DtypeOf<bf16x4> { static constexpr int v = PS_BF16X4; };
 template <> struct DtypeOf<f16x4> { static constexpr int v = PS_F16X4; };
 
 template <typename Tc, int NC, int MODE>
-ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st) {
+ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st,
+                        float* rows_ws = nullptr) {
   // brick_kernel -1 (default): the quad form for three components, the phased
   // kernel for one
   int k = tuning().brick_kernel;
@@ -1522,7 +1523,7 @@ ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st) {
   if constexpr (NC == 3 && DtypeOf<Tc>::v >= 0) {
     if (k == 5) {
       bool done = false;
-      ps_status rc = launch_quad(a, (ps_dtype)DtypeOf<Tc>::v, MODE, st, &done);
+      ps_status rc = launch_quad(a, (ps_dtype)DtypeOf<Tc>::v, MODE, st, &done, rows_ws);
       if (rc || done) return rc;
     }
   }
@@ -1766,11 +1767,29 @@ ps_status rk2_launch_staged(const ps_grid* grid, const int32_t brick[3], int E,
 
 using namespace ps;
 
+// The workspace for `rows` result rows in bin order, if the caller gave one
+// that holds them and there is a permutation to undo; else NULL (the results
+// are stored where they belong, one particle at a time).
+static float* result_rows(const int64_t* perm, int64_t np, int rows, void* ws, size_t ws_bytes) {
+  if (!perm || !ws || (reinterpret_cast<uintptr_t>(ws) & 255)) return nullptr;
+  return ws_bytes >= ps_unsort_workspace_size(np, rows) ? static_cast<float*>(ws) : nullptr;
+}
+
 extern "C" ps_status ps_interp(const ps_grid* grid, int ncomp, ps_dtype coef_t,
                                const void* coef, const float* scale, int64_t np,
                                const double* pos, const int64_t* perm,
                                const int32_t* bin_offsets, const int32_t brick[3],
                                float* vel, float* grad, int32_t* status, void* stream) {
+  return ps_interp_ws(grid, ncomp, coef_t, coef, scale, np, pos, perm, bin_offsets, brick, vel,
+                      grad, nullptr, 0, status, stream);
+}
+
+extern "C" ps_status ps_interp_ws(const ps_grid* grid, int ncomp, ps_dtype coef_t,
+                                  const void* coef, const float* scale, int64_t np,
+                                  const double* pos, const int64_t* perm,
+                                  const int32_t* bin_offsets, const int32_t brick[3],
+                                  float* vel, float* grad, void* ws, size_t ws_bytes,
+                                  int32_t* status, void* stream) {
   ps_status rc = validate_grid(grid);
   if (rc) return rc;
   if (ncomp != 1 && ncomp != 3) return fail(PS_ERR_INVALID_ARG, "ncomp must be 1 or 3");
@@ -1826,7 +1845,10 @@ extern "C" ps_status ps_interp(const ps_grid* grid, int ncomp, ps_dtype coef_t,
       return PS_ERR_UNSUPPORTED;
     } else {
       if (ncomp == 3)
-        return grad ? launch_staged<Tc, 3, 1>(a, smem, st) : launch_staged<Tc, 3, 0>(a, smem, st);
+        return grad ? launch_staged<Tc, 3, 1>(a, smem, st,
+                                              result_rows(perm, np, 12, ws, ws_bytes))
+                    : launch_staged<Tc, 3, 0>(a, smem, st,
+                                              result_rows(perm, np, 3, ws, ws_bytes));
       return grad ? launch_staged<Tc, 1, 1>(a, smem, st) : launch_staged<Tc, 1, 0>(a, smem, st);
     }
   });
@@ -1888,8 +1910,8 @@ static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* 
                               const float* scale, const void* coef2, const float* scale2,
                               double inv_dt, int64_t np, const double* pos,
                               const int64_t* perm, const int32_t* bin_offsets,
-                              const int32_t brick[3], float* out, float* vel, int32_t* status,
-                              int mode, cudaStream_t st, bool* done) {
+                              const int32_t brick[3], float* out, float* vel, float* rows_ws,
+                              int32_t* status, int mode, cudaStream_t st, bool* done) {
   *done = false;
   StagedArgs a{};
   size_t smem;
@@ -1908,7 +1930,7 @@ static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* 
   a.vel = vel;
   a.dt = inv_dt;
   a.status = status;
-  return launch_quad(a, coef_t, mode, st, done);
+  return launch_quad(a, coef_t, mode, st, done, rows_ws);
 }
 
 extern "C" ps_status ps_interp_hessian(const ps_grid* grid, int ncomp, ps_dtype coef_t,
@@ -1916,6 +1938,16 @@ extern "C" ps_status ps_interp_hessian(const ps_grid* grid, int ncomp, ps_dtype 
                                        const double* pos, const int64_t* perm,
                                        const int32_t* bin_offsets, const int32_t brick[3],
                                        float* hess, int32_t* status, void* stream) {
+  return ps_interp_hessian_ws(grid, ncomp, coef_t, coef, scale, np, pos, perm, bin_offsets, brick,
+                              hess, nullptr, 0, status, stream);
+}
+
+extern "C" ps_status ps_interp_hessian_ws(const ps_grid* grid, int ncomp, ps_dtype coef_t,
+                                          const void* coef, const float* scale, int64_t np,
+                                          const double* pos, const int64_t* perm,
+                                          const int32_t* bin_offsets, const int32_t brick[3],
+                                          float* hess, void* ws, size_t ws_bytes,
+                                          int32_t* status, void* stream) {
   ps_status rc = validate_grid(grid);
   if (rc) return rc;
   if (ncomp != 1 && ncomp != 3) return fail(PS_ERR_INVALID_ARG, "ncomp must be 1 or 3");
@@ -1931,7 +1963,8 @@ extern "C" ps_status ps_interp_hessian(const ps_grid* grid, int ncomp, ps_dtype 
   if (bin_offsets && ncomp == 3 && coef_t != PS_F64) {
     bool done = false;
     rc = staged_extra(grid, coef_t, coef, scale, nullptr, nullptr, 0.0, np, pos, perm,
-                      bin_offsets, brick, hess, nullptr, status, 3, st, &done);
+                      bin_offsets, brick, hess, nullptr, result_rows(perm, np, 18, ws, ws_bytes),
+                      status, 3, st, &done);
     if (rc || done) return rc;
   }
   GridArgs g = make_grid_args(grid, coef_t);
@@ -1955,6 +1988,19 @@ extern "C" ps_status ps_lagrangian_accel(const ps_grid* grid, ps_dtype coef_t,
                                          const int64_t* perm, const int32_t* bin_offsets,
                                          const int32_t brick[3], float* acc, float* vel,
                                          int32_t* status, void* stream) {
+  return ps_lagrangian_accel_ws(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, dt_field, np,
+                                pos, perm, bin_offsets, brick, acc, vel, nullptr, 0, status,
+                                stream);
+}
+
+extern "C" ps_status ps_lagrangian_accel_ws(const ps_grid* grid, ps_dtype coef_t,
+                                            const void* coef_n, const float* scale_n,
+                                            const void* coef_np1, const float* scale_np1,
+                                            double dt_field, int64_t np, const double* pos,
+                                            const int64_t* perm, const int32_t* bin_offsets,
+                                            const int32_t brick[3], float* acc, float* vel,
+                                            void* ws, size_t ws_bytes, int32_t* status,
+                                            void* stream) {
   ps_status rc = validate_grid(grid);
   if (rc) return rc;
   if ((rc = check_coef(coef_t, coef_n, scale_n))) return rc;
@@ -1971,7 +2017,8 @@ extern "C" ps_status ps_lagrangian_accel(const ps_grid* grid, ps_dtype coef_t,
   if (bin_offsets && coef_t != PS_F64) {
     bool done = false;
     rc = staged_extra(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, inv_dt, np, pos, perm,
-                      bin_offsets, brick, acc, vel, status, 4, st, &done);
+                      bin_offsets, brick, acc, vel, result_rows(perm, np, vel ? 6 : 3, ws, ws_bytes),
+                      status, 4, st, &done);
     if (rc || done) return rc;
   }
   GridArgs g = make_grid_args(grid, coef_t);

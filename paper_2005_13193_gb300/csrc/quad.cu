@@ -87,7 +87,7 @@ bool halo_map(StagedArgs* a) {
 }
 
 template <typename Tc, int MODE>
-ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done) {
+ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done, float* rows_ws) {
   StagedArgs a = a0;
   constexpr bool n16 = IsNode16<Tc>::value;
   if (a.E != 0 || a.S[1] > 1023 || a.S[2] > 1023) return PS_OK;  // not handled here
@@ -133,9 +133,20 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done) {
   }
   *done = true;
   const int threads = a.two ? 128 : 64;
+  // results by way of bin order: vel, then the gradient's or the second
+  // derivatives' rows
+  constexpr int rows = MODE == 1 ? 9 : MODE == 3 ? 18 : MODE == 4 ? 3 : 0;
+  const bool unsort = rows_ws && a.perm && (MODE <= 1 || MODE == 3 || MODE == 4);
+  if (unsort) {
+    a.slot_out = 1;
+    a.vel = a0.vel ? rows_ws : nullptr;
+    a.grad = rows_ws + (a0.vel ? 3 * a.np : 0);
+  }
   kern<<<dim3((unsigned)a.b.nb[0], (unsigned)a.b.nb[1], (unsigned)a.b.nb[2]), threads, smem, st>>>(
       a);
-  return check_launch("quad_kernel");
+  ps_status rc = check_launch("quad_kernel");
+  if (rc || !unsort) return rc;
+  return unsort_launch(a.np, a.perm, rows_ws, a0.vel, a0.vel ? 3 : 0, a0.grad, rows, st);
 }
 
 }  // namespace
@@ -144,16 +155,16 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done) {
 // F32/BF16/F16.  *done stays false where it does not apply (E != 0, a halo
 // above the shared memory), and the caller takes another form.
 ps_status launch_quad(const StagedArgs& a, ps_dtype coef_t, int mode, cudaStream_t st,
-                      bool* done) {
+                      bool* done, float* rows_ws) {
   *done = false;
   auto go = [&](auto tag) -> ps_status {
     using Tc = decltype(tag);
     switch (mode) {
-      case 0: return launch_quad_t<Tc, 0>(a, st, done);
-      case 1: return launch_quad_t<Tc, 1>(a, st, done);
-      case 2: return launch_quad_t<Tc, 2>(a, st, done);
-      case 3: return launch_quad_t<Tc, 3>(a, st, done);
-      default: return launch_quad_t<Tc, 4>(a, st, done);
+      case 0: return launch_quad_t<Tc, 0>(a, st, done, rows_ws);
+      case 1: return launch_quad_t<Tc, 1>(a, st, done, rows_ws);
+      case 2: return launch_quad_t<Tc, 2>(a, st, done, rows_ws);
+      case 3: return launch_quad_t<Tc, 3>(a, st, done, rows_ws);
+      default: return launch_quad_t<Tc, 4>(a, st, done, rows_ws);
     }
   };
   switch (coef_t) {

@@ -54,6 +54,7 @@ struct StagedArgs {
   // high word of the double 2^30 L/n per axis: |x| has a smaller high word
   // (sign cleared) only if |x n/L| < 2^30, read without an FP64 operation
   int xguard_hi[3];
+  int slot_out;       // 1: results at the particle's slot in bin order, not at perm[slot]
   CUtensorMap tmap;   // node halo box (valid when tma == 1)
   CUtensorMap tmap2;  // 16-bit nodes: the box of the halo rows' scales
 };
@@ -65,9 +66,21 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t);
 // The quad-per-particle brick kernel (quad.cu) for three components; mode 0
 // velocities, 1 with the gradient tensor, 2 fused Heun step, 3 second
 // derivatives (into a.grad), 4 Lagrangian acceleration (into a.grad; a.dt
-// holds 1 / dt_field).  Leaves *done false where it does not apply.
+// holds 1 / dt_field).  With a permutation and a workspace for the result rows (modes 0, 1, 3, 4) the
+// kernel stores in bin order and the rows are put in place afterwards.
+// Leaves *done false where it does not apply.
 ps_status launch_quad(const StagedArgs& a, ps_dtype coef_t, int mode, cudaStream_t st,
-                      bool* done);
+                      bool* done, float* rows_ws = nullptr);
+// Rows in bin order -> rows in the particles' order (unsort.cu): n0 rows to
+// d0, the next n1 to d1.
+ps_status unsort_launch(int64_t np, const int64_t* perm, const float* src, float* d0, int n0,
+                        float* d1, int n1, cudaStream_t st);
+
+// The scatter of a binned cotangent onto a cleared field (adjoint.cu).
+ps_status scatter_bricks_launch(const ps_grid* grid, const int32_t brick[3], int64_t np,
+                                const double* pos, const int64_t* perm, const int32_t* offs,
+                                const float* gvel, float* gfield, int32_t* status,
+                                void* ws, size_t ws_bytes, cudaStream_t st, bool* done);
 
 #ifdef __CUDACC__
 namespace {

@@ -1,0 +1,65 @@
+// Rows of results written in bin order -> rows in the particles' own order.
+// A brick kernel that follows a permutation stores every value of a particle
+// at a random place of its row; with more rows than the L2 holds, each 4-byte
+// store goes to DRAM as a sector of its own.  Here the brick kernel stores in
+// bin order (full lines), and the rows are then scattered a few at a time, so
+// that the group of rows being written stays in the L2 until its sectors are
+// whole.
+#include <algorithm>
+
+#include "ps_internal.cuh"
+
+namespace ps {
+namespace {
+
+constexpr int kUnsortThreads = 256, kUnsortItems = 4;
+// Bytes of result rows in flight: well under the 129 MB L2, of which the two
+// dies hold a part each (4 M particles: three rows).
+constexpr int64_t kUnsortGroupBytes = 48ll << 20;
+
+// Rows [blockIdx.y * group, + group): entry perm[s] of row r takes entry s of
+// src row r.  Rows r < n0 go to d0, the others to d1.
+__global__ void __launch_bounds__(kUnsortThreads)
+    unsort_rows(int64_t np, const int64_t* __restrict__ perm, const float* __restrict__ src,
+                float* __restrict__ d0, int n0, float* __restrict__ d1, int rows, int group) {
+  int64_t p[kUnsortItems];
+  const int64_t s0 = (int64_t)blockIdx.x * (kUnsortThreads * kUnsortItems) + threadIdx.x;
+#pragma unroll
+  for (int u = 0; u < kUnsortItems; ++u) {
+    const int64_t s = s0 + u * kUnsortThreads;
+    p[u] = s < np ? __ldg(perm + s) : -1;
+  }
+  const int r1 = min(rows, ((int)blockIdx.y + 1) * group);
+  for (int r = blockIdx.y * group; r < r1; ++r) {
+    const float* sr = src + r * np;
+    float* dr = r < n0 ? d0 + r * np : d1 + (r - n0) * np;
+    float v[kUnsortItems];
+#pragma unroll
+    for (int u = 0; u < kUnsortItems; ++u)
+      if (p[u] >= 0) v[u] = __ldcs(sr + s0 + u * kUnsortThreads);
+#pragma unroll
+    for (int u = 0; u < kUnsortItems; ++u)
+      if (p[u] >= 0) dr[p[u]] = v[u];
+  }
+}
+
+}  // namespace
+
+ps_status unsort_launch(int64_t np, const int64_t* perm, const float* src, float* d0, int n0,
+                        float* d1, int n1, cudaStream_t st) {
+  const int rows = n0 + n1;
+  if (np <= 0 || rows <= 0) return PS_OK;
+  const int group =
+      (int)std::min<int64_t>(rows, std::max<int64_t>(1, kUnsortGroupBytes / (4 * np)));
+  const int64_t per = kUnsortThreads * kUnsortItems;
+  const dim3 grid((unsigned)((np + per - 1) / per), (unsigned)((rows + group - 1) / group));
+  unsort_rows<<<grid, kUnsortThreads, 0, st>>>(np, perm, src, d0, n0, d1, rows, group);
+  return check_launch("unsort_rows");
+}
+
+}  // namespace ps
+
+extern "C" size_t ps_unsort_workspace_size(int64_t np, int rows) {
+  if (np < 0 || rows < 0) return 0;
+  return ps::align_up((size_t)np * (size_t)rows * sizeof(float), 256);
+}

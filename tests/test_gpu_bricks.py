@@ -80,3 +80,31 @@ def test_bricks_of_every_fill(n, brick, dtype, bar):
     np.testing.assert_array_equal(off.cpu().numpy(),
                                   oracle.bin_particles(n, brick, x1.cpu().numpy())[1])
     assert ps.ps_status_read(st)[0] == 0
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, ps.BF16X4])
+def test_results_by_way_of_bin_order(dtype):
+    # with a workspace a permuted call stores in bin order and puts the rows in
+    # place afterwards: the same bits, for every row count and a ragged last block
+    n, brick = (40, 24, 17), (8, 8, 8)
+    field = synth.random_field(n, ncomp=3, seed=15).astype(np.float32)
+    sf = ps.SplineField.from_field(torch.from_numpy(field).to(DEV), dtype)
+    for np_ in (1, 1023, 5000):
+        pg = torch.from_numpy(synth.uniform_particles(np_, seed=16) * 1.3 - 0.5).to(DEV)
+        bins = ps.bin_particles(n, brick, pg)
+        kw = dict(scale=sf.scale, perm=bins.perm, bin_offsets=bins.offsets, brick=brick)
+
+        def both(rows, call):
+            outs = []
+            for ws in (None, ps.workspace(ps._lib().ps_unsort_workspace_size(np_, rows))):
+                o = torch.full((rows, np_), math.nan, device=DEV)
+                call(o, ws)
+                outs.append(o)
+            assert not torch.isnan(outs[0]).any() and torch.equal(*outs)
+
+        both(3, lambda o, ws: ps.ps_interp(sf.coef, n, pg, o, ws=ws, **kw))
+        both(12, lambda o, ws: ps.ps_interp(sf.coef, n, pg, o[:3], grad=o[3:], ws=ws, **kw))
+        both(18, lambda o, ws: ps.ps_interp_hessian(sf.coef, n, pg, o, ws=ws, **kw))
+        kw["scale_n"] = kw.pop("scale")
+        both(6, lambda o, ws: ps.ps_lagrangian_accel(sf.coef, n, pg, o[3:], coef_np1=sf.coef,
+                                                     scale_np1=sf.scale, vel=o[:3], ws=ws, **kw))
