@@ -293,6 +293,26 @@ ps_status ps_interp_backward(const ps_grid* grid, int ncomp, ps_dtype coef_t,
                              size_t ws_bytes, int32_t* status, void* stream);
 
 /* ------------------------------------------------------------------------ */
+/* ps_interp_backward for binned particles (bin_offsets required; perm and  */
+/* brick as for ps_interp): with three components the position gradient is  */
+/* gathered in bin order and the scatter of a brick's particles is summed   */
+/* in shared memory before it goes to g_field.  The same results up to the  */
+/* order of the field gradient's sums.  One component: ps_interp_backward.  */
+/*   ws (optional): ps_backward_workspace_size bytes (0: not used), 256-byte */
+/*   aligned: the bricks' sums are added up from there instead of by atomics. */
+/* ------------------------------------------------------------------------ */
+size_t ps_backward_workspace_size(const ps_grid* grid, const int32_t brick[3]);
+ps_status ps_interp_backward_binned(const ps_grid* grid, int ncomp,
+                                    ps_dtype coef_t, const void* coef,
+                                    const float* scale, int64_t np,
+                                    const double* pos, const int64_t* perm,
+                                    const int32_t* bin_offsets,
+                                    const int32_t brick[3], const float* g_vel,
+                                    double* g_pos, float* g_field, void* ws,
+                                    size_t ws_bytes, int32_t* status,
+                                    void* stream);
+
+/* ------------------------------------------------------------------------ */
 /* Second derivatives of the interpolant (the cubic spline is twice         */
 /* continuously differentiable, Sec. 2.2): the 64-term sum of Eq. (spline)  */
 /* with d2b/dt2 = (1-t, 3t-2, 1-3t, t) along one axis (or db/dt along two), */

@@ -303,8 +303,12 @@ def ps_interp(coef: torch.Tensor, n, pos: torch.Tensor, vel: torch.Tensor,
 def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Tensor,
                        g_pos: Optional[torch.Tensor] = None, g_field: Optional[torch.Tensor] = None,
                        scale: Optional[torch.Tensor] = None, status: Optional[torch.Tensor] = None,
-                       L=DEFAULT_L, stream=None):
-    """Adjoint of ps_interp and of the coefficient solve."""
+                       L=DEFAULT_L, stream=None, perm: Optional[torch.Tensor] = None,
+                       bin_offsets: Optional[torch.Tensor] = None, brick=None,
+                       ws: Optional[torch.Tensor] = None):
+    """Adjoint of ps_interp and of the coefficient solve.  With bin_offsets (and brick,
+    perm as for ps_interp) both gradients are formed brick by brick; ws
+    (ps_backward_workspace_size) holds the bricks' sums."""
     _check_coef_shape(coef, n)
     ncomp = _ncomp_of(coef)
     np_ = pos.shape[1]
@@ -315,9 +319,21 @@ def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Te
     _dev(g_field, "g_field", torch.float32, ncomp * n[0] * n[1] * n[2])
     _dev(status, "status", torch.int32, 4)
     g = make_grid(n, L)
+    if bin_offsets is not None:
+        _dev(perm, "perm", torch.int64, np_)
+        _dev(bin_offsets, "bin_offsets", torch.int32)
+        _check(_lib().ps_interp_backward_binned(
+            ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef), _ptr(scale), np_, _ptr(pos),
+            _ptr(perm), _ptr(bin_offsets), _brick_arr(brick), _ptr(g_vel), _ptr(g_pos),
+            _ptr(g_field), _ptr(ws), _nbytes(ws), _ptr(status), _stream(stream)))
+        return
     _check(_lib().ps_interp_backward(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef),
                                      _ptr(scale), np_, _ptr(pos), _ptr(g_vel), _ptr(g_pos),
                                      _ptr(g_field), None, 0, _ptr(status), _stream(stream)))
+
+
+def ps_backward_workspace_size(n, brick, L=DEFAULT_L) -> int:
+    return int(_lib().ps_backward_workspace_size(ctypes.byref(make_grid(n, L)), _brick_arr(brick)))
 
 
 def ps_interp_hessian(coef: torch.Tensor, n, pos: torch.Tensor, hess: torch.Tensor,
@@ -636,6 +652,13 @@ class Tracker:
         self._counted = mode >= 2 and self.brick is not None
 
 
+# Particles of one differentiable call from which, and per brick of 8^3 cells on average
+# from which, binning them first pays (forward and both gradients go brick by brick).
+_FN_BRICK = (8, 8, 8)
+_FN_MIN_PARTICLES = 50_000
+_FN_MIN_PER_BRICK = 8
+
+
 class InterpFn(torch.autograd.Function):
     """u = I(pos; spline(field)) with the hand-written adjoint:
     d/dpos via the spline derivative, d/dfield via scatter-add + the transposed
@@ -644,9 +667,17 @@ class InterpFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L):
         sf = SplineField.from_field(field.detach().float(), torch.float32, L)
-        vel = sf.interp(pos.detach())
+        x = pos.detach()
+        bins = None
+        nbins = math.prod(-(-sf.n[d] // _FN_BRICK[d]) for d in range(3))
+        if (sf.ncomp == 3 and x.shape[1] >= max(_FN_MIN_PARTICLES, _FN_MIN_PER_BRICK * nbins)
+                and x.shape[1] < 2**31):
+            bins = bin_particles(sf.n, _FN_BRICK, x, L)
+            bins.bin_of = None  # the backward needs the order alone
+        vel = sf.interp(x, bins=bins)
         ctx.save_for_backward(pos)
         ctx.sf = sf
+        ctx.bins = bins
         ctx.field_dtype = field.dtype
         return vel
 
@@ -660,9 +691,18 @@ class InterpFn(torch.autograd.Function):
         g_pos = torch.empty_like(pos) if want_pos else None
         g_field = (torch.empty((sf.ncomp, sf.n[2], sf.n[1], sf.n[0]), dtype=torch.float32,
                                device=pos.device) if want_field else None)
+        ws = None
+        if bins is not None and want_field:
+            try:
+                ws = workspace(ps_backward_workspace_size(sf.n, bins.brick, sf.L), pos.device)
+            except torch.cuda.OutOfMemoryError:
+                pass  # the bricks' sums then go to the field by atomics
         if want_pos or want_field:
             ps_interp_backward(sf.coef, sf.n, pos.detach(), g_vel, g_pos, g_field,
-                               scale=sf.scale, L=sf.L)
+                               scale=sf.scale, L=sf.L, ws=ws,
+                               perm=bins.perm if bins is not None else None,
+                               bin_offsets=bins.offsets if bins is not None else None,
+                               brick=bins.brick if bins is not None else None)
         if g_field is not None:
             g_field = g_field.to(ctx.field_dtype)
         return g_pos, g_field, None

@@ -63,6 +63,9 @@ SIGNATURES = {
     "ps_lagrangian_accel_ws": (_I, [_GP, _I, _P, _P, _P, _P, _D, _I64, _P, _P, _P, _P, _P, _P,
                                     _P, _SZ, _P, _P]),
     "ps_interp_backward": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _SZ, _P, _P]),
+    "ps_backward_workspace_size": (_SZ, [_GP, _P]),
+    "ps_interp_backward_binned": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _P, _P, _P,
+                                       _SZ, _P, _P]),
     "ps_interp_hessian": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _P, _P]),
     "ps_lagrangian_accel": (_I, [_GP, _I, _P, _P, _P, _P, _D, _I64, _P, _P, _P, _P, _P, _P,
                                 _P, _P]),

@@ -1903,6 +1903,51 @@ extern "C" ps_status ps_interp_backward(const ps_grid* grid, int ncomp, ps_dtype
   return PS_OK;
 }
 
+extern "C" ps_status ps_interp_backward_binned(
+    const ps_grid* grid, int ncomp, ps_dtype coef_t, const void* coef, const float* scale,
+    int64_t np, const double* pos, const int64_t* perm, const int32_t* bin_offsets,
+    const int32_t brick[3], const float* g_vel, double* g_pos, float* g_field, void* ws,
+    size_t ws_bytes, int32_t* status, void* stream) {
+  ps_status rc = validate_grid(grid);
+  if (rc) return rc;
+  if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
+  if (!bin_offsets) return fail(PS_ERR_INVALID_ARG, "bin_offsets is required");
+  BrickArgs ba;
+  if ((rc = make_brick_args(grid, brick, &ba))) return rc;
+  cudaStream_t st = as_stream(stream);
+  const bool three = ncomp == 3 && np > 0 && np < ((int64_t)1 << 31) && pos && g_vel;
+  bool have_pos = false, have_field = false;
+  if (three && g_pos) {
+    // the unbinned kernel, its particles taken in bin order: neighbouring
+    // quads then find one another's rows in the caches
+    if ((rc = check_coef(coef_t, coef, scale))) return rc;
+    const GridArgs g = make_grid_args(grid, coef_t);
+    rc = with_coef_type(coef_t, [&](auto tag) -> ps_status {
+      using Tc = decltype(tag);
+      interp_direct<Tc, 3, 2><<<quad_blocks(np), 256, 0, st>>>(
+          g, static_cast<const Tc*>(coef), scale, np, pos, perm, nullptr, nullptr, g_vel, g_pos,
+          status);
+      return check_launch("interp_backward_pos");
+    });
+    if (rc) return rc;
+    have_pos = true;
+  }
+  if (three && g_field) {
+    rc = check_cuda(cudaMemsetAsync(g_field, 0, sizeof(float) * grid_volume(grid) * ncomp, st),
+                    "g_field memset");
+    if (rc) return rc;
+    if ((rc = scatter_bricks_launch(grid, brick, np, pos, perm, bin_offsets, g_vel, g_field,
+                                    status, ws, ws_bytes, st, &have_field)))
+      return rc;
+    if (have_field && (rc = solve_unpadded_inplace_f32(grid, ncomp, g_field, st))) return rc;
+  }
+  // what the brick forms do not take (and the argument errors) goes the direct way
+  if ((!g_pos || have_pos) && (!g_field || have_field) && three) return PS_OK;
+  return ps_interp_backward(grid, ncomp, coef_t, coef, scale, np, pos, g_vel,
+                            have_pos ? nullptr : g_pos, have_field ? nullptr : g_field, nullptr, 0,
+                            status, stream);
+}
+
 // Brick-staged form of the second derivatives (mode 3) or the Lagrangian
 // acceleration (mode 4) by the quad kernel; *done false where it does not
 // apply (the caller then gathers directly).

@@ -108,3 +108,60 @@ def test_results_by_way_of_bin_order(dtype):
         kw["scale_n"] = kw.pop("scale")
         both(6, lambda o, ws: ps.ps_lagrangian_accel(sf.coef, n, pg, o[3:], coef_np1=sf.coef,
                                                      scale_np1=sf.scale, vel=o[:3], ws=ws, **kw))
+
+
+@pytest.mark.parametrize("n,brick", [((24, 16, 40), (8, 8, 8)), ((9, 21, 5), (8, 8, 8)),
+                                     ((3, 4, 5), (8, 8, 8)), ((20, 18, 12), (5, 7, 3)),
+                                     ((40, 8, 8), (20, 4, 4)), ((32, 16, 24), (8, 8, 8))])
+@pytest.mark.parametrize("crowd", [False, True])
+def test_binned_adjoint(n, brick, crowd):
+    # a cell holding more particles than one warp takes (512), bricks below and
+    # above the staging threshold, positions outside the box, stale bins
+    rng = np.random.Generator(np.random.PCG64(25))
+    field = synth.random_field(n, ncomp=3, seed=26).astype(np.float32)
+    cref = oracle.spline_coeffs(field.astype(np.float64))
+    pos = np.ascontiguousarray(rng.random((3, 4000)) * TWO_PI * 1.5 - 1.0)
+    if crowd:
+        pos[:, :2500] = (rng.random((3, 2500)) + 1.0) * TWO_PI / np.array(n)[:, None]
+    w = rng.standard_normal((3, pos.shape[1])).astype(np.float32)
+    gp_ref, gf_ref = oracle.interp_backward(cref, pos, w.astype(np.float64))
+    sf = ps.SplineField.from_field(torch.from_numpy(field).to(DEV), torch.float32)
+    pg, wg = torch.from_numpy(pos).to(DEV), torch.from_numpy(w).to(DEV)
+    bins = ps.bin_particles(n, brick, pg)
+    stale = ps.bin_particles(n, brick, (pg + 0.7).contiguous())
+    cmax, wsum = np.abs(cref).max(), np.abs(w).sum(0).max()
+    direct = torch.empty_like(pg)
+    ps.ps_interp_backward(sf.coef, n, pg, wg, direct, None)
+    ws = ps.workspace(ps.ps_backward_workspace_size(n, brick))
+    for b, w_ in ((bins, None), (bins, ws), (stale, ws)):
+        g_pos = torch.empty_like(pg)
+        g_field = torch.empty((3,) + tuple(reversed(n)), dtype=torch.float32, device=DEV)
+        st = torch.zeros(4, dtype=torch.int32, device=DEV)
+        ps.ps_interp_backward(sf.coef, n, pg, wg, g_pos, g_field, status=st, perm=b.perm,
+                              bin_offsets=b.offsets, brick=brick, ws=w_)
+        assert torch.equal(g_pos, direct)  # the same sums in the same order
+        assert ps.ps_status_read(st)[0] == 0
+        for d in range(3):
+            tol = 1e-5 * 3 * (n[d] / TWO_PI) * cmax * wsum
+            assert np.abs(g_pos[d].cpu().numpy() - gp_ref[d]).max() <= tol
+        gf = g_field.cpu().numpy()
+        assert np.abs(gf - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
+
+
+def test_autograd_bins_enough_particles():
+    n = (32, 24, 16)
+    field = synth.random_field(n, ncomp=3, seed=35).astype(np.float32)
+    cref = oracle.spline_coeffs(field.astype(np.float64))
+    pos = synth.uniform_particles(60_000, seed=36)
+    w = np.random.Generator(np.random.PCG64(37)).standard_normal((3, 60_000)).astype(np.float32)
+    gp_ref, gf_ref = oracle.interp_backward(cref, pos, w.astype(np.float64))
+    x = torch.from_numpy(pos).to(DEV).requires_grad_()
+    f = torch.from_numpy(field).to(DEV).requires_grad_()
+    u = ps.interp_autograd(x, f)
+    ref = oracle.interp(cref, pos)
+    assert np.abs(u.detach().cpu().numpy() - ref).max() <= 1e-5 * np.sqrt((ref ** 2).mean())
+    gp, gf = torch.autograd.grad(u, (x, f), torch.from_numpy(w).to(DEV))
+    for d in range(3):
+        tol = 1e-5 * 3 * (n[d] / TWO_PI) * np.abs(cref).max() * np.abs(w).sum(0).max()
+        assert np.abs(gp[d].cpu().numpy() - gp_ref[d]).max() <= tol
+    assert np.abs(gf.cpu().numpy() - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
