@@ -88,6 +88,8 @@ void layout(ps_plan* p) {
   p->ws_bytes = align_up(c.used, 256);
 }
 
+bool cube(const ps_plan* p) { return p->brick[0] == 8 && p->brick[1] == 8 && p->brick[2] == 8; }
+
 template <typename T>
 T* at(void* ws, size_t off) {
   return reinterpret_cast<T*>(static_cast<char*>(ws) + off);
@@ -251,7 +253,7 @@ ps_status enqueue_persistent(ps_plan* p, double* pos, int64_t* ids, int nsteps, 
                     "batch barrier memset");
   if (rc) return rc;
   return staged_batch_persistent(
-      p->coef_t, at<char>(ws, p->off_args), at<int32_t>(ws, p->off_binbase),
+      p->coef_t, cube(p), at<char>(ws, p->off_args), at<int32_t>(ws, p->off_binbase),
       at<BinField>(ws, p->off_bintab), p->nfields, p->total_bins, p->np_total, nsteps, pos, ids,
       at<double>(ws, p->off_pos), ids ? at<int64_t>(ws, p->off_ids) : nullptr,
       at<int32_t>(ws, p->off_binof), at<int32_t>(ws, p->off_rank),
@@ -286,7 +288,7 @@ ps_status enqueue_step(ps_plan* p, double* pos, int64_t* ids, void* ws, int32_t*
                             at<int32_t>(ws, p->off_scan), status, st);
   }
   if (rc) return rc;
-  return staged_batch_launch(p->coef_t, at<char>(ws, p->off_args),
+  return staged_batch_launch(p->coef_t, cube(p), at<char>(ws, p->off_args),
                              at<int32_t>(ws, p->off_binbase), p->h_args.data(), p->bin_base.data(),
                              p->nfields, p->total_bins, p->smem, false, st);
 }
@@ -368,7 +370,7 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
       (rc = check_cuda(cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking),
                        "capture stream")))
     return rc;
-  if ((rc = staged_batch_launch(p->coef_t, nullptr, nullptr, nullptr, nullptr, 0, 0, p->smem, true,
+  if ((rc = staged_batch_launch(p->coef_t, cube(p), nullptr, nullptr, nullptr, nullptr, 0, 0, p->smem, true,
                                 p->cap)))
     return rc;
   if ((rc = check_cuda(cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal),

@@ -415,11 +415,9 @@ __global__ void __launch_bounds__(256) rk2_direct(GridArgs g, const Tc* __restri
 // round (kRecords), stored field-major so that neither the per-axis writers
 // nor the 8-lane readers conflict on banks:
 //   b[d][i]    float4  b_0..3(t_d) of particle i along axis d
-//   u[i]       float4  (u, v, w, ok) result of the last gather
 //   db[d][i]   float4  b'_0..3(t_d)   (gradient mode only)
 //   loc[d][i]  int     brick-local stencil start along d, -1 = outside halo
 //   cell[d][i] int     global cell along d, -1 = position not finite
-//   nbc[d][i]  int     brick of the new position along d (Heun step only)
 // 80 particles per round: a brick of the mid density (64 particles on
 // average, Poisson) rarely needs a second, mostly empty round, and the 240
 // (particle, axis) tasks still fit two per thread.
@@ -427,27 +425,24 @@ constexpr int kRecords = 80;   // particles per round
 constexpr int kThreads = 128;  // threads per brick CTA
 
 struct Recs {
-  float4* f;  // b[3], u, then db[3] in gradient mode
-  int* ip;    // lw, cell[3], then nbc[3] in the Heun step
+  float4* f;  // b[3], then db[3] in gradient mode
+  int* ip;    // lw, cell[3]
   __device__ __forceinline__ float4* b(int d) const { return f + d * kRecords; }
-  __device__ __forceinline__ float4* u() const { return f + 3 * kRecords; }
-  __device__ __forceinline__ float4* db(int d) const { return f + (4 + d) * kRecords; }
+  __device__ __forceinline__ float4* db(int d) const { return f + (3 + d) * kRecords; }
   // byte d of lw[i]: brick-local stencil start along d, -1 outside the halo,
   // -2 position not finite
   __device__ __forceinline__ int* lw() const { return ip; }
   __device__ __forceinline__ int* cell(int d) const { return ip + (1 + d) * kRecords; }
-  __device__ __forceinline__ int* nbc(int d) const { return ip + (4 + d) * kRecords; }
 };
 __host__ __device__ constexpr size_t rec_bytes(bool grad) {
-  return (size_t)kRecords * (grad ? 7 * sizeof(float4) + 4 * sizeof(int)
-                                  : 4 * sizeof(float4) + 7 * sizeof(int));
+  return (size_t)kRecords * ((grad ? 6 : 3) * sizeof(float4) + 4 * sizeof(int));
 }
 
 template <bool GRAD>
 __device__ __forceinline__ Recs carve_recs(void* base) {
   Recs r;
   r.f = static_cast<float4*>(base);
-  r.ip = reinterpret_cast<int*>(r.f + (GRAD ? 7 : 4) * kRecords);
+  r.ip = reinterpret_cast<int*>(r.f + (GRAD ? 6 : 3) * kRecords);
   return r;
 }
 
@@ -487,14 +482,14 @@ __device__ __forceinline__ bool gather8(const float4* __restrict__ halo, int PS,
                                         const Tc* __restrict__ coef,
                                         const float* __restrict__ scale, int q, int kh,
                                         float out[NC], float dx[NC], float dy[NC],
-                                        float dz[NC], bool staged_ok = true) {
+                                        float dz[NC]) {
   const float bxq = reinterpret_cast<const float*>(R.b(0))[4 * i + q];
   const float4 by = R.b(1)[i];
   const float2 bzp = reinterpret_cast<const float2*>(R.b(2))[2 * i + kh];
   const float bz[2] = {bzp.x, bzp.y};
   const int w = R.lw()[i];
   const bool ok = (__vcmpeq4(w, 0xfefefefe) & 0x00ffffff) == 0;
-  const bool inh = staged_ok && (w & 0x00808080) == 0;
+  const bool inh = (w & 0x00808080) == 0;
   float4 dby = make_float4(0.f, 0.f, 0.f, 0.f);
   float dbz[2] = {0.f, 0.f};
   if (GRAD) {
@@ -510,39 +505,21 @@ __device__ __forceinline__ bool gather8(const float4* __restrict__ halo, int PS,
     const int lx = (signed char)(w & 0xff), ly = (signed char)((w >> 8) & 0xff),
               lz = (signed char)((w >> 16) & 0xff);
     const float4* hp = halo + (lz + kh) * PS + ly * Sx + lx + q;
-    if constexpr (NC == 3 && !GRAD) {
-      // u and v as one packed pair (two FP32 FMAs per instruction, each
-      // rounded as fmaf), w alone
-      float2 auv = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int kk = 0; kk < 2; ++kk) {
+    for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 v = hp[2 * kk * PS + j * Sx];
-          const float w = f4get(by, j) * bz[kk];
-          auv = __ffma2_rn(make_float2(w, w), make_float2(v.x, v.y), auv);
-          acc[2] = fmaf(w, v.z, acc[2]);
-        }
-      }
-      acc[0] = auv.x;
-      acc[1] = auv.y;
-    } else {
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = hp[2 * kk * PS + j * Sx];
+        const float vv[3] = {v.x, v.y, v.z};
+        const float w = f4get(by, j) * bz[kk];
 #pragma unroll
-      for (int kk = 0; kk < 2; ++kk) {
+        for (int c = 0; c < NC; ++c) acc[c] = fmaf(w, vv[c], acc[c]);
+        if (GRAD) {
+          const float wy = f4get(dby, j) * bz[kk], wz = f4get(by, j) * dbz[kk];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 v = hp[2 * kk * PS + j * Sx];
-          const float vv[3] = {v.x, v.y, v.z};
-          const float w = f4get(by, j) * bz[kk];
-#pragma unroll
-          for (int c = 0; c < NC; ++c) acc[c] = fmaf(w, vv[c], acc[c]);
-          if (GRAD) {
-            const float wy = f4get(dby, j) * bz[kk], wz = f4get(by, j) * dbz[kk];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-              accy[c] = fmaf(wy, vv[c], accy[c]);
-              accz[c] = fmaf(wz, vv[c], accz[c]);
-            }
+          for (int c = 0; c < NC; ++c) {
+            accy[c] = fmaf(wy, vv[c], accy[c]);
+            accz[c] = fmaf(wz, vv[c], accz[c]);
           }
         }
       }
@@ -554,27 +531,9 @@ __device__ __forceinline__ bool gather8(const float4* __restrict__ halo, int PS,
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float w = f4get(by, j) * bz[kk];
-        // a node's components by one load, the values load_coef would give
-        float nv[3] = {0.f, 0.f, 0.f};
-        if constexpr (IsNode4<Tc>::value && NC == 3) {
-          const int64_t row = (int64_t)(az + kh + 2 * kk) * g.m[1] + ay + j;
-          if constexpr (IsNode16<Tc>::value) {
-            const Tc n = coef[row * g.rx + ax + q];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) nv[c] = node16_value(n.v[c]) * __ldg(scale + row * 4 + c);
-          } else {
-            const float4 n = __ldg(reinterpret_cast<const float4*>(coef) + row * g.rx + ax + q);
-            nv[0] = n.x;
-            nv[1] = n.y;
-            nv[2] = n.z;
-          }
-        }
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          const float v = (IsNode4<Tc>::value && NC == 3)
-                              ? nv[c]
-                              : (float)load_coef<Tc>(coef, scale, g, c, az + kh + 2 * kk, ay + j,
-                                                     ax + q);
+          const float v = (float)load_coef<Tc>(coef, scale, g, c, az + kh + 2 * kk, ay + j, ax + q);
           acc[c] = fmaf(w, v, acc[c]);
           if (GRAD) {
             accy[c] = fmaf(f4get(dby, j) * bz[kk], v, accy[c]);
@@ -584,17 +543,8 @@ __device__ __forceinline__ bool gather8(const float4* __restrict__ halo, int PS,
       }
     }
   }
-  if constexpr (NC == 3) {
-    // the butterfly over the group with u and v packed (each sum rounded as
-    // the scalar one)
-    const float2 uv = group_sum2<8>(__fmul2_rn(make_float2(bxq, bxq), make_float2(acc[0], acc[1])));
-    out[0] = uv.x;
-    out[1] = uv.y;
-    out[2] = group_sum<8>(bxq * acc[2]);
-  } else {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) out[c] = group_sum<8>(bxq * acc[c]);
-  }
+  for (int c = 0; c < NC; ++c) out[c] = group_sum<8>(bxq * acc[c]);
   if (GRAD) {
     const float dbxq = reinterpret_cast<const float*>(R.db(0))[4 * i + q];
 #pragma unroll
@@ -611,20 +561,12 @@ __device__ __forceinline__ bool gather8(const float4* __restrict__ halo, int PS,
 // of kRecords:
 //   A  one thread per (particle, axis): locate (exact FP64 index arithmetic),
 //      basis along the axis, brick-local index;
-//   B  8 lanes per particle: gather and sum (writes the result or u1);
-//   A' (Heun) one thread per (particle, axis): predictor cell in FP32;
-//   B' second gather (u2);
-//   C  one thread per (particle, axis): FP64 position update and stores.
+//   B  8 lanes per particle: gather, sum and store.
 template <typename Tc, int NC, int MODE, int KS = 0>
 __device__ __forceinline__ void process_brick(const StagedArgs& a, int beg, int end,
                                               const int P0[3], const float4* halo,
-                                              const Recs& R,
-                                              unsigned long long* mbar = nullptr,
-                                              const unsigned char* raw16 = nullptr,
-                                              unsigned parity = 0,
-                                              unsigned long long* probe = nullptr) {
+                                              const Recs& R) {
   constexpr bool GRAD = MODE == 1;
-  bool copied = true;  // the halo's tensor copy completed (or there is none)
   const GridArgs& g = a.g;
   const Tc* coef = static_cast<const Tc*>(a.coef);
   const int tid = threadIdx.x, lane = tid & 31;
@@ -632,83 +574,21 @@ __device__ __forceinline__ void process_brick(const StagedArgs& a, int beg, int 
   const int warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int64_t np = a.np;
   const float nanf_ = __int_as_float(0x7fc00000);
-  constexpr int TPT = (3 * kRecords + kThreads - 1) / kThreads;  // tasks per thread
   const HaloGeo<KS> hg(a);
 
   for (int cb = beg; cb < end; cb += kRecords) {
     const int m = min(kRecords, end - cb);
     // phase A: tasks (particle i, axis d), task = d * m + i
-    int ti[TPT], td[TPT], tcell[TPT];
-    float tt[TPT];
-    double tx[TPT];
-    int64_t tp[TPT];
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      const int task = tid + k * kThreads;
-      td[k] = task < m ? 0 : (task < 2 * m ? 1 : (task < 3 * m ? 2 : -1));
-      ti[k] = task - max(td[k], 0) * m;
-      tcell[k] = 0;
-      tt[k] = 0.f;
-      tx[k] = 0.0;
-      tp[k] = 0;
-      if (td[k] >= 0) {
-        const int i = ti[k], d = td[k];
-        tp[k] = a.perm ? a.perm[cb + i] : (int64_t)(cb + i);
-        tx[k] = a.pos_in[d * np + tp[k]];
-        const bool ok = locate(tx[k], g.inv_h[d], g.n[d], tcell[k], tt[k]);
-        write_axis<GRAD>(R, i, d, tcell[k], tt[k], ok, sel3(P0, d),
-                         d == 0 ? hg.Sx : (d == 1 ? hg.Sy : hg.Sz));
-      }
+    for (int task = tid; task < 3 * m; task += kThreads) {
+      const int d = task < m ? 0 : (task < 2 * m ? 1 : 2), i = task - d * m;
+      const int64_t p = a.perm ? a.perm[cb + i] : (int64_t)(cb + i);
+      int cell;
+      float t;
+      const bool ok = locate(a.pos_in[d * np + p], g.inv_h[d], g.n[d], cell, t);
+      write_axis<GRAD>(R, i, d, cell, t, ok, sel3(P0, d),
+                       d == 0 ? hg.Sx : (d == 1 ? hg.Sy : hg.Sz));
     }
     __syncthreads();
-    // the barrier above also ordered the mbarrier's initialisation before
-    // these waits; a copy that does not complete in time is reported and the
-    // brick's particles read global memory (one decision for the whole
-    // block: the 16-bit widening below is shared)
-    if (mbar && cb == beg) {
-      bool done = tma_wait(mbar, parity);
-      if (done && probe) done = tma_wait(probe, 0, a.wait_probe);
-      copied = __syncthreads_and(done);
-      if (!copied && threadIdx.x == 0) flag_status(a.status, PS_DEV_TIMEOUT, beg);
-    }
-    // (16-bit node copies come only with the 8^3 halo of 12-node rows)
-    if constexpr (IsNode16<Tc>::value && KS == 12) {
-      if (raw16 && cb == beg) {
-        // the copied 16-bit nodes and their rows' scales -> float4 halo in
-        // the same buffer, slice by slice; the copy's rows are SX nodes long,
-        // the halo's rows too (dense planes)
-        const Tc* nodes = reinterpret_cast<const Tc*>(raw16);
-        const float4* scl = reinterpret_cast<const float4*>(
-            raw16 + (node16_scale_offset(hg.Sz, hg.PS, hg.Sy) -
-                     node16_raw_offset(hg.Sz, hg.PS, hg.Sy, hg.SX)));
-        float4* h = const_cast<float4*>(halo);
-        constexpr int npts = HaloGeo<KS>::Sz * HaloGeo<KS>::Sy * HaloGeo<KS>::SX;
-        constexpr int per = (npts + kNode16Slices - 1) / kNode16Slices;
-        constexpr int kPer = (per + kThreads - 1) / kThreads;  // nodes per thread per slice
-#pragma unroll 1
-        for (int sl = 0; sl < kNode16Slices; ++sl) {
-          const int lo = sl * per, hi = min(npts, lo + per);
-          float4 v[kPer];
-#pragma unroll
-          for (int k = 0; k < kPer; ++k) {
-            const int it = lo + threadIdx.x + k * kThreads;
-            if (it < hi) {
-              const Tc n = nodes[it];
-              const float4 sc = scl[it / hg.SX];
-              v[k] = make_float4(node16_value(n.v[0]) * sc.x, node16_value(n.v[1]) * sc.y,
-                                 node16_value(n.v[2]) * sc.z, 0.f);
-            }
-          }
-          __syncthreads();
-#pragma unroll
-          for (int k = 0; k < kPer; ++k) {
-            const int it = lo + threadIdx.x + k * kThreads;
-            if (it < hi) h[it] = v[k];
-          }
-        }
-        __syncthreads();
-      }
-    }
     // phase B: gathers, 8 lanes per particle; the loop is uniform per warp
     // (the butterfly uses full-warp shuffles), idle groups redo record b4
     for (int b4 = warp * 4; b4 < m; b4 += nwarps * 4) {
@@ -716,136 +596,31 @@ __device__ __forceinline__ void process_brick(const StagedArgs& a, int beg, int 
       const bool vi = i < m;
       float u[NC], dx[NC], dy[NC], dz[NC];
       const bool oki = gather8<Tc, NC, GRAD>(halo, hg.PS, hg.SX, R, vi ? i : b4, g, coef, a.scale,
-                                             q, kh, u, dx, dy, dz, copied);
+                                             q, kh, u, dx, dy, dz);
       if (!vi) continue;
-      if constexpr (MODE <= 1) {
-        const int64_t pi = a.perm ? a.perm[cb + i] : (int64_t)(cb + i);
+      const int64_t pi = a.perm ? a.perm[cb + i] : (int64_t)(cb + i);
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
-          if (sub == c) a.vel[(int64_t)c * np + pi] = oki ? u[c] : nanf_;
-        if (GRAD && a.grad) {
+      for (int c = 0; c < NC; ++c)
+        if (sub == c) a.vel[(int64_t)c * np + pi] = oki ? u[c] : nanf_;
+      if (GRAD && a.grad) {
 #pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            if (sub == 3) a.grad[((int64_t)c * 3 + 0) * np + pi] = oki ? dx[c] : nanf_;
-            if (sub == 4) a.grad[((int64_t)c * 3 + 1) * np + pi] = oki ? dy[c] : nanf_;
-            if (sub == 5) a.grad[((int64_t)c * 3 + 2) * np + pi] = oki ? dz[c] : nanf_;
-          }
-        }
-        if (sub == 7 && !oki) flag_status(a.status, PS_DEV_NONFINITE_POS, pi);
-      } else {
-        if (sub == 0) R.u()[i] = make_float4(u[0], u[1], u[2], __int_as_float(oki ? 1 : 0));
-      }
-    }
-    __syncthreads();
-    if constexpr (MODE == 2) {
-    // phase A': predictor located in FP32 relative to the stage-1 cell
-    float tu1[TPT];
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      tu1[k] = 0.f;
-      if (td[k] >= 0) {
-        const int i = ti[k], d = td[k];
-        const float4 r = R.u()[i];
-        const bool ok = __float_as_int(r.w) != 0;
-        tu1[k] = f4get(r, d);
-        float t2 = tt[k] + (ok ? tu1[k] * a.dtih[d] : 0.f);
-        float fl = floorf(t2);
-        if (!(fabsf(fl) < 1.0e9f)) fl = 0.f;
-        t2 = fminf(fmaxf(t2 - fl, 0.f), 1.f);
-        int c = tcell[k] + (int)fl;
-        if (c < 0 || c >= g.n[d]) {
-          c %= g.n[d];
-          if (c < 0) c += g.n[d];
-        }
-        write_axis<false>(R, i, d, c, t2, ok, sel3(P0, d), d == 0 ? hg.Sx : (d == 1 ? hg.Sy : hg.Sz));
-        if (a.coef2 && ok)  // second field: its coefficients are not staged
-          reinterpret_cast<signed char*>(R.lw())[4 * i + d] = (signed char)-1;
-        // the predictor's fraction waits in nbc for phase C (the same task
-        // reads it there before it writes the slot)
-        if (a.next_counts) R.nbc(d)[i] = __float_as_int(t2);
-      }
-    }
-    __syncthreads();
-    // phase B': second gathers
-    const Tc* cf2 = a.coef2 ? static_cast<const Tc*>(a.coef2) : coef;
-    const float* sc2 = a.coef2 ? a.scale2 : a.scale;
-    for (int b4 = warp * 4; b4 < m; b4 += nwarps * 4) {
-      const int i = b4 + (lane >> 3);
-      const bool vi = i < m;
-      float u[NC], dx[NC], dy[NC], dz[NC];
-      const bool oki = gather8<Tc, NC, false>(halo, hg.PS, hg.SX, R, vi ? i : b4, g, cf2, sc2, q,
-                                              kh, u, dx, dy, dz, copied);
-      if (vi && sub == 0) R.u()[i] = make_float4(u[0], u[1], u[2], __int_as_float(oki ? 1 : 0));
-    }
-    __syncthreads();
-    // phase C: FP64 position update, one thread per (particle, axis); with
-    // next_counts the new brick coordinate along the axis goes to nbc
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      if (td[k] >= 0) {
-        const int i = ti[k], d = td[k];
-        const float4 r = R.u()[i];
-        const bool ok = __float_as_int(r.w) != 0;
-        const int64_t pp = tp[k];
-        const double xn = ok ? fma(a.dt * 0.5, (double)(tu1[k] + f4get(r, d)), tx[k])
-                             : __longlong_as_double(0x7ff8000000000000ll);
-        a.pos_out[d * np + pp] = xn;
-        if (a.vel) a.vel[d * np + pp] = ok ? tu1[k] : nanf_;
-        if (d == 0) {
-          if (a.ids_out) a.ids_out[pp] = a.ids_in[pp];
-          if (!ok) flag_status(a.status, PS_DEV_NONFINITE_POS, pp);
-        }
-        if (a.next_counts) {
-          // The new cell: the predictor's cell plus the floor of its fraction
-          // plus the corrector's displacement dt (u2 - u1) / 2 in cells, in
-          // FP32 (x^{n+1} = x* + dt (u2 - u1) / 2).  That floor is the exact
-          // one wherever the sum lies 2^-10 or more from a cell face and
-          // |x n/L| < 2^30: the FP32 and FP64 roundings on both routes stay
-          // below 1e-6 cell.  Elsewhere (and for positions that are not
-          // finite) the FP64 location decides.
-          const float w = __int_as_float(R.nbc(d)[i]) +
-                          0.5f * a.dtih[d] * (f4get(r, d) - tu1[k]);
-          const float fl = floorf(w), fr = w - fl;
-          int c;
-          if (ok && fr >= 0x1p-10f && fr <= 1.f - 0x1p-10f && fabsf(fl) <= 2.f &&
-              (__double2hiint(tx[k]) & 0x7fffffff) < a.xguard_hi[d]) {
-            const int nd = g.n[d];
-            c = R.cell(d)[i] + (int)fl;  // in [-2, n + 1], n >= 3
-            c = c < 0 ? c + nd : (c >= nd ? c - nd : c);
-          } else {
-            float tn;
-            if (!locate(xn, g.inv_h[d], g.n[d], c, tn)) c = -1;
-          }
-          R.nbc(d)[i] = c < 0 ? -1 : (a.bshift[d] >= 0 ? c >> a.bshift[d] : c / a.b.B[d]);
+        for (int c = 0; c < NC; ++c) {
+          if (sub == 3) a.grad[((int64_t)c * 3 + 0) * np + pi] = oki ? dx[c] : nanf_;
+          if (sub == 4) a.grad[((int64_t)c * 3 + 1) * np + pi] = oki ? dy[c] : nanf_;
+          if (sub == 5) a.grad[((int64_t)c * 3 + 2) * np + pi] = oki ? dz[c] : nanf_;
         }
       }
+      if (sub == 7 && !oki) flag_status(a.status, PS_DEV_NONFINITE_POS, pi);
     }
     __syncthreads();
-    // phase D: the next step's counting, one thread per particle in the last
-    // warps, which hold fewer (particle, axis) tasks in phases A and C than
-    // the first ones (nothing below reads these records before the next
-    // round's phase C, several barriers on)
-    constexpr int kCountWarps = (kRecords + 31) / 32;
-    if (a.next_counts && warp >= nwarps - kCountWarps) {
-      const int i = tid - (nwarps - kCountWarps) * 32;
-      const bool vi = i < m;
-      const int64_t pp = vi ? (a.perm ? a.perm[cb + i] : (int64_t)(cb + i)) : 0;
-      int key = vi ? bin_of_coords(a.b, R.nbc(0)[i], R.nbc(1)[i], R.nbc(2)[i]) : 0;
-      if (a.next_runs > 0 && key >= 0) key = (int)((int64_t)key * a.next_runs / a.b.nbins);
-      count_into_bin(a.next_counts, a.next_bin, a.status, vi, pp, key, a.next_key_base);
-    }
-    }  // MODE == 2
   }
-  // a copy still in flight must land before the block's memory is released
-  if (!copied) tma_wait(mbar, parity);
 }
 
 // Phased form of one brick: stage the halo (unless the brick holds fewer than
 // min_stage particles, whose stencils are then read from global memory), then
-// the location / gather / update phases of process_brick.
-template <typename Tc, int NC, int MODE, bool TMA = false>
-__device__ __forceinline__ void brick_phased(const StagedArgs& a, int bin, float4* smem,
-                                             const StagedArgs* maps = nullptr) {
+// the location and gather phases of process_brick.
+template <typename Tc, int NC, int MODE>
+__device__ __forceinline__ void brick_phased(const StagedArgs& a, int bin, float4* smem) {
   const int beg = a.offs[bin], end = a.offs[bin + 1];
   if (beg >= end) return;
   const int nbx = a.b.nb[0], nby = a.b.nb[1];
@@ -856,50 +631,17 @@ __device__ __forceinline__ void brick_phased(const StagedArgs& a, int bin, float
   const Tc* coef = static_cast<const Tc*>(a.coef);
   float4* halo = smem;
   const Recs R = carve_recs<MODE == 1>(smem + a.S[2] * a.PS);
-  if (end - beg < a.min_stage || a.chunked) {
+  if (end - beg < a.min_stage) {
     // an origin far from every cell sends every stencil to global memory
     const int far[3] = {-(1 << 29), -(1 << 29), -(1 << 29)};
     process_brick<Tc, NC, MODE>(a, beg, end, far, halo, R);
     return;
-  }
-  if constexpr (TMA && IsNode4<Tc>::value) {
-    // `maps` (with the tensor maps) is the kernel argument block or lies in
-    // global memory; the destinations must be 128-byte aligned
-    if (a.tma && maps && is_cube11_rows12(a) && (smem_u32(halo) & 127) == 0) {
-      __shared__ __align__(8) unsigned long long mbar, probe_bar;
-      using G = HaloGeo<12>;
-      // test knob: a barrier that nothing completes, waited on after the copy
-      unsigned long long* probe = a.wait_probe > 0 ? &probe_bar : nullptr;
-      if (probe && threadIdx.x == 0) tma_init_barrier(probe);
-      if constexpr (IsNode16<Tc>::value) {
-        unsigned char* base = reinterpret_cast<unsigned char*>(halo);
-        unsigned char* raw = base + node16_raw_offset(G::Sz, G::PS, G::Sy, G::SX);
-        unsigned char* sraw = base + node16_scale_offset(G::Sz, G::PS, G::Sy);
-        if (threadIdx.x == 0)
-          tma_issue_node16(&maps->tmap, &maps->tmap2, raw, sraw, &mbar, P0,
-                           (unsigned)(G::Sz * G::Sy * (G::SX * 8 + 16)));
-        process_brick<Tc, NC, MODE, 12>(a, beg, end, P0, halo, R, &mbar,
-                                        raw, 0, probe);
-      } else {
-        if (threadIdx.x == 0)
-          tma_issue_halo(&maps->tmap, halo, &mbar, P0,
-                         (unsigned)(sizeof(float4) * G::PS * G::Sz));
-        process_brick<Tc, NC, MODE, 12>(a, beg, end, P0, halo, R, &mbar,
-                                        nullptr, 0, probe);
-      }
-      return;
-    }
   }
   // no barrier here: phase A of the first round does not read the halo, and
   // the barrier that follows it also publishes the staged halo
   if (a.vec && is_cube11(a)) {
     stage_halo_vec<Tc, NC, 11>(a, coef, P0, halo, false, a.scale);
     process_brick<Tc, NC, MODE, 11>(a, beg, end, P0, halo, R);
-    return;
-  }
-  if (a.vec && is_cube11_rows12(a)) {
-    stage_halo_vec<Tc, NC, 12>(a, coef, P0, halo, false, a.scale);
-    process_brick<Tc, NC, MODE, 12>(a, beg, end, P0, halo, R);
     return;
   }
   if (a.vec)
@@ -909,226 +651,11 @@ __device__ __forceinline__ void brick_phased(const StagedArgs& a, int bin, float
   process_brick<Tc, NC, MODE>(a, beg, end, P0, halo, R);
 }
 
-// MODE 0: vel; 1: vel + grad; 2: fused Heun step.  One CTA per brick.  The
-// argument block is a grid constant so that its tensor map can be named by
-// the tensor copy.
+// One component.  MODE 0: vel; 1: vel + grad.  One CTA per brick.
 template <typename Tc, int NC, int MODE>
-__global__ void __launch_bounds__(kThreads, sizeof(Tc) == 2 ? 6 : 7)
-    interp_staged(const __grid_constant__ StagedArgs a) {
+__global__ void __launch_bounds__(kThreads, 7) interp_staged(const __grid_constant__ StagedArgs a) {
   extern __shared__ __align__(128) float4 smem_a128[];
-  brick_phased<Tc, NC, MODE, true>(a, blockIdx.x, smem_a128, &a);
-}
-
-// Global brick b of a many-field batch: the field is the last f with
-// bin_base[f] <= b; its arguments are copied to shared memory (sa), its tensor
-// map stays in the global table.  Empty bins return at once.  Every thread of
-// the block calls.
-template <typename Tc, int NC, int MODE>
-__device__ __forceinline__ void batch_brick(const StagedArgs* __restrict__ tab,
-                                            const int* __restrict__ bin_base, int nfields,
-                                            int b, float4* smem, StagedArgs& sa) {
-  // field 0's offsets are the global offsets: empty bins leave at once
-  const int32_t* goffs = tab[0].offs;
-  if (goffs[b] >= goffs[b + 1]) return;
-  int lo = 0, hi = nfields;  // bin_base[lo] <= b < bin_base[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (bin_base[mid] <= b) lo = mid;
-    else hi = mid;
-  }
-  constexpr int kWords = (int)(sizeof(StagedArgs) / sizeof(int4));
-  static_assert(sizeof(StagedArgs) % sizeof(int4) == 0, "argument block copied in 16 bytes");
-  for (int i = threadIdx.x; i < kWords; i += blockDim.x)
-    reinterpret_cast<int4*>(&sa)[i] = reinterpret_cast<const int4*>(tab + lo)[i];
-  // the field's tensor map stays in the global table (a tensor copy cannot
-  // name one in shared memory); order its upload before the copy proxy
-  if (threadIdx.x == 0 && IsNode4<Tc>::value && tab[lo].tma) {
-    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
-                     reinterpret_cast<unsigned long long>(&tab[lo].tmap))
-                 : "memory");
-    if (IsNode16<Tc>::value)
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
-                       reinterpret_cast<unsigned long long>(&tab[lo].tmap2))
-                   : "memory");
-  }
-  __syncthreads();
-  brick_phased<Tc, NC, MODE, true>(sa, b - bin_base[lo], smem, tab + lo);
-}
-
-// Many fields in one launch: block b handles global brick b.
-template <typename Tc, int NC, int MODE>
-__global__ void __launch_bounds__(kThreads, 5)
-    interp_staged_batch(const StagedArgs* __restrict__ tab, const int* __restrict__ bin_base,
-                        int nfields) {
-  extern __shared__ __align__(128) float4 smem_b128[];
-  __shared__ StagedArgs sa;
-  batch_brick<Tc, NC, MODE>(tab, bin_base, nfields, blockIdx.x, smem_b128, sa);
-}
-
-constexpr int kParamFields = 48;  // 48 x 640 bytes of arguments: within the 32 KB of parameters
-struct BatchParams {
-  StagedArgs a[kParamFields];
-  int bin_base[kParamFields + 1];
-  int nfields;
-};
-static_assert(sizeof(BatchParams) <= 32764, "kernel parameters are limited to 32764 bytes");
-
-// A batch of at most kParamFields fields passes its argument table as one
-// kernel parameter: the brick body then reads each field's arguments from the
-// constant bank, as the single-field kernel does (72 registers, 7 blocks per
-// SM), instead of from a shared-memory copy (96 registers, 5 blocks); the
-// tensor maps are named in parameter space like the single-field kernel's.
-template <typename Tc, int NC, int MODE>
-__global__ void __launch_bounds__(kThreads, sizeof(Tc) == 2 ? 6 : 7)
-    interp_staged_batch_p(const __grid_constant__ BatchParams tab) {
-  extern __shared__ __align__(128) float4 smem_bp128[];
-  const int b = blockIdx.x;
-  // field 0's offsets are the global offsets: empty bins leave at once
-  const int32_t* goffs = tab.a[0].offs;
-  if (goffs[b] >= goffs[b + 1]) return;
-  int lo = 0, hi = tab.nfields;  // bin_base[lo] <= b < bin_base[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (tab.bin_base[mid] <= b) lo = mid;
-    else hi = mid;
-  }
-  brick_phased<Tc, NC, MODE, true>(tab.a[lo], b - tab.bin_base[lo], smem_bp128, &tab.a[lo]);
-}
-
-// ----------------------------------------------------- persistent batch ----
-// All Heun steps of a many-field batch in one cooperative launch: per step
-// the three scan phases, the scatter into bin order, then the bricks of all
-// fields, which count the bins of the positions they write for the next
-// step (the first step counts from the positions, scatters by rank and
-// clears the counters; later ones scatter from the counts, which end at
-// zero); the phases are separated by grid-wide barriers.  Each barrier is an arrival
-// counter and a generation word; a wait gives up after about 2^31 clocks,
-// sets the block-stop word and PS_DEV_TIMEOUT, and every block leaves at its
-// next barrier.  sync[3] is a word nothing sets: with wait_probe > 0 (a test
-// knob) every block waits on it after the first barrier, for that many
-// clocks, so that the give-up path runs.  sync[4] is the brick pass's claim
-// counter: blocks take kClaim consecutive global bins at a time.
-struct BatchRun {
-  const StagedArgs* tab;   // per-field brick-kernel arguments
-  const int* bin_base;     // nfields + 1
-  const BinField* bintab;  // per-field binning table
-  int nfields;
-  int nsteps;
-  int64_t total_bins, np;
-  double* pos;             // the caller's positions (bin order after a step)
-  int64_t* ids;
-  double* pos_s;           // copies in bin order (workspace)
-  int64_t* ids_s;
-  int32_t* bin_of;
-  int32_t* rank;
-  int32_t* counts;         // total_bins + 1, zero at launch
-  int32_t* offsets;        // total_bins + 1
-  int32_t* scan_tmp;
-  int32_t* status;
-  unsigned* sync;          // arrivals, generation, stop, never set, claims; zero at launch
-  int wait_probe;
-};
-
-__device__ __forceinline__ bool grid_barrier(const BatchRun& r, int& nbar) {
-  __shared__ int go;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned* vs = r.sync;
-    bool ok = vs[2] == 0;
-    if (ok) {
-      const unsigned gen = vs[1];
-      __threadfence();
-      if (atomicAdd(&r.sync[0], 1u) + 1u == gridDim.x) {
-        atomicExch(&r.sync[0], 0u);
-        __threadfence();
-        atomicAdd(&r.sync[1], 1u);
-      } else {
-        const long long t0 = clock64();
-        while (vs[1] == gen) {
-          if (vs[2]) {
-            ok = false;
-            break;
-          }
-          if (clock64() - t0 > (1ll << 31)) {
-            if (atomicExch(&r.sync[2], 1u) == 0u) flag_status(r.status, PS_DEV_TIMEOUT, nbar);
-            ok = false;
-            break;
-          }
-          __nanosleep(100);
-        }
-      }
-      __threadfence();
-      if (ok && r.wait_probe > 0 && nbar == 0) {
-        const long long t0 = clock64();
-        while (vs[3] == 0 && clock64() - t0 <= r.wait_probe) __nanosleep(100);
-        if (vs[3] == 0) {
-          if (atomicExch(&r.sync[2], 1u) == 0u) flag_status(r.status, PS_DEV_TIMEOUT, nbar);
-          ok = false;
-        }
-      }
-    }
-    go = ok ? 1 : 0;
-  }
-  __syncthreads();
-  ++nbar;
-  return go != 0;
-}
-
-constexpr int kClaim = 4;  // global bins per claim of the persistent brick pass
-
-template <typename Tc>
-__global__ void __launch_bounds__(kThreads, 5) batch_persistent(const __grid_constant__ BatchRun r) {
-  extern __shared__ __align__(128) float4 smem_bp[];
-  __shared__ StagedArgs sa;
-  __shared__ int32_t scan_sh[kThreads / 32];
-  __shared__ int64_t claim;
-  int nbar = 0;
-  const int lane = threadIdx.x & 31;
-  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t gs = (int64_t)gridDim.x * blockDim.x;
-  const int64_t ntiles = (r.total_bins + kScanTile - 1) / kScanTile;
-  for (int step = 0; step < r.nsteps; ++step) {
-    // the first step counts from the positions; later ones scan the counts
-    // the previous step's bricks took
-    if (step == 0) {
-      batch_count_range(r.bintab, r.nfields, r.np, r.pos, r.bin_of, r.rank, r.counts, r.status,
-                        gt - lane, gs);
-      if (!grid_barrier(r, nbar)) return;
-    }
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-      scan_tile_sum<kThreads>(r.counts, r.total_bins, t, r.scan_tmp, scan_sh);
-    if (!grid_barrier(r, nbar)) return;
-    if (blockIdx.x == 0) scan_tile_offsets_block<kThreads>(r.scan_tmp, ntiles, scan_sh);
-    if (!grid_barrier(r, nbar)) return;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-      scan_tile<kThreads>(r.counts, r.total_bins, r.scan_tmp, r.offsets, -1, t, ntiles,
-                          scan_sh);
-    if (!grid_barrier(r, nbar)) return;
-    if (step == 0) {
-      scatter_range(r.np, r.pos, r.bin_of, r.rank, r.offsets, nullptr, r.pos_s, r.ids,
-                    r.ids ? r.ids_s : nullptr, gt, gs);
-      for (int64_t i = gt; i <= r.total_bins; i += gs) r.counts[i] = 0;
-    } else {  // the counters end at zero, ready for this step's counting
-      scatter_counted_range(r.np, r.pos, r.bin_of, r.counts, r.offsets, nullptr, r.pos_s,
-                            r.ids, r.ids ? r.ids_s : nullptr, r.total_bins, r.status, gt >> 5,
-                            gs >> 5);
-    }
-    if (gt == 0) atomicExch(&r.sync[4], 0u);
-    if (!grid_barrier(r, nbar)) return;
-    // bricks claimed kClaim at a time (their costs vary with their particles)
-    while (true) {
-      if (threadIdx.x == 0) claim = (int64_t)atomicAdd(&r.sync[4], 1u) * kClaim;
-      __syncthreads();
-      const int64_t b0 = claim;
-      __syncthreads();
-      if (b0 >= r.total_bins) break;
-      for (int64_t b = b0; b < b0 + kClaim && b < r.total_bins; ++b) {
-        batch_brick<Tc, 3, 2>(r.tab, r.bin_base, r.nfields, (int)b, smem_bp, sa);
-        __syncthreads();  // sa and the shared memory are refilled by the next brick
-      }
-    }
-    if (!grid_barrier(r, nbar)) return;
-  }
+  brick_phased<Tc, NC, MODE>(a, blockIdx.x, smem_a128);
 }
 
 // ------------------------------------------------- thread per particle ----
@@ -1377,6 +904,8 @@ int plane_stride(int sx, int sy) {
   return ps;
 }
 
+}  // namespace
+
 ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3], int E,
                       bool grad, StagedArgs* a, size_t* smem) {
   ps_status rc = make_brick_args(grid, brick, &a->b);
@@ -1407,8 +936,7 @@ ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[
     // the padded array when the bricks tile the grid
     vec = E == 0;
     for (int d = 0; d < 3; ++d) vec = vec && grid->n[d] % a->b.B[d] == 0;
-    // rows padded so that a plane is 4 (mod 8) nodes long: the layout a
-    // tensor copy of the halo box produces, conflict-free for the gathers
+    // rows padded so that a plane is 4 (mod 8) nodes long
     for (int sx = a->S[0]; vec && sx < a->S[0] + 8; ++sx)
       if ((sx * a->S[1]) % 8 == 4) {
         a->SX = sx;
@@ -1420,13 +948,12 @@ ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[
   a->tma = 0;
   a->min_stage = tuning().brick_min_stage;
   a->wait_probe = tuning().wait_probe;
-  // (tensor copies of 16-bit nodes land inside the float4 halo's buffer)
-  *smem = (size_t)a->S[2] * a->PS * sizeof(float4) + rec_bytes(grad);
-  if (*smem > 227 * 1024) return fail(PS_ERR_UNSUPPORTED, "brick halo exceeds shared memory");
+  const size_t halo = (size_t)a->S[2] * a->PS * sizeof(float4);
+  *smem = halo + rec_bytes(grad);
+  if (halo + (grad ? 10240 : 7360) > 227 * 1024)
+    return fail(PS_ERR_UNSUPPORTED, "brick halo exceeds shared memory");
   return PS_OK;
 }
-
-}  // namespace
 
 // Tensor map of the halo box over the coefficients (nodes: S[1] x S[2] rows of
 // SX nodes; planar FP32: rows of SX floats of the three components); the
@@ -1491,20 +1018,6 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
 
 namespace {
 
-// Use a tensor copy for the halo when the coefficients are nodes, the halo
-// rows fit the copy layout and the array is 16-byte aligned.
-void attach_tma(StagedArgs* a, ps_dtype coef_t) {
-  a->tma = 0;
-  const bool n16 = coef_t == PS_BF16X4 || coef_t == PS_F16X4;
-  if ((coef_t != PS_F32X4 && !n16) || !a->vec || !tuning().node_tma) return;
-  if ((a->SX * a->S[1]) % 8 != 4 || a->SX > 256 || a->S[1] > 256 || a->S[2] > 256) return;
-  if (!a->coef || (reinterpret_cast<uintptr_t>(a->coef) & 15)) return;
-  if (n16 && ((a->SX & 1) || (a->b.B[0] & 1) || (a->g.rx & 1) || !a->scale ||
-              (reinterpret_cast<uintptr_t>(a->scale) & 15)))
-    return;
-  a->tma = encode_node_halo_map(a, coef_t) ? 1 : 0;
-}
-
 template <typename Tc> struct DtypeOf { static constexpr int v = -1; };
 template <> struct DtypeOf<float> { static constexpr int v = PS_F32; };
 template <> struct DtypeOf<float4> { static constexpr int v = PS_F32X4; };
@@ -1516,16 +1029,11 @@ template <> struct DtypeOf<f16x4> { static constexpr int v = PS_F16X4; };
 template <typename Tc, int NC, int MODE>
 ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st,
                         float* rows_ws = nullptr) {
-  // brick_kernel -1 (default): the quad form for three components, the phased
-  // kernel for one
-  int k = tuning().brick_kernel;
-  if (k < 0) k = 5;
+  // three components take the quad form (brick_kernel 2: the thread per
+  // particle), one the phased kernel
+  const int k = tuning().brick_kernel;
   if constexpr (NC == 3 && DtypeOf<Tc>::v >= 0) {
-    if (k == 5) {
-      bool done = false;
-      ps_status rc = launch_quad(a, (ps_dtype)DtypeOf<Tc>::v, MODE, st, &done, rows_ws);
-      if (rc || done) return rc;
-    }
+    if (k != 2) return launch_quad(a, (ps_dtype)DtypeOf<Tc>::v, MODE, st, rows_ws);
   }
   if (k == 2) {
     auto tk = interp_thread<Tc, NC, MODE>;
@@ -1539,172 +1047,27 @@ ps_status launch_staged(const StagedArgs& a, size_t smem, cudaStream_t st,
     tk<<<(unsigned)a.b.nbins, 64, hs, st>>>(a);
     return check_launch("interp_thread");
   }
-  auto kern = interp_staged<Tc, NC, MODE>;
-  if (smem > 48 * 1024) {
-    ps_status rc = check_cuda(
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-        "staged smem attribute");
-    if (rc) return rc;
+  if constexpr (NC == 1 && MODE <= 1) {
+    auto kern = interp_staged<Tc, NC, MODE>;
+    if (smem > 48 * 1024) {
+      ps_status rc = check_cuda(
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+          "staged smem attribute");
+      if (rc) return rc;
+    }
+    if (a.b.nbins > 0x7fffffff) return fail(PS_ERR_UNSUPPORTED, "too many bins");
+    kern<<<(unsigned)a.b.nbins, kThreads, smem, st>>>(a);
+    return check_launch("interp_staged");
+  } else {
+    return fail(PS_ERR_UNSUPPORTED, "no brick kernel for this case");
   }
-  if (a.b.nbins > 0x7fffffff) return fail(PS_ERR_UNSUPPORTED, "too many bins");
-  kern<<<(unsigned)a.b.nbins, kThreads, smem, st>>>(a);
-  return check_launch("interp_staged");
-}
-
-float3 dt_over_h(const GridArgs& g, double dt) {
-  return make_float3((float)(dt * g.inv_h[0]), (float)(dt * g.inv_h[1]),
-                     (float)(dt * g.inv_h[2]));
 }
 
 }  // namespace
 
-// ---------------------------------------------------------------- batch ----
-// Helpers of the many-field form (batch.cu); StagedArgs stays private to this
-// file and travels as opaque bytes.
-
-size_t staged_args_size() { return sizeof(StagedArgs); }
-
-// Arguments of one field's fused Heun step inside a batch: positions are the
-// concatenated [3][np_total] arrays, offs points at the field's first bin.
-ps_status staged_fill_rk2(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3],
-                          const void* coef, const float* scale, int64_t np_total,
-                          const double* pos_in, double* pos_out, const int32_t* offs,
-                          float* vel, const int64_t* ids_in, int64_t* ids_out, double dt,
-                          int32_t* status, int chunked, int32_t* next_counts, int32_t* next_bin,
-                          int next_key_base, int next_runs, void* out, size_t* smem) {
-  if (coef_t == PS_F64) return fail(PS_ERR_UNSUPPORTED, "batched RK2 needs F32/BF16/F16");
-  StagedArgs a{};
-  ps_status rc = fill_staged(grid, coef_t, brick, 0, false, &a, smem);
-  if (rc) return rc;
-  a.coef = coef;
-  a.scale = scale;
-  attach_tma(&a, coef_t);
-  a.np = np_total;
-  a.pos_in = pos_in;
-  a.pos_out = pos_out;
-  a.offs = offs;
-  a.vel = vel;
-  a.ids_in = ids_in;
-  a.ids_out = ids_out;
-  a.dt = dt;
-  const float3 d = dt_over_h(a.g, dt);
-  a.dtih[0] = d.x;
-  a.dtih[1] = d.y;
-  a.dtih[2] = d.z;
-  a.status = status;
-  a.chunked = chunked;
-  a.next_counts = next_counts;
-  a.next_bin = next_bin;
-  a.next_key_base = next_key_base;
-  a.next_runs = next_runs;
-  memcpy(out, &a, sizeof(a));
-  return PS_OK;
-}
-
-// Launch the batched fused Heun step over total_bins bricks of nfields
-// fields.  Set prepare = true once before any stream capture (it only sets the
-// shared-memory limit of the kernel).
-ps_status staged_batch_launch(ps_dtype coef_t, const void* d_tab, const int* d_bin_base,
-                              const void* h_tab, const int* h_bin_base, int nfields,
-                              int64_t total_bins, size_t smem, bool prepare, cudaStream_t st) {
-  return with_coef_type(coef_t, [&](auto tag) -> ps_status {
-    using Tc = decltype(tag);
-    if constexpr (std::is_same<Tc, double>::value) {
-      return fail(PS_ERR_UNSUPPORTED, "batched RK2 needs F32/BF16/F16");
-    } else {
-      auto kern = interp_staged_batch<Tc, 3, 2>;
-      auto kern_p = interp_staged_batch_p<Tc, 3, 2>;
-      if (prepare) {
-        ps_status rc = PS_OK;
-        if (smem > 48 * 1024) {
-          rc = check_cuda(
-              cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-              "batch smem attribute");
-          if (!rc)
-            rc = check_cuda(cudaFuncSetAttribute(
-                                kern_p, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                            "batch smem attribute");
-        }
-        return rc;
-      }
-      if (total_bins <= 0) return PS_OK;
-      if (h_tab && h_bin_base && nfields <= kParamFields) {
-        // the table by value (a graph captures it with the launch)
-        BatchParams tab;
-        memcpy(tab.a, h_tab, (size_t)nfields * sizeof(StagedArgs));
-        memcpy(tab.bin_base, h_bin_base, (size_t)(nfields + 1) * sizeof(int));
-        tab.nfields = nfields;
-        kern_p<<<(unsigned)total_bins, kThreads, smem, st>>>(tab);
-        return check_launch("interp_staged_batch_p");
-      }
-      kern<<<(unsigned)total_bins, kThreads, smem, st>>>(
-          static_cast<const StagedArgs*>(d_tab), d_bin_base, nfields);
-      return check_launch("interp_staged_batch");
-    }
-  });
-}
-
-// All nsteps Heun steps of a batch in one cooperative launch (batch_persistent):
-// a grid of every block the device holds at once.  counts and sync must be
-// zero at launch (the caller clears them on the same stream).
-ps_status staged_batch_persistent(ps_dtype coef_t, const void* d_tab, const int* d_bin_base,
-                                  const BinField* d_bintab, int nfields, int64_t total_bins,
-                                  int64_t np, int nsteps, double* pos, int64_t* ids,
-                                  double* pos_s, int64_t* ids_s, int32_t* bin_of, int32_t* rank,
-                                  int32_t* counts, int32_t* offsets, int32_t* scan_tmp,
-                                  int32_t* status, unsigned* sync, size_t smem,
-                                  cudaStream_t st) {
-  return with_coef_type(coef_t, [&](auto tag) -> ps_status {
-    using Tc = decltype(tag);
-    if constexpr (std::is_same<Tc, double>::value) {
-      return fail(PS_ERR_UNSUPPORTED, "batched RK2 needs F32/BF16/F16");
-    } else {
-      auto kern = batch_persistent<Tc>;
-      if (smem > 48 * 1024) {
-        ps_status rc = check_cuda(
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-            "persistent batch smem attribute");
-        if (rc) return rc;
-      }
-      int per_sm = 0;
-      ps_status rc = check_cuda(
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem),
-          "persistent batch occupancy");
-      if (rc) return rc;
-      if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "persistent batch kernel does not fit an SM");
-      BatchRun r;
-      r.tab = static_cast<const StagedArgs*>(d_tab);
-      r.bin_base = d_bin_base;
-      r.bintab = d_bintab;
-      r.nfields = nfields;
-      r.nsteps = nsteps;
-      r.total_bins = total_bins;
-      r.np = np;
-      r.pos = pos;
-      r.ids = ids;
-      r.pos_s = pos_s;
-      r.ids_s = ids_s;
-      r.bin_of = bin_of;
-      r.rank = rank;
-      r.counts = counts;
-      r.offsets = offsets;
-      r.scan_tmp = scan_tmp;
-      r.status = status;
-      r.sync = sync;
-      r.wait_probe = tuning().wait_probe;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(per_sm * sm_count()));
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeCooperative;
-      attr[0].val.cooperative = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      return check_cuda(cudaLaunchKernelEx(&cfg, kern, r), "persistent batch launch");
-    }
-  });
+float3 dt_over_h(const GridArgs& g, double dt) {
+  return make_float3((float)(dt * g.inv_h[0]), (float)(dt * g.inv_h[1]),
+                     (float)(dt * g.inv_h[2]));
 }
 
 // RK2 kernels used by ps_rk2_step (rk2.cu).
@@ -1740,7 +1103,6 @@ ps_status rk2_launch_staged(const ps_grid* grid, const int32_t brick[3], int E,
   a.scale = s0;
   a.coef2 = c1;
   a.scale2 = s1;
-  attach_tma(&a, coef_t);
   a.np = np;
   a.pos_in = pos_in;
   a.pos_out = pos_out;
@@ -1831,7 +1193,6 @@ extern "C" ps_status ps_interp_ws(const ps_grid* grid, int ncomp, ps_dtype coef_
   if ((rc = fill_staged(grid, coef_t, brick, 0, grad != nullptr, &a, &smem))) return rc;
   a.coef = coef;
   a.scale = scale;
-  attach_tma(&a, coef_t);
   a.np = np;
   a.pos_in = pos;
   a.perm = perm;
@@ -1949,15 +1310,13 @@ extern "C" ps_status ps_interp_backward_binned(
 }
 
 // Brick-staged form of the second derivatives (mode 3) or the Lagrangian
-// acceleration (mode 4) by the quad kernel; *done false where it does not
-// apply (the caller then gathers directly).
+// acceleration (mode 4) by the quad kernel.
 static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* coef,
                               const float* scale, const void* coef2, const float* scale2,
                               double inv_dt, int64_t np, const double* pos,
                               const int64_t* perm, const int32_t* bin_offsets,
                               const int32_t brick[3], float* out, float* vel, float* rows_ws,
-                              int32_t* status, int mode, cudaStream_t st, bool* done) {
-  *done = false;
+                              int32_t* status, int mode, cudaStream_t st) {
   StagedArgs a{};
   size_t smem;
   ps_status rc = fill_staged(grid, coef_t, brick, 0, false, &a, &smem);
@@ -1966,7 +1325,6 @@ static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* 
   a.scale = scale;
   a.coef2 = coef2;
   a.scale2 = scale2;
-  attach_tma(&a, coef_t);
   a.np = np;
   a.pos_in = pos;
   a.perm = perm;
@@ -1975,7 +1333,7 @@ static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* 
   a.vel = vel;
   a.dt = inv_dt;
   a.status = status;
-  return launch_quad(a, coef_t, mode, st, done, rows_ws);
+  return launch_quad(a, coef_t, mode, st, rows_ws);
 }
 
 extern "C" ps_status ps_interp_hessian(const ps_grid* grid, int ncomp, ps_dtype coef_t,
@@ -2006,11 +1364,9 @@ extern "C" ps_status ps_interp_hessian_ws(const ps_grid* grid, int ncomp, ps_dty
   if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
   cudaStream_t st = as_stream(stream);
   if (bin_offsets && ncomp == 3 && coef_t != PS_F64) {
-    bool done = false;
-    rc = staged_extra(grid, coef_t, coef, scale, nullptr, nullptr, 0.0, np, pos, perm,
-                      bin_offsets, brick, hess, nullptr, result_rows(perm, np, 18, ws, ws_bytes),
-                      status, 3, st, &done);
-    if (rc || done) return rc;
+    return staged_extra(grid, coef_t, coef, scale, nullptr, nullptr, 0.0, np, pos, perm,
+                        bin_offsets, brick, hess, nullptr, result_rows(perm, np, 18, ws, ws_bytes),
+                        status, 3, st);
   }
   GridArgs g = make_grid_args(grid, coef_t);
   return with_coef_type(coef_t, [&](auto tag) -> ps_status {
@@ -2060,11 +1416,9 @@ extern "C" ps_status ps_lagrangian_accel_ws(const ps_grid* grid, ps_dtype coef_t
   cudaStream_t st = as_stream(stream);
   const double inv_dt = coef_np1 ? 1.0 / dt_field : 0.0;
   if (bin_offsets && coef_t != PS_F64) {
-    bool done = false;
-    rc = staged_extra(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, inv_dt, np, pos, perm,
+    return staged_extra(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, inv_dt, np, pos, perm,
                       bin_offsets, brick, acc, vel, result_rows(perm, np, vel ? 6 : 3, ws, ws_bytes),
-                      status, 4, st, &done);
-    if (rc || done) return rc;
+                      status, 4, st);
   }
   GridArgs g = make_grid_args(grid, coef_t);
   return with_coef_type(coef_t, [&](auto tag) -> ps_status {

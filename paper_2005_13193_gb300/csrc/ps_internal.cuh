@@ -125,7 +125,7 @@ ps_status bin_run_batch(const BinField* d_tab, int nfields, int64_t total_bins, 
                         int32_t* counts, int32_t* rank, int32_t* scan_tmp, int32_t* status,
                         cudaStream_t st);
 
-// Many-field brick kernel (interp.cu).
+// Many-field step kernels (batch_step.cu); cube: the bricks are 8^3 cells.
 size_t staged_args_size();
 ps_status staged_fill_rk2(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3],
                           const void* coef, const float* scale, int64_t np_total,
@@ -137,12 +137,12 @@ ps_status staged_fill_rk2(const ps_grid* grid, ps_dtype coef_t, const int32_t br
 constexpr int kBatchChunk = 128;
 // h_tab, h_bin_base: host copies of the same tables; with at most 48 fields
 // they go by value as a kernel parameter (else pass NULL).
-ps_status staged_batch_launch(ps_dtype coef_t, const void* d_tab, const int* d_bin_base,
+ps_status staged_batch_launch(ps_dtype coef_t, bool cube, const void* d_tab, const int* d_bin_base,
                               const void* h_tab, const int* h_bin_base, int nfields,
                               int64_t total_bins, size_t smem, bool prepare, cudaStream_t st);
 // All nsteps Heun steps of a batch in one cooperative launch (counts and sync,
 // four words, zero at launch).
-ps_status staged_batch_persistent(ps_dtype coef_t, const void* d_tab, const int* d_bin_base,
+ps_status staged_batch_persistent(ps_dtype coef_t, bool cube, const void* d_tab, const int* d_bin_base,
                                   const BinField* d_bintab, int nfields, int64_t total_bins,
                                   int64_t np, int nsteps, double* pos, int64_t* ids,
                                   double* pos_s, int64_t* ids_s, int32_t* bin_of, int32_t* rank,

@@ -86,52 +86,62 @@ bool halo_map(StagedArgs* a) {
   }
 }
 
-template <typename Tc, int MODE>
-ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done, float* rows_ws) {
-  StagedArgs a = a0;
-  constexpr bool n16 = IsNode16<Tc>::value;
-  if (a.E != 0 || a.S[1] > 1023 || a.S[2] > 1023) return PS_OK;  // not handled here
-  a.SX = n16                     ? quad_row4(a.S[0], a.S[1], 2)
-         : IsPlanar<Tc>::value ? quad_row4(a.S[0], a.S[1], 4)
-                               : quad_row(a.S[0], a.S[1]);
-  a.PS = a.SX * a.S[1];
-  a.half_dt = 0.5 * a.dt;
-  for (int d = 0; d < 3; ++d) a.ih32[d] = a.g.inv_h[d] * 4294967296.0;
-  a.wait_probe = tuning().wait_probe;
-  a.tma = halo_map<Tc>(&a) ? 1 : 0;
-  size_t smem = (size_t)halo_bytes<Tc>(a.S[2], a.S[1], a.PS);
-  if (smem > 226 * 1024) return PS_OK;
+// Geometry, shared memory and tensor maps of the quad form; *ct: the
+// compile-time geometry that applies (0: none).
+template <typename Tc>
+void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
+  constexpr bool n16 = IsNode16<Tc>::value, planar = IsPlanar<Tc>::value;
+  a->SX = n16      ? quad_row4(a->S[0], a->S[1], 2)
+          : planar ? quad_row4(a->S[0], a->S[1], 4)
+                   : quad_row(a->S[0], a->S[1]);
+  a->PS = a->SX * a->S[1];
+  a->half_dt = 0.5 * a->dt;
+  for (int d = 0; d < 3; ++d) a->ih32[d] = a->g.inv_h[d] * 4294967296.0;
+  a->wait_probe = tuning().wait_probe;
+  *ct = a->S[0] == 11 && a->S[1] == 11 && a->S[2] == 11 && a->SX == (n16 || planar ? 12 : 14)
+            ? a->SX
+            : 0;
+  a->two = 0;
+  a->tma = halo_map<Tc>(a) ? 1 : 0;
+  *smem = (size_t)halo_bytes<Tc>(a->S[2], a->S[1], a->PS);
+  if (*smem > 226 * 1024) {  // no halo: every stencil from global memory
+    *smem = 0;
+    a->tma = 0;
+    a->min_stage = 0x7fffffff;
+    return;
+  }
   // a second field's halo beside the first where both fit
-  a.two = 0;
-  if ((MODE == 2 || MODE == 4) && a.coef2 && 2 * smem <= 226 * 1024) {
-    a.two = 1;
-    smem *= 2;
+  if (second && a->coef2 && 2 * *smem <= 226 * 1024) {
+    a->two = 1;
+    *smem *= 2;
     if constexpr (!n16) {
       // the later field's map in tmap2 (tma = 2)
-      StagedArgs t = a;
-      t.coef = a.coef2;
-      if (a.tma == 1 && halo_map<Tc>(&t)) {
-        a.tmap2 = t.tmap;
-        a.tma = 2;
+      StagedArgs t = *a;
+      t.coef = a->coef2;
+      if (a->tma == 1 && halo_map<Tc>(&t)) {
+        a->tmap2 = t.tmap;
+        a->tma = 2;
       }
     }
   }
+}
+
+template <typename Tc, int MODE>
+ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, float* rows_ws) {
+  StagedArgs a = a0;
+  size_t smem;
+  int ct;
+  setup_t<Tc>(&a, MODE == 2 || MODE == 4, &smem, &ct);
   if (a.b.nbins > 0x7fffffff || a.b.nb[1] > 65535 || a.b.nb[2] > 65535)
     return fail(PS_ERR_UNSUPPORTED, "too many bins");
-  const bool cube = a.S[0] == 11 && a.S[1] == 11 && a.S[2] == 11;
-  auto kern = quad_kernel<Tc, MODE, 0>;
-  if constexpr (n16 || IsPlanar<Tc>::value) {
-    if (cube && a.SX == 12) kern = quad_kernel<Tc, MODE, 12>;
-  } else {
-    if (cube && a.SX == 14) kern = quad_kernel<Tc, MODE, 14>;
-  }
+  constexpr int kCt = IsNode16<Tc>::value || IsPlanar<Tc>::value ? 12 : 14;
+  auto kern = ct == kCt ? quad_kernel<Tc, MODE, kCt> : quad_kernel<Tc, MODE, 0>;
   if (smem > 48 * 1024) {
     ps_status rc = check_cuda(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
         "quad smem attribute");
     if (rc) return rc;
   }
-  *done = true;
   const int threads = a.two ? 128 : 64;
   // results by way of bin order: vel, then the gradient's or the second
   // derivatives' rows
@@ -152,30 +162,27 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, bool* done, float
 }  // namespace
 
 // The quad form for three components: node coefficients or planar
-// F32/BF16/F16.  *done stays false where it does not apply (E != 0, a halo
-// above the shared memory), and the caller takes another form.
+// F32/BF16/F16.
 ps_status launch_quad(const StagedArgs& a, ps_dtype coef_t, int mode, cudaStream_t st,
-                      bool* done, float* rows_ws) {
-  *done = false;
+                      float* rows_ws) {
   auto go = [&](auto tag) -> ps_status {
     using Tc = decltype(tag);
     switch (mode) {
-      case 0: return launch_quad_t<Tc, 0>(a, st, done, rows_ws);
-      case 1: return launch_quad_t<Tc, 1>(a, st, done, rows_ws);
-      case 2: return launch_quad_t<Tc, 2>(a, st, done, rows_ws);
-      case 3: return launch_quad_t<Tc, 3>(a, st, done, rows_ws);
-      default: return launch_quad_t<Tc, 4>(a, st, done, rows_ws);
+      case 0: return launch_quad_t<Tc, 0>(a, st, rows_ws);
+      case 1: return launch_quad_t<Tc, 1>(a, st, rows_ws);
+      case 2: return launch_quad_t<Tc, 2>(a, st, rows_ws);
+      case 3: return launch_quad_t<Tc, 3>(a, st, rows_ws);
+      default: return launch_quad_t<Tc, 4>(a, st, rows_ws);
     }
   };
-  switch (coef_t) {
-    case PS_F32X4: return go(float4{});
-    case PS_F32: return go(float{});
-    case PS_BF16: return go(__nv_bfloat16{});
-    case PS_F16: return go(__half{});
-    case PS_BF16X4: return go(bf16x4{});
-    case PS_F16X4: return go(f16x4{});
-    default: return PS_OK;
-  }
+  return with_quad_type(coef_t, go);
+}
+
+ps_status quad_setup(StagedArgs* a, ps_dtype coef_t, size_t* smem, int* ct) {
+  return with_quad_type(coef_t, [&](auto tag) -> ps_status {
+    setup_t<decltype(tag)>(a, false, smem, ct);
+    return PS_OK;
+  });
 }
 
 }  // namespace ps

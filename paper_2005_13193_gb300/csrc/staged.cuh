@@ -63,14 +63,35 @@ struct StagedArgs {
 // planes) over a node coefficient array (interp.cu).
 bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t);
 
+// Geometry of the brick-staged kernels (interp.cu): extents, plain-load layout,
+// thresholds; *smem for the phased kernel.
+ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3], int E,
+                      bool grad, StagedArgs* a, size_t* smem);
+float3 dt_over_h(const GridArgs& g, double dt);
+
 // The quad-per-particle brick kernel (quad.cu) for three components; mode 0
 // velocities, 1 with the gradient tensor, 2 fused Heun step, 3 second
 // derivatives (into a.grad), 4 Lagrangian acceleration (into a.grad; a.dt
-// holds 1 / dt_field).  With a permutation and a workspace for the result rows (modes 0, 1, 3, 4) the
-// kernel stores in bin order and the rows are put in place afterwards.
-// Leaves *done false where it does not apply.
+// holds 1 / dt_field).  With a permutation and a workspace for the result rows
+// (modes 0, 1, 3, 4) the kernel stores in bin order and the rows are put in
+// place afterwards.
 ps_status launch_quad(const StagedArgs& a, ps_dtype coef_t, int mode, cudaStream_t st,
-                      bool* done, float* rows_ws = nullptr);
+                      float* rows_ws = nullptr);
+// The same form's layout, maps and shared memory for a kernel that calls the
+// brick body itself (batch_step.cu); *ct its compile-time geometry or 0.
+ps_status quad_setup(StagedArgs* a, ps_dtype coef_t, size_t* smem, int* ct);
+template <typename F>
+ps_status with_quad_type(ps_dtype t, F&& f) {
+  switch (t) {
+    case PS_F32X4: return f(float4{});
+    case PS_F32: return f(float{});
+    case PS_BF16: return f(__nv_bfloat16{});
+    case PS_F16: return f(__half{});
+    case PS_BF16X4: return f(bf16x4{});
+    case PS_F16X4: return f(f16x4{});
+    default: return fail(PS_ERR_UNSUPPORTED, "brick kernels need F32, BF16 or F16 coefficients");
+  }
+}
 // Rows in bin order -> rows in the particles' order (unsort.cu): n0 rows to
 // d0, the next n1 to d1.
 ps_status unsort_launch(int64_t np, const int64_t* perm, const float* src, float* d0, int n0,
@@ -153,19 +174,9 @@ template <> struct HaloGeo<11> {
   static constexpr int Sx = 11, Sy = 11, Sz = 11, SX = 11, PS = 124;
   __device__ __forceinline__ explicit HaloGeo(const StagedArgs&) {}
 };
-// The same halo with 12-point rows: the layout of a tensor copy of a node
-// halo, whose plane of 12 x 11 points is 132 = 4 (mod 8) float4 long.
-template <> struct HaloGeo<12> {
-  static constexpr int Sx = 11, Sy = 11, Sz = 11, SX = 12, PS = 132;
-  __device__ __forceinline__ explicit HaloGeo(const StagedArgs&) {}
-};
 __device__ __forceinline__ bool is_cube11(const StagedArgs& a) {
   return a.S[0] == 11 && a.S[1] == 11 && a.S[2] == 11 && a.SX == 11 && a.PS == 124;
 }
-__device__ __forceinline__ bool is_cube11_rows12(const StagedArgs& a) {
-  return a.S[0] == 11 && a.S[1] == 11 && a.S[2] == 11 && a.SX == 12 && a.PS == 132;
-}
-
 // ------------------------------------------------- tensor-copy staging ----
 // One thread arms an mbarrier with the byte count of the box and issues the
 // tensor copy of the brick's node halo; the copy completes the barrier's
@@ -192,50 +203,7 @@ __device__ __forceinline__ void tma_copy_halo(const CUtensorMap* map, float4* ds
       "r"(smem_u32(mbar))
       : "memory");
 }
-__device__ __forceinline__ void tma_issue_halo(const CUtensorMap* map, float4* dst,
-                                               unsigned long long* mbar, const int P0[3],
-                                               unsigned bytes) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)) : "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
-               "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<unsigned long long>(map)), "r"(4 * P0[0]), "r"(P0[1]), "r"(P0[2]),
-      "r"(smem_u32(mbar))
-      : "memory");
-}
-// 16-bit node halos: the tensor copies put the raw nodes and their rows'
-// scales into the float4 halo's own buffer, near its end (both 128-byte
-// aligned), and the block widens them in place in kNode16Slices slices of
-// nodes: each slice is read into registers, a barrier, then written as
-// float4.  The float4 writes of a slice reach raw bytes of its own or of
-// earlier slices only, and the scales only in the last slice (checked below
-// for the compile-time 8^3 halo).  Offsets in bytes from the halo's start.
-constexpr int kNode16Slices = 4;
-__host__ __device__ constexpr int align_down128(int v) { return v & ~127; }
-__host__ __device__ constexpr int node16_scale_offset(int Sz, int PS, int Sy) {
-  return align_down128(Sz * PS * 16 - Sz * Sy * 16);
-}
-__host__ __device__ constexpr int node16_raw_offset(int Sz, int PS, int Sy, int SX) {
-  return align_down128(node16_scale_offset(Sz, PS, Sy) - Sz * Sy * SX * 8);
-}
-// slice s (s < kNode16Slices - 1) writes float4 nodes below (s + 1) * per;
-// the raw nodes of slice s + 1 start at raw + 8 (s + 1) per
-__host__ __device__ constexpr bool node16_in_place_ok(int Sz, int PS, int Sy, int SX) {
-  const int npts = Sz * Sy * SX, per = (npts + kNode16Slices - 1) / kNode16Slices;
-  bool ok = Sz * PS >= npts && node16_raw_offset(Sz, PS, Sy, SX) >= 0;
-  for (int s = 0; s + 1 < kNode16Slices; ++s) {
-    const int end_write = 16 * (s + 1) * per;
-    ok = ok && end_write <= node16_raw_offset(Sz, PS, Sy, SX) + 8 * (s + 1) * per &&
-         end_write <= node16_scale_offset(Sz, PS, Sy);
-  }
-  return ok;
-}
-static_assert(node16_in_place_ok(11, 132, 11, 12), "16-bit node halo cannot widen in place");
-
+// 16-bit nodes and their rows' scales, both on one initialised barrier.
 __device__ __forceinline__ void tma_copy_node16(const CUtensorMap* nodes,
                                                 const CUtensorMap* scales, void* raw,
                                                 void* sraw, unsigned long long* mbar,
@@ -256,14 +224,6 @@ __device__ __forceinline__ void tma_copy_node16(const CUtensorMap* nodes,
       "l"(reinterpret_cast<unsigned long long>(scales)), "r"(4 * P0[1]), "r"(P0[2]),
       "r"(smem_u32(mbar))
       : "memory");
-}
-
-__device__ __forceinline__ void tma_issue_node16(const CUtensorMap* nodes,
-                                                 const CUtensorMap* scales, void* raw,
-                                                 void* sraw, unsigned long long* mbar,
-                                                 const int P0[3], unsigned bytes) {
-  tma_init_barrier(mbar);
-  tma_copy_node16(nodes, scales, raw, sraw, mbar, P0, bytes);
 }
 
 // A planar halo (rows of floats, three components; P0[0] is a
