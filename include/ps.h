@@ -117,14 +117,14 @@ const char* ps_version(void);
 int64_t ps_coef_row_pitch(int nx, ps_dtype coef_t);
 
 /* Launch-shape knobs (not part of the method):
- *  "brick_kernel" (for the brick-staged calls, bins given): -1 = automatic
- *     (default; 5 for three components, 0 for one), 0 = one CTA per brick, 8
- *     lanes per particle, phases separated by block barriers, 2 = one CTA per
- *     brick, one thread per particle, 5 = one CTA per brick, each warp on its
- *     own with 32 particles at a time, four lanes per particle holding one
- *     z-row of the stencil each in registers (the Heun predictor reuses it
- *     when it stays in its cell); 16-bit node halos stay 16-bit in shared
- *     memory.  Forms a case does not support fall back to 0.
+ *  "brick_kernel" (for the brick-staged calls, bins given): three components
+ *     take one block per brick, each warp on its own with 32 particles at a
+ *     time, four lanes per particle holding one z-row of the stencil each in
+ *     registers (the Heun predictor reuses it when it stays in its cell; 16-bit
+ *     node halos stay 16-bit in shared memory), with -1 (default), 0 and 5
+ *     alike; 2 = one thread per particle.  One component takes one CTA per
+ *     brick, 8 lanes per particle, phases separated by block barriers (2: one
+ *     thread per particle).
  *  "brick_min_stage" in [0, 2^20] (default 8): bricks holding fewer particles
  *     skip the halo staging and gather their stencils from global memory.
  *  "node_tma" 0 or 1 (default 1): halos of node coefficients by tensor copy.
@@ -171,8 +171,8 @@ ps_status ps_status_read(const int32_t* status, int32_t* host_out, void* stream)
 /*   ignored.  field and coef must not overlap.  ncomp in [1, 16].          */
 /*   ws: ps_spline_coeffs_workspace_size bytes, 256-byte aligned; required  */
 /*   for the 16-bit and node forms.  For PS_F32 it is nonzero when nx is    */
-/*   128, 256 or 512 and ny, nz >= 32: given it (and a 16-byte aligned F32  */
-/*   field) the solve takes two streamed passes (x and y of every plane,    */
+/*   64 to 768 (or a multiple of 4) and ny, nz >= 32: given it (and an F32   */
+/*   field) the solve may take two streamed passes (x and y of every plane, */
 /*   then z), which truncate each periodic recursion's look-ahead at 16     */
 /*   lines (terms below 7.2e-10 of the values skipped, under FP32           */
 /*   rounding); without it the three passes run in place.  PS_F32X4 takes   */
@@ -184,6 +184,13 @@ ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype field_t,
                            const void* field, ps_dtype coef_t, void* coef,
                            float* scale, void* ws, size_t ws_bytes,
                            void* stream);
+/* ps_spline_coeffs, keeping the three passes on rows other than 128, 256 or */
+/* 512 values: for callers whose FP64 results follow the coefficients'       */
+/* rounding (the position gradients of the differentiable interpolation).    */
+ps_status ps_spline_coeffs_rows3(const ps_grid* grid, int ncomp,
+                                 ps_dtype field_t, const void* field,
+                                 ps_dtype coef_t, void* coef, float* scale,
+                                 void* ws, size_t ws_bytes, void* stream);
 
 /* ------------------------------------------------------------------------ */
 /* Operation 1 through the inverse (Sec. 2.2's periodic system, solved as a */
@@ -469,8 +476,8 @@ ps_status ps_rk2_sort(const ps_grid* grid, const int32_t brick[3], int64_t np,
 /* (ps_batch_workspace_size).  tune_cache: optional text file whose line    */
 /* "brick <bx> <by> <bz>" overrides `brick` (written by the autotuner).     */
 /* Coefficients: PS_F32, PS_BF16, PS_F16 or their node forms (PS_F32X4,    */
-/* PS_BF16X4, PS_F16X4, whose halos are tensor copies); the batch uses the  */
-/* one-CTA-per-brick kernel.                                                */
+/* PS_BF16X4, PS_F16X4), halos by tensor copies; the bricks run the         */
+/* single-field kernel's body.                                              */
 /* ------------------------------------------------------------------------ */
 typedef struct ps_plan ps_plan;
 typedef struct {

@@ -208,8 +208,10 @@ def ps_spline_coeffs_workspace_size(n, ncomp: int, coef_dtype: torch.dtype,
 
 
 def ps_spline_coeffs(field: torch.Tensor, coef: torch.Tensor, scale: Optional[torch.Tensor] = None,
-                     ws: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None):
-    """Operation 1 (Sec. 2.2): field [ncomp][nz][ny][nx] -> coef [ncomp][nz+3][ny+3][nx+3]."""
+                     ws: Optional[torch.Tensor] = None, L=DEFAULT_L, stream=None,
+                     rows3: bool = False):
+    """Operation 1 (Sec. 2.2): field [ncomp][nz][ny][nx] -> coef [ncomp][nz+3][ny+3][nx+3].
+    rows3: three passes on rows other than 128, 256 or 512 values (ps_spline_coeffs_rows3)."""
     n = grid_of_field(field)
     ncomp = field.shape[0]
     _dev(field, "field")
@@ -219,9 +221,9 @@ def ps_spline_coeffs(field: torch.Tensor, coef: torch.Tensor, scale: Optional[to
     _dev(ws, "ws")
     g = make_grid(n, L)
     ws_bytes = ws.numel() * ws.element_size() if ws is not None else 0
-    _check(_lib().ps_spline_coeffs(ctypes.byref(g), ncomp, _DT[field.dtype], _ptr(field),
-                                   _coef_type(coef), _ptr(coef), _ptr(scale), _ptr(ws), ws_bytes,
-                                   _stream(stream)))
+    call = _lib().ps_spline_coeffs_rows3 if rows3 else _lib().ps_spline_coeffs
+    _check(call(ctypes.byref(g), ncomp, _DT[field.dtype], _ptr(field), _coef_type(coef),
+                _ptr(coef), _ptr(scale), _ptr(ws), ws_bytes, _stream(stream)))
 
 
 def ps_bin_workspace_size(n, brick, np_: int, L=DEFAULT_L) -> int:
@@ -509,7 +511,7 @@ class SplineField:
     @classmethod
     def from_field(cls, field: torch.Tensor, coef_dtype=torch.float32, L=DEFAULT_L,
                    out: Optional["SplineField"] = None, ws: Optional[torch.Tensor] = None,
-                   stream=None) -> "SplineField":
+                   stream=None, rows3: bool = False) -> "SplineField":
         n = grid_of_field(field)
         ncomp = field.shape[0]
         if out is None:
@@ -522,7 +524,8 @@ class SplineField:
         need = ps_spline_coeffs_workspace_size(n, ncomp, coef_kind(out.coef), L)
         if need and (ws is None or ws.numel() < need):
             ws = workspace(need, field.device)
-        ps_spline_coeffs(field, out.coef, out.scale, ws if need else None, L=L, stream=stream)
+        ps_spline_coeffs(field, out.coef, out.scale, ws if need else None, L=L, stream=stream,
+                         rows3=rows3)
         return out
 
     def hessian(self, pos: torch.Tensor, status: Optional[torch.Tensor] = None,
@@ -666,7 +669,7 @@ class InterpFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L):
-        sf = SplineField.from_field(field.detach().float(), torch.float32, L)
+        sf = SplineField.from_field(field.detach().float(), torch.float32, L, rows3=True)
         x = pos.detach()
         bins = None
         nbins = math.prod(-(-sf.n[d] // _FN_BRICK[d]) for d in range(3))

@@ -18,12 +18,13 @@
 // 1e-12 (FP32) or 1e-24 (FP64) after a chunk or two, where the sum stops, so
 // every pencil is read once and written once.
 //
-// FP32 coefficients of FP32 fields on rows of 128, 256 or 512 values take two
+// FP32 coefficients of FP32 fields on rows of 64 to 768 values take two
 // streamed passes (x and y of every plane, then z; see below).  Otherwise
 // three passes: y, then z (strided: threads along x read coalesced rows),
 // then x (one warp per row, staged through shared memory), which writes the
 // padded N+3 layout with periodic ghosts and, for BF16/FP16, a power-of-two
 // scale per x-line.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -227,16 +228,17 @@ __device__ __forceinline__ int skew_l(int e, int L, float inv_L) {
 // The recursions of one periodic line held by a warp, lane l holding its
 // chunk v[0..len) (the line's values [l L, l L + len)): causal and
 // anti-causal, each with its chunk carries by shuffles; before the gain.
+// (nl: the lanes that hold values, the first ones of the warp)
 template <typename T, int LMAX>
-__device__ __forceinline__ void line_recur(T (&v)[LMAX], int len, int lane, T z) {
+__device__ __forceinline__ void line_recur(T (&v)[LMAX], int len, int lane, T z, int nl = 32) {
   const unsigned FULL = 0xffffffffu;
   const T thr = Thr<T>::v;
   const T y = chunk_causal<T, LMAX>(v, len, z);
   const T a = chunk_zlen<T>(len);
   T carry = T(0), fac = T(1);
   bool wrapped = true;
-  for (int j = 1; j <= 32; ++j) {
-    const int sl = (lane - j) & 31;
+  for (int j = 1; j <= nl; ++j) {
+    const int sl = nl == 32 ? (lane - j) & 31 : (lane >= j ? lane - j : lane - j + nl);
     const T ej = __shfl_sync(FULL, y, sl);
     const T aj = __shfl_sync(FULL, a, sl);
     carry += fac * ej;
@@ -253,8 +255,8 @@ __device__ __forceinline__ void line_recur(T (&v)[LMAX], int len, int lane, T z)
   carry = T(0);
   fac = T(1);
   wrapped = true;
-  for (int j = 1; j <= 32; ++j) {
-    const int sl = (lane + j) & 31;
+  for (int j = 1; j <= nl; ++j) {
+    const int sl = nl == 32 ? (lane + j) & 31 : (lane + j < nl ? lane + j : lane + j - nl);
     const T fj = __shfl_sync(FULL, w, sl);
     const T aj = __shfl_sync(FULL, a, sl);
     carry += fac * fj;
@@ -672,6 +674,17 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
+// PE = 4, 2 or 1 floats (rows of a multiple of 4, of 2, of any length).
+template <int PE>
+__device__ __forceinline__ void cp_async_piece(float* dst, const float* src) {
+  if constexpr (PE == 4) {
+    cp_async16(dst, src);
+  } else {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"(4 * PE)
+                 : "memory");
+  }
+}
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
@@ -774,62 +787,105 @@ __device__ __forceinline__ void sb_stream(int n, float z, Copy copy, Read read, 
   cp_async_wait<0>();
 }
 
-// Pass 1: one block per (c, z) plane of an unpadded array, nx = 32 LMAX
-// (LMAX = 4, 8 or 16), one thread per x column, streaming y.  A stage holds
-// kSB rows with x at x + 4 floor(x / 32): the 16-byte copies stay aligned, a
-// lane's chunk of LMAX values is read and written as 16-byte accesses on
-// distinct banks, and a warp's column reads fall on distinct banks.  Each
-// chunk's rows are solved along x in place (a warp per row), then every
-// thread takes its column through the y recursions and stores its outputs,
-// coalesced across the warp.
-template <int LMAX, int S>
-__global__ void __launch_bounds__(32 * LMAX, 1024 / (32 * LMAX)) solve_xy_stream(
-    const float* src, View sv, float* dst, View dv, int ny, int nz, float z, float gain) {
+// Pass 1: one block per (c, z) plane of an unpadded array, one thread per x
+// column (up to 768), streaming y.  A lane takes chunks of LMAX values (a
+// multiple of 4) of a row; ROWS 0: nx = 32 LMAX, 1: the first nx / LMAX lanes
+// hold whole chunks, 2: the first ceil(nx / LMAX) lanes hold the row.  A stage holds kSB rows with x at x + 4 floor(x / 32):
+// the copies stay aligned, a lane's chunk is read and written as 16-byte
+// accesses on distinct banks, and a warp's column reads fall on distinct
+// banks.  Each chunk's rows are solved along x in place (a warp per row), then
+// every thread takes its column through the y recursions and stores its
+// outputs, coalesced across the warp.  It may write in place (rows are stored
+// after the chunk behind them has been read).
+__host__ __device__ constexpr int xy_pitch(int padded) { return padded + 4 * ((padded + 31) / 32); }
+template <int LMAX, int S, int PE, int ROWS>
+__global__ void __launch_bounds__(32 * LMAX, (ROWS == 0 || LMAX == 24 ? 1024 : 768) / (32 * LMAX))
+    solve_xy_stream(
+    const float* src, View sv, float* dst, View dv, int nx_, int ny, int nz, float z, float gain) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int NX = 32 * LMAX, T = NX, RP = NX + NX / 8;  // padded row
-  constexpr int PR = NX / 4;                                // 16-byte pieces per row
-  float* stage = reinterpret_cast<float*>(smem_raw);       // [S][kSB][RP]
+  constexpr bool FULL = ROWS == 0;
+  const int nx = FULL ? 32 * LMAX : nx_;
+  const int nl = FULL ? 32 : (nx + LMAX - 1) / LMAX;        // lanes that hold a row
+  const int T = FULL ? 32 * LMAX : (int)blockDim.x;
+  const int RP = FULL ? xy_pitch(32 * LMAX) : xy_pitch(nl * LMAX);  // padded row
+  const int PR = nx / PE;                                   // pieces per row
+  float* stage = reinterpret_cast<float*>(smem_raw);        // [S][kSB][RP]
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int c = blockIdx.x / nz, zz = blockIdx.x - c * nz;
   const float* sp = src + sv.off + c * sv.sc + zz * sv.sz;
   float* dp = dst + dv.off + c * dv.sc + zz * dv.sz + t;
   const int xcol = t + 4 * (t >> 5);                        // this thread's column
-  const int xchunk = lane * LMAX + 4 * ((lane * LMAX) >> 5);  // this lane's chunk
+  const int j0 = t / PR, m0 = t - j0 * PR, dj = T / PR, dm = T - dj * PR;
+  // this lane's part of a row (lanes beyond whole chunks run on zeros)
+  int llen = ROWS < 2 ? LMAX : nx - lane * LMAX;
+  if (ROWS == 2) llen = llen < 0 ? 0 : (llen > LMAX ? LMAX : llen);
+
+  // place of value e (a multiple of 4) of this lane's chunk; a chunk that
+  // divides 32 lies in one piece
+  const int e0 = lane * LMAX, xchunk = e0 + 4 * (e0 >> 5);
+  auto at = [&](int e) {
+    if constexpr (32 % LMAX == 0) return xchunk + e;
+    return e0 + e + 4 * ((e0 + e) >> 5);
+  };
 
   auto copy = [&](int q) {
     const int len = sb_len(q, ny);
     const float* g = sp + sb_start(q, ny) * sv.sy;
     float* st = stage + (q % S) * kSB * RP;
-    const int m = t % PR;
+    if constexpr (FULL) {
+      const int m = t % (8 * LMAX);
 #pragma unroll
-    for (int j = t / PR; j < kSB; j += T / PR)
-      if (j < len) cp_async16(st + j * RP + 4 * m + 4 * (m >> 3), g + j * sv.sy + 4 * m);
+      for (int j = t / (8 * LMAX); j < kSB; j += 4)
+        if (j < len) cp_async16(st + j * RP + 4 * m + 4 * (m >> 3), g + j * sv.sy + 4 * m);
+    } else {
+      for (int j = j0, m = m0; j < len;) {
+        const int e = PE * m;
+        cp_async_piece<PE>(st + j * RP + e + 4 * (e >> 5), g + j * sv.sy + e);
+        j += dj;
+        m += dm;
+        if (m >= PR) {
+          m -= PR;
+          ++j;
+        }
+      }
+    }
   };
   auto read = [&](int q, float (&g)[kSB]) {
     const int len = sb_len(q, ny);
     float* st = stage + (q % S) * kSB * RP;
     // the chunk's rows along x, in place
     for (int j = warp; j < len; j += T / 32) {
-      float* row = st + j * RP + xchunk;
+      float* row = st + j * RP;
       float v[LMAX];
+      if (ROWS == 1) {
 #pragma unroll
-      for (int e = 0; e < LMAX; e += 4) {  // a chunk never straddles 32 values
-        const float4 f = *reinterpret_cast<const float4*>(row + e);
-        v[e] = f.x;
-        v[e + 1] = f.y;
-        v[e + 2] = f.z;
-        v[e + 3] = f.w;
+        for (int e = 0; e < LMAX; ++e) v[e] = 0.f;
       }
-      line_recur<float, LMAX>(v, LMAX, lane, z);
+      if (FULL || lane < nl) {
 #pragma unroll
-      for (int e = 0; e < LMAX; e += 4)
-        *reinterpret_cast<float4*>(row + e) =
-            make_float4(__fmul_rn(gain, v[e]), __fmul_rn(gain, v[e + 1]),
-                        __fmul_rn(gain, v[e + 2]), __fmul_rn(gain, v[e + 3]));
+        for (int e = 0; e < LMAX; e += 4) {  // four values never straddle 32
+          const float4 f = *reinterpret_cast<const float4*>(row + at(e));
+          v[e] = f.x;
+          v[e + 1] = f.y;
+          v[e + 2] = f.z;
+          v[e + 3] = f.w;
+        }
+      }
+      line_recur<float, LMAX>(v, llen, lane, z, nl);
+      if (FULL || lane < nl) {
+#pragma unroll
+        for (int e = 0; e < LMAX; e += 4)
+          *reinterpret_cast<float4*>(row + at(e)) =
+              make_float4(__fmul_rn(gain, v[e]), __fmul_rn(gain, v[e + 1]),
+                          __fmul_rn(gain, v[e + 2]), __fmul_rn(gain, v[e + 3]));
+      }
     }
     __syncthreads();
     const float* col = st + xcol;
-    if (len == kSB) {
+    if (!FULL && t >= nx) {
+#pragma unroll
+      for (int j = 0; j < kSB; ++j) g[j] = 0.f;
+    } else if (len == kSB) {
 #pragma unroll
       for (int j = 0; j < kSB; ++j) g[j] = col[j * RP];
     } else {
@@ -839,6 +895,7 @@ __global__ void __launch_bounds__(32 * LMAX, 1024 / (32 * LMAX)) solve_xy_stream
   };
   auto emit = [&](int qo, float (&y)[kSB], int len, float w) {
     float* o = dp + sb_start(qo, ny) * dv.sy;
+    if (!FULL && t >= nx) return;
     if (len == kSB) {
 #pragma unroll
       for (int i = kSB - 1; i >= 0; --i) {
@@ -865,8 +922,8 @@ struct OutView {
   int64_t off, sc, sz, sy, sx;
 };
 
-// Lines along one axis of an unpadded array (nx a multiple of 4, rows
-// 16-byte aligned): the source's line stride sv.sz, blockIdx.y the other
+// Lines along one axis of an unpadded array (nx a multiple of PE, rows
+// aligned to PE values): the source's line stride sv.sz, blockIdx.y the other
 // axis at stride sv.sy; ZT columns of x per block, one thread per (column,
 // component), streaming the nl lines.  It may write in place (a thread
 // reads all of its pencil's lines before it writes them).  LPC = 1: one
@@ -876,13 +933,13 @@ struct OutView {
 // stage holds kSB lines of the block's columns per component (component
 // blocks padded by 8 floats: the three components of a column fall on
 // distinct banks).
-template <int LPC, int ZT, int S>
+template <int LPC, int ZT, int S, int PE>
 __global__ void __launch_bounds__(ZT * LPC, 1024 / (ZT * LPC)) solve_line_stream(
     const float* src, View sv, float* dst, OutView ov, int nx, int nl, float z, float gain) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NCB = LPC == 1 ? 1 : 3;               // components per block
   constexpr int CS = kSB * ZT + (LPC == 1 ? 0 : 8);   // one component's lines
-  constexpr int T = ZT * LPC, PL = ZT / 4;            // 16-byte pieces per line
+  constexpr int T = ZT * LPC, PL = ZT / PE;           // pieces of PE values per line
   float* stage = reinterpret_cast<float*>(smem_raw);  // [S][NCB][CS]
   const int t = threadIdx.x;
   const int col = t / LPC, x0 = blockIdx.x * ZT, x = x0 + col;
@@ -892,10 +949,10 @@ __global__ void __launch_bounds__(ZT * LPC, 1024 / (ZT * LPC)) solve_line_stream
   const int sz = (int)ov.sz;  // < 2^31 elements per plane
   float* op = dst + ov.off + (c0 + k) * ov.sc + blockIdx.y * ov.sy + x * ov.sx;
   const float og = pad ? 0.f : gain;
-  const bool xin = 4 * (t % PL) < nx - x0;
+  const bool xin = PE * (t % PL) < nx - x0;
 
   // piece p = t + T u of a chunk: line (p / PL) % kSB of component
-  // p / (PL kSB), 16 bytes at 4 (p % PL)
+  // p / (PL kSB), PE values at PE (p % PL)
   auto copy = [&](int q) {
     const int len = sb_len(q, nl), r0 = sb_start(q, nl);
     float* st = stage + (q % S) * NCB * CS;
@@ -904,7 +961,8 @@ __global__ void __launch_bounds__(ZT * LPC, 1024 / (ZT * LPC)) solve_line_stream
     for (int p = t; p < NCB * kSB * PL; p += T) {
       const int m = p % PL, j = (p / PL) % kSB, kk = p / (PL * kSB);
       if (j < len)
-        cp_async16(st + kk * CS + j * ZT + 4 * m, sp + kk * sv.sc + (r0 + j) * sv.sz + 4 * m);
+        cp_async_piece<PE>(st + kk * CS + j * ZT + PE * m,
+                           sp + kk * sv.sc + (r0 + j) * sv.sz + PE * m);
     }
   };
   auto read = [&](int q, float (&g)[kSB]) {
@@ -1142,58 +1200,129 @@ ps_status launch_x_node4(const float* src, View sv, NodeT* dst, float* scale4, i
 }
 
 // Two-pass solve: applies to FP32 fields and FP32 coefficients (planar or
-// nodes) when a row is 128, 256 or 512 values (a warp's chunks of 4, 8 or
-// 16) and every streamed pencil holds two chunks (tune "solve_stream" 0
-// keeps the three passes).  It needs the unpadded FP32 intermediate in the
-// workspace.
+// nodes) when a thread per value of a row fits a block (64 to 768 values; a
+// stage of 16 rows of 768 takes 55 KB, three of them one block per SM), every
+// streamed pencil holds two chunks and the planes are many or large enough
+// (tune "solve_stream" 0 keeps the three passes).  It needs the unpadded FP32 intermediate in the workspace.
 bool stream_grid(const ps_grid* g) {
   const int nx = g->n[0];
-  return (nx == 128 || nx == 256 || nx == 512) && g->n[1] >= 2 * kSB && g->n[2] >= 2 * kSB;
+  return nx >= 64 && nx <= 768 && g->n[1] >= 2 * kSB && g->n[2] >= 2 * kSB;
 }
-bool stream_solve_ok(const ps_grid* g) {
-  return tuning().solve_stream && stream_grid(g);
+// Values of a lane's chunk for rows of nx: the smallest that covers the row
+// with 32 lanes, or a larger one that cuts it into whole chunks (a chunk cut
+// short takes the predicated path besides the full one).
+int xy_chunk(int nx) {
+  const int least = (nx + 127) / 128 * 4;
+  for (int L = least; L <= 24 && nx % 4 == 0; L += 4)
+    if (nx % L == 0) return L;
+  return least;
+}
+// Rows other than 128, 256 and 512 values: whether the x-y pass beats the y and
+// the x pass it replaces.  A block works through its plane in chunks of 16
+// rows, each warp solving its share of a chunk's rows one after the other
+// (about 0.5 us and 0.1 us per value of a lane's chunk each, 1.7 times that
+// when the last chunk is cut short); the two passes take about 7 us and 5 us
+// per million values.  Measured, three components, three -> two passes, us:
+// 96^3 34 -> 52, 112^3 45 -> 50, 64 x 700 x 40 89 -> 353 (kept at three);
+// 100 x 60 x 300 68 -> 53, 192^3 137 -> 92, 250 x 200 x 150 170 -> 111,
+// 300^3 567 -> 318, 384^3 960 -> 520.
+bool xy_stream_pays(const ps_grid* g, int ncomp) {
+  const int nx = g->n[0], L = xy_chunk(nx), warps = (nx + 31) / 32;
+  const int64_t planes = (int64_t)ncomp * g->n[2];
+  const int64_t fit = (int64_t)sm_count() * std::max(1, 768 / (32 * warps));
+  const double waves = (double)((planes + fit - 1) / fit);
+  const double row = (0.5 + 0.1 * L) * (nx % L ? 1.7 : 1.0);
+  const double xy = waves * ((double)g->n[1] / kSB + 2) * ((kSB + warps - 1) / warps) * row;
+  return xy < 7.0 + 5e-6 * (double)ncomp * (double)grid_volume(g);
+}
+// `rows3` keeps the three passes on rows other than 128, 256 or 512 values.
+bool stream_solve_ok(const ps_grid* g, int ncomp, bool rows3 = false) {
+  const int nx = g->n[0];
+  if (!tuning().solve_stream || !stream_grid(g)) return false;
+  if (nx == 128 || nx == 256 || nx == 512) return true;
+  return !rows3 && xy_stream_pays(g, ncomp);
+}
+// The gains of the x-y and the z pass.  Rows of 128, 256 and 512 values take
+// the three axes' gain one by one, others all three in the z pass: two
+// roundings fewer per value (rms error against 64 bits on white noise, rows of
+// 510: 8.1e-7 with a gain per axis).
+struct StreamGains {
+  float xy, z;
+};
+StreamGains stream_gains(int nx, float gain) {
+  if (nx == 128 || nx == 256 || nx == 512) return {gain, gain};
+  return {1.f, (float)((double)gain * gain * gain)};
+}
+// Values per copy of rows of nx floats starting at a and b.
+int piece_of(int nx, const void* a, const void* b) {
+  const uintptr_t p = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+  return nx % 4 == 0 && p % 16 == 0 ? 4 : nx % 2 == 0 && p % 8 == 0 ? 2 : 1;
 }
 
-template <int LMAX, int S>
-ps_status launch_xy_stream_s(const float* src, View sv, float* dst, View dv, int ny, int nz,
+template <int LMAX, int S, int PE, int ROWS>
+ps_status launch_xy_stream_s(const float* src, View sv, float* dst, View dv, int nx, int ny, int nz,
                              int ncomp, float z, float gain, cudaStream_t st) {
-  constexpr int NX = 32 * LMAX;
-  const size_t smem = (size_t)S * kSB * (NX + NX / 8) * sizeof(float);
-  auto kern = solve_xy_stream<LMAX, S>;
+  const int lanes = (nx + LMAX - 1) / LMAX, threads = (nx + 31) / 32 * 32;
+  const size_t smem = (size_t)S * kSB * xy_pitch(lanes * LMAX) * sizeof(float);
+  auto kern = solve_xy_stream<LMAX, S, PE, ROWS>;
   if (smem > 48 * 1024) {
     ps_status rc = check_cuda(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
         "solve_xy_stream smem attribute");
     if (rc) return rc;
   }
-  kern<<<(unsigned)(ncomp * nz), NX, smem, st>>>(src, sv, dst, dv, ny, nz, z, gain);
+  kern<<<(unsigned)(ncomp * nz), threads, smem, st>>>(src, sv, dst, dv, nx, ny, nz, z, gain);
   return check_launch("solve_xy_stream");
 }
 
-template <int LMAX>
-ps_status launch_xy_stream_l(const float* src, View sv, float* dst, View dv, int ny, int nz,
+template <int LMAX, int PE, int ROWS>
+ps_status launch_xy_stream_l(const float* src, View sv, float* dst, View dv, int nx, int ny, int nz,
                              int ncomp, float z, float gain, cudaStream_t st) {
-  const int S = tuning().solve_stages > 0 ? tuning().solve_stages : 3;
-  if (S == 2) return launch_xy_stream_s<LMAX, 2>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
-  if (S == 4) return launch_xy_stream_s<LMAX, 4>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
-  return launch_xy_stream_s<LMAX, 3>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
+  // (the tune key: full rows of up to 512 values, of which four stages fit)
+  if constexpr (ROWS == 0 && LMAX <= 16) {
+    const int S = tuning().solve_stages;
+    if (S == 2)
+      return launch_xy_stream_s<LMAX, 2, PE, ROWS>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st);
+    if (S == 4)
+      return launch_xy_stream_s<LMAX, 4, PE, ROWS>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st);
+  }
+  return launch_xy_stream_s<LMAX, 3, PE, ROWS>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st);
 }
 
-// nx = 128, 256 or 512 (stream_grid)
+// 64 <= nx <= 768 (stream_grid)
 ps_status launch_xy_stream(const float* src, View sv, float* dst, View dv, int nx, int ny,
                            int nz, int ncomp, float z, float gain, cudaStream_t st) {
-  if (nx == 128) return launch_xy_stream_l<4>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
-  if (nx == 256) return launch_xy_stream_l<8>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
-  return launch_xy_stream_l<16>(src, sv, dst, dv, ny, nz, ncomp, z, gain, st);
+  const int pe = piece_of(nx, src, nullptr);
+  const int chunk = xy_chunk(nx);
+#define PS_XY(L)                                                                            \
+  if (chunk == L) {                                                                         \
+    if (nx == 32 * L && pe == 4)                                                            \
+      return launch_xy_stream_l<L, 4, 0>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st); \
+    if (nx % L == 0 && pe == 4)                                                             \
+      return launch_xy_stream_l<L, 4, 1>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st); \
+    if (pe == 4)                                                                            \
+      return launch_xy_stream_l<L, 4, 2>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st); \
+    if (pe == 2)                                                                            \
+      return launch_xy_stream_l<L, 2, 2>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st); \
+    return launch_xy_stream_l<L, 1, 2>(src, sv, dst, dv, nx, ny, nz, ncomp, z, gain, st);   \
+  }
+  PS_XY(4)
+  PS_XY(8)
+  PS_XY(12)
+  PS_XY(16)
+  PS_XY(20)
+  PS_XY(24)
+#undef PS_XY
+  return fail(PS_ERR_UNSUPPORTED, "row of %d values", nx);
 }
 
-template <int LPC, int ZT>
+template <int LPC, int ZT, int PE>
 ps_status launch_line_stream_t(const float* src, View sv, float* dst, OutView ov, int nx,
                                int nother, int nl, int cblocks, float z, float gain,
                                cudaStream_t st) {
   constexpr int S = 4;
   const size_t smem = (size_t)S * (LPC == 1 ? 1 : 3) * (kSB * ZT + (LPC == 1 ? 0 : 8)) * 4;
-  auto kern = solve_line_stream<LPC, ZT, S>;
+  auto kern = solve_line_stream<LPC, ZT, S, PE>;
   if (smem > 48 * 1024) {
     ps_status rc = check_cuda(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
@@ -1213,8 +1342,15 @@ ps_status launch_line_stream(const float* src, View sv, float* dst, OutView ov, 
                              cudaStream_t st) {
   // measured at 512^3: one component 256 columns per block, nodes 64 (256 threads)
   const int zt = tuning().solve_zt > 0 ? tuning().solve_zt : (LPC == 1 ? 256 : 64);
-#define PS_LS(L, Z) \
-  return launch_line_stream_t<L, Z>(src, sv, dst, ov, nx, nother, nl, cblocks, z, gain, st)
+  const int pe = piece_of(nx, src, nullptr);
+#define PS_LS(L, Z)                                                                              \
+  do {                                                                                           \
+    if (pe == 4)                                                                                 \
+      return launch_line_stream_t<L, Z, 4>(src, sv, dst, ov, nx, nother, nl, cblocks, z, gain, st); \
+    if (pe == 2)                                                                                 \
+      return launch_line_stream_t<L, Z, 2>(src, sv, dst, ov, nx, nother, nl, cblocks, z, gain, st); \
+    return launch_line_stream_t<L, Z, 1>(src, sv, dst, ov, nx, nother, nl, cblocks, z, gain, st); \
+  } while (0)
   if (LPC == 1) {
     if (zt <= 32) PS_LS(1, 32);
     if (zt <= 64) PS_LS(1, 64);
@@ -1303,10 +1439,11 @@ ps_status run_solve_stream_planar(const ps_grid* g, int ncomp, const float* fiel
   const float z = (float)zd, gain = (float)(-6.0 * zd);
   const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
   View fv = unpadded_view(g), pv = padded_view(g, rx);
-  ps_status rc = launch_xy_stream(field, fv, inter, fv, nx, ny, nz, ncomp, z, gain, st);
+  const StreamGains sg = stream_gains(nx, gain);
+  ps_status rc = launch_xy_stream(field, fv, inter, fv, nx, ny, nz, ncomp, z, sg.xy, st);
   if (rc) return rc;
   OutView ov{pv.off + pv.sz + pv.sy + 1, pv.sc, pv.sz, pv.sy, 1};  // the interior
-  rc = launch_line_stream<1>(inter, fv, coef, ov, nx, ny, nz, ncomp, z, gain, st);
+  rc = launch_line_stream<1>(inter, fv, coef, ov, nx, ny, nz, ncomp, z, sg.z, st);
   if (rc) return rc;
   return launch_fill_images<float>(coef, pv.sc, rx, nx, ny, nz, ncomp, st);
 }
@@ -1321,12 +1458,13 @@ ps_status run_solve_stream_node4(const ps_grid* g, const float* field, float* in
   const float z = (float)zd, gain = (float)(-6.0 * zd);
   const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
   View fv = unpadded_view(g);
-  ps_status rc = launch_xy_stream(field, fv, inter, fv, nx, ny, nz, 3, z, gain, st);
+  const StreamGains sg = stream_gains(nx, gain);
+  ps_status rc = launch_xy_stream(field, fv, inter, fv, nx, ny, nz, 3, z, sg.xy, st);
   if (rc) return rc;
   const int64_t my = ny + 3;
   OutView ov{(my * rx + rx + 1) * 4, 1, my * rx * 4, rx * 4, 4};  // the interior
   rc = launch_line_stream<4>(inter, fv, reinterpret_cast<float*>(out), ov, nx, ny, nz, 1, z,
-                             gain, st);
+                             sg.z, st);
   if (rc) return rc;
   return launch_fill_images<float4>(out, 0, rx, nx, ny, nz, 1, st);
 }
@@ -1419,6 +1557,18 @@ ps_status run_solve_node4(const ps_grid* g, const Tin* field, View fv, float* in
 ps_status solve_unpadded_inplace_f32(const ps_grid* g, int ncomp, float* a,
                                      cudaStream_t st) {
   View v = unpadded_view(g);
+  if (stream_solve_ok(g, ncomp)) {
+    // x and y of every plane, then z, both in place
+    const double zd = sqrt(3.0) - 2.0;
+    if (ps_status rc = upload_zpow(zd)) return rc;
+    const float z = (float)zd, gain = (float)(-6.0 * zd);
+    const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
+    const StreamGains sg = stream_gains(nx, gain);
+    ps_status rc = launch_xy_stream(a, v, a, v, nx, ny, nz, ncomp, z, sg.xy, st);
+    if (rc) return rc;
+    return launch_line_stream<1>(a, v, a, OutView{0, v.sc, v.sz, v.sy, 1}, nx, ny, nz, ncomp, z,
+                                 sg.z, st);
+  }
   return run_solve<float, float, float, false>(g, ncomp, a, v, a, v, a, v, nullptr, 0, st);
 }
 
@@ -1436,10 +1586,9 @@ extern "C" size_t ps_spline_coeffs_workspace_size(const ps_grid* grid, int ncomp
   return 0;
 }
 
-extern "C" ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype field_t,
-                                      const void* field, ps_dtype coef_t, void* coef,
-                                      float* scale, void* ws, size_t ws_bytes,
-                                      void* stream) {
+static ps_status spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype field_t,
+                               const void* field, ps_dtype coef_t, void* coef, float* scale,
+                               void* ws, size_t ws_bytes, void* stream, bool rows3) {
   ps_status rc = validate_grid(grid);
   if (rc) return rc;
   if (ncomp < 1 || ncomp > 16) return fail(PS_ERR_INVALID_ARG, "ncomp=%d outside [1,16]", ncomp);
@@ -1470,7 +1619,7 @@ extern "C" ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype f
     // the three passes in place
     const size_t inter_bytes = (size_t)ncomp * (size_t)grid_volume(grid) * sizeof(float);
     const bool have_ws = ws && ws_bytes >= inter_bytes && (reinterpret_cast<uintptr_t>(ws) & 255) == 0;
-    if (field_t == PS_F32 && stream_solve_ok(grid) && aligned16 && have_ws)
+    if (field_t == PS_F32 && stream_solve_ok(grid, ncomp, rows3) && have_ws && (!rows3 || aligned16))
       return run_solve_stream_planar(grid, ncomp, ff, static_cast<float*>(ws), c, rx, st);
     if (field_t == PS_F32 && tuning().solve_stream && stream3_grid(grid) && aligned16 && have_ws)
       return run_solve<float, float, float, false>(grid, ncomp, ff, fv, static_cast<float*>(ws),
@@ -1496,7 +1645,7 @@ extern "C" ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype f
   float* inter = static_cast<float*>(ws);
   if (coef_t == PS_F32X4) {
     float4* c = static_cast<float4*>(coef);
-    if (field_t == PS_F32 && stream_solve_ok(grid) && aligned16)
+    if (field_t == PS_F32 && stream_solve_ok(grid, ncomp, rows3) && (!rows3 || aligned16))
       return run_solve_stream_node4(grid, ff, inter, c, rx, st);
     return field_t == PS_F32 ? run_solve_node4<float>(grid, ff, fv, inter, c, nullptr, rx, st)
                              : run_solve_node4<double>(grid, fd, fv, inter, c, nullptr, rx, st);
@@ -1525,4 +1674,20 @@ extern "C" ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype f
                                                      scale, 1, st)
              : run_solve<double, float, __half, true>(grid, ncomp, fd, fv, inter, fv, c, pv,
                                                       scale, 1, st);
+}
+
+extern "C" ps_status ps_spline_coeffs(const ps_grid* grid, int ncomp, ps_dtype field_t,
+                                      const void* field, ps_dtype coef_t, void* coef,
+                                      float* scale, void* ws, size_t ws_bytes,
+                                      void* stream) {
+  return spline_coeffs(grid, ncomp, field_t, field, coef_t, coef, scale, ws, ws_bytes, stream,
+                       false);
+}
+
+extern "C" ps_status ps_spline_coeffs_rows3(const ps_grid* grid, int ncomp, ps_dtype field_t,
+                                            const void* field, ps_dtype coef_t, void* coef,
+                                            float* scale, void* ws, size_t ws_bytes,
+                                            void* stream) {
+  return spline_coeffs(grid, ncomp, field_t, field, coef_t, coef, scale, ws, ws_bytes, stream,
+                       true);
 }

@@ -165,3 +165,34 @@ def test_autograd_bins_enough_particles():
         tol = 1e-5 * 3 * (n[d] / TWO_PI) * np.abs(cref).max() * np.abs(w).sum(0).max()
         assert np.abs(gp[d].cpu().numpy() - gp_ref[d]).max() <= tol
     assert np.abs(gf.cpu().numpy() - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
+
+
+@pytest.mark.parametrize("n", [(100, 60, 300), (192, 64, 101), (250, 200, 100), (255, 200, 90),
+                               (300, 64, 50), (320, 49, 75), (384, 64, 50), (510, 64, 50),
+                               (640, 33, 50), (767, 50, 50), (768, 33, 50)])
+def test_streamed_solve_of_any_row(n):
+    # grids that take two passes, with rows that fill a warp's chunks, leave its
+    # last lanes empty or a lane's chunk cut short, copied in pieces of 4, 2 and
+    # 1 values; nodes and planar rows hold the same bits, the transposed solve
+    # (in place) the same values
+    field = synth.random_field(n, ncomp=3, seed=45).astype(np.float32)
+    f = torch.from_numpy(field).to(DEV)
+    ref = oracle.spline_coeffs(field.astype(np.float64))
+    tol = 2e-6 * np.abs(field).max()
+    p4 = ps.SplineField.from_field(f, ps.F32X4)
+    p32 = ps.SplineField.from_field(f, torch.float32)
+    assert np.abs(p32.padded().cpu().numpy() - ref).max() <= tol
+    assert torch.equal(p4.padded(), p32.padded())
+    assert torch.count_nonzero(p32.coef[..., n[0] + 3:]) == 0
+    # an offset start: the field is 4-byte aligned only
+    g = torch.empty(f.numel() + 1, device=DEV)[1:].view_as(f).copy_(f)
+    q32 = ps.SplineField.from_field(g, torch.float32)
+    assert torch.equal(q32.padded(), p32.padded())
+    # the transposed solve, after a scatter
+    pos = synth.uniform_particles(3000, seed=46)
+    w = np.random.Generator(np.random.PCG64(47)).standard_normal((3, 3000)).astype(np.float32)
+    _, gf_ref = oracle.interp_backward(ref, pos, w.astype(np.float64))
+    gf = torch.empty((3,) + tuple(reversed(n)), device=DEV)
+    ps.ps_interp_backward(p32.coef, n, torch.from_numpy(pos).to(DEV), torch.from_numpy(w).to(DEV),
+                          None, gf)
+    assert np.abs(gf.cpu().numpy() - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
