@@ -366,6 +366,12 @@ ps_status ps_lagrangian_accel(const ps_grid* grid, ps_dtype coef_t,
 /*   or too small, or without perm: as the calls above.                      */
 /* ------------------------------------------------------------------------ */
 size_t ps_unsort_workspace_size(int64_t np, int rows);
+/* Rows [rows][np] of 4- or 8-byte elements between the particles' order and  */
+/* bin order: to_bins = 1, dst[r][s] = src[r][perm[s]]; 0, dst[r][perm[s]] =  */
+/* src[r][s].  src and dst must not overlap; rows <= 64.                      */
+ps_status ps_permute_rows(int64_t np, int rows, int elem_bytes,
+                          const int64_t* perm, const void* src, void* dst,
+                          int to_bins, void* stream);
 ps_status ps_interp_ws(const ps_grid* grid, int ncomp, ps_dtype coef_t,
                        const void* coef, const float* scale, int64_t np,
                        const double* pos, const int64_t* perm,

@@ -334,6 +334,19 @@ def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Te
                                      _ptr(g_field), None, 0, _ptr(status), _stream(stream)))
 
 
+def ps_permute_rows(src: torch.Tensor, perm: torch.Tensor, dst: torch.Tensor, to_bins: bool,
+                    stream=None):
+    """Rows [..., np] of 4- or 8-byte elements: dst[r, s] = src[r, perm[s]] (to_bins) or
+    dst[r, perm[s]] = src[r, s]."""
+    np_ = src.shape[-1]
+    _dev(src, "src")
+    _dev(dst, "dst", src.dtype, src.numel())
+    _dev(perm, "perm", torch.int64, np_)
+    rows = src.numel() // np_ if np_ else 0
+    _check(_lib().ps_permute_rows(np_, rows, src.element_size(), _ptr(perm), _ptr(src), _ptr(dst),
+                                  1 if to_bins else 0, _stream(stream)))
+
+
 def ps_backward_workspace_size(n, brick, L=DEFAULT_L) -> int:
     return int(_lib().ps_backward_workspace_size(ctypes.byref(make_grid(n, L)), _brick_arr(brick)))
 
@@ -467,9 +480,11 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
     return t
 
 
-# Result rows from this size on go through bin order (see ps_interp_ws): about half
-# the L2, beyond which scattered 4-byte stores reach DRAM one by one.
-_UNSORT_BYTES = 48 << 20
+# Result rows from this size on go through bin order (see ps_interp_ws): beyond a good
+# half of the L2, scattered 4-byte stores reach DRAM one by one.  Stored directly / by
+# way of bin order, us: 34 MiB 86 / 133, 46 MiB 386 / 392, 69 MiB 159 / 247,
+# 92 MiB 594 / 390 and 1011 / 742, 183 MiB 1668 / 741, 549 MiB 5697 / 1934.
+_UNSORT_BYTES = 80 << 20
 
 
 def _unsort_ws(bins: Optional["Bins"], np_: int, rows: int, device):
@@ -655,11 +670,22 @@ class Tracker:
         self._counted = mode >= 2 and self.brick is not None
 
 
-# Particles of one differentiable call from which, and per brick of 8^3 cells on average
-# from which, binning them first pays (forward and both gradients go brick by brick).
+# Particles of one differentiable call from which binning them first pays (forward and
+# both gradients go brick by brick).  Forward and backward in particle order / binned, us:
+#   256^3: 100 k particles 646 / 884, 200 k 902 / 910, 500 k 1667 / 995, 1 M 2950 / 1194
+#   128^3: 200 k 339 / 502, 500 k 468 / 511, 1 M 796 / 655;  64^3: 1 M 745 / 706
+# Coefficients that the L2 holds are gathered from it at any order, and the binned way has
+# more launches; beyond it, binning pays from some particles per brick.
 _FN_BRICK = (8, 8, 8)
-_FN_MIN_PARTICLES = 50_000
+_FN_L2_BYTES = 64 << 20
+_FN_MIN_IN_L2 = 800_000
 _FN_MIN_PER_BRICK = 8
+
+
+def _fn_binned(n, np_: int) -> bool:
+    nbins = math.prod(-(-n[d] // _FN_BRICK[d]) for d in range(3))
+    least = _FN_MIN_IN_L2 if 12 * math.prod(n) <= _FN_L2_BYTES else 0
+    return max(least, _FN_MIN_PER_BRICK * nbins) <= np_ < 2**31
 
 
 class InterpFn(torch.autograd.Function):
@@ -671,44 +697,67 @@ class InterpFn(torch.autograd.Function):
     def forward(ctx, pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L):
         sf = SplineField.from_field(field.detach().float(), torch.float32, L, rows3=True)
         x = pos.detach()
-        bins = None
-        nbins = math.prod(-(-sf.n[d] // _FN_BRICK[d]) for d in range(3))
-        if (sf.ncomp == 3 and x.shape[1] >= max(_FN_MIN_PARTICLES, _FN_MIN_PER_BRICK * nbins)
-                and x.shape[1] < 2**31):
-            bins = bin_particles(sf.n, _FN_BRICK, x, L)
-            bins.bin_of = None  # the backward needs the order alone
-        vel = sf.interp(x, bins=bins)
+        order = None
+        if sf.ncomp == 3 and _fn_binned(sf.n, x.shape[1]):
+            # positions in bin order serve the forward and both gradients; what
+            # goes in or out in the particles' own order is moved by rows
+            try:
+                bins, xs = bin_particles(sf.n, _FN_BRICK, x, L, want_sorted=True)
+                vs = sf.interp(xs, bins=Bins(_FN_BRICK, bins.offsets, None))
+                vel = torch.empty_like(vs)
+                ps_permute_rows(vs, bins.perm, vel, to_bins=False)
+                order = (bins.perm, bins.offsets, xs)
+            except torch.cuda.OutOfMemoryError:
+                order = None  # the direct way needs no further memory
+        if order is None:
+            vel = sf.interp(x)
         ctx.save_for_backward(pos)
         ctx.sf = sf
-        ctx.bins = bins
+        ctx.order = order
         ctx.field_dtype = field.dtype
         return vel
 
     @staticmethod
     def backward(ctx, g_vel):
         (pos,) = ctx.saved_tensors
-        sf, bins = ctx.sf, ctx.bins
+        sf = ctx.sf
         g_vel = g_vel.contiguous().float()
         want_pos = ctx.needs_input_grad[0]
         want_field = ctx.needs_input_grad[1]
         g_pos = torch.empty_like(pos) if want_pos else None
         g_field = (torch.empty((sf.ncomp, sf.n[2], sf.n[1], sf.n[0]), dtype=torch.float32,
                                device=pos.device) if want_field else None)
-        ws = None
-        if bins is not None and want_field:
-            try:
-                ws = workspace(ps_backward_workspace_size(sf.n, bins.brick, sf.L), pos.device)
-            except torch.cuda.OutOfMemoryError:
-                pass  # the bricks' sums then go to the field by atomics
         if want_pos or want_field:
-            ps_interp_backward(sf.coef, sf.n, pos.detach(), g_vel, g_pos, g_field,
-                               scale=sf.scale, L=sf.L, ws=ws,
-                               perm=bins.perm if bins is not None else None,
-                               bin_offsets=bins.offsets if bins is not None else None,
-                               brick=bins.brick if bins is not None else None)
+            if ctx.order is None or not InterpFn._binned_backward(ctx, g_vel, g_pos, g_field):
+                ps_interp_backward(sf.coef, sf.n, pos.detach(), g_vel, g_pos, g_field,
+                                   scale=sf.scale, L=sf.L)
         if g_field is not None:
             g_field = g_field.to(ctx.field_dtype)
         return g_pos, g_field, None
+
+    @staticmethod
+    def _binned_backward(ctx, g_vel, g_pos, g_field) -> bool:
+        """Both gradients over the particles in bin order; False where the memory for the
+        reordered arrays is not there."""
+        sf = ctx.sf
+        perm, offsets, xs = ctx.order
+        try:
+            gs = torch.empty_like(g_vel)
+            ps_sorted = torch.empty_like(xs) if g_pos is not None else None
+        except torch.cuda.OutOfMemoryError:
+            return False
+        ws = None
+        if g_field is not None:
+            try:
+                ws = workspace(ps_backward_workspace_size(sf.n, _FN_BRICK, sf.L), xs.device)
+            except torch.cuda.OutOfMemoryError:
+                pass  # the bricks' sums then go to the field by atomics
+        ps_permute_rows(g_vel, perm, gs, to_bins=True)
+        ps_interp_backward(sf.coef, sf.n, xs, gs, ps_sorted, g_field, scale=sf.scale, L=sf.L,
+                           bin_offsets=offsets, brick=_FN_BRICK, ws=ws)
+        if g_pos is not None:
+            ps_permute_rows(ps_sorted, perm, g_pos, to_bins=False)
+        return True
 
 
 class BatchPlan:

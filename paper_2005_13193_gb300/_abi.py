@@ -58,6 +58,7 @@ SIGNATURES = {
     "ps_bin_particles_noalloc": (_I, [_GP, _P, _I64, _P, _P, _P, _P, _P, _P, _P]),
     "ps_interp": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _P, _P, _P]),
     "ps_unsort_workspace_size": (_SZ, [_I64, _I]),
+    "ps_permute_rows": (_I, [_I64, _I, _I, _P, _P, _P, _I, _P]),
     "ps_interp_ws": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _P, _P, _SZ, _P, _P]),
     "ps_interp_hessian_ws": (_I, [_GP, _I, _I, _P, _P, _I64, _P, _P, _P, _P, _P, _P, _SZ, _P,
                                   _P]),

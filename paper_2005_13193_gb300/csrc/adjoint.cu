@@ -14,7 +14,11 @@
 // per axis that reach it; without a workspace (or where the bricks do not tile
 // the grid) they go to the field by atomics, one per node and component
 // (1411 us in all at that size, bound by the atomics' rate, about 1.8e11 a
-// second).  Measured there: 4447 us of atomics -> 875 + 306 us.
+// second).  Measured there: 4447 us of atomics -> 549 us for the bricks and
+// 171 us for the sums (875 and 306 us before a round's records held the products
+// of the x and y weights, read one particle ahead, and before a thread summed all
+// three components of its node).  What bounds it is the chain load, add, store of
+// a warp's float4, one per particle.
 #include <algorithm>
 
 #include "brick.cuh"
@@ -41,13 +45,14 @@ struct ScatterArgs {
   int32_t* status;
 };
 
-// Records of a round's particles: weights per axis (z in the order 0, 2, 1, 3,
-// so that a lane finds its plane's at 2 * first row + plane), (g_u, g_v, g_w, twice
-// the stencil's first node plus the parity of its first plane; -1 outside the
-// halo, -2 not finite), the cell.
+// Records of a round's particles: the 16 products of the x and y weights (in
+// the order of the lanes), the z weights in the order 0, 2, 1, 3 (a lane finds
+// its plane's at 2 * first row + plane), (g_u, g_v, g_w, twice the stencil's
+// first node plus the parity of its first plane; -1 outside the halo, -2 not
+// finite).
 struct ScatterRecs {
-  float4 bx[kScatterThreads], by[kScatterThreads], bz[kScatterThreads], gi[kScatterThreads];
-  int cell[3][kScatterThreads];
+  float4 wxy[kScatterThreads][4];
+  float4 bz[kScatterThreads], gi[kScatterThreads];
 };
 
 __device__ __forceinline__ void add_global(const ScatterArgs& a, int cx, int cy, int cz, float w,
@@ -77,8 +82,7 @@ __device__ __forceinline__ void scatter_segment(const ScatterArgs& a, int bin, i
   }
   float4* mine = acc + 2 * lk * a.PS + lj * a.SX + li;  // + the warp's first plane of a stencil
   const float* wz = reinterpret_cast<const float*>(R.bz) + lk;
-  const float* wx = reinterpret_cast<const float*>(R.bx) + li;
-  const float* wy = reinterpret_cast<const float*>(R.by) + lj;
+  const float* wxy = reinterpret_cast<const float*>(R.wxy) + (lane & 15);
   for (int c0 = lo; c0 < hi; c0 += kScatterThreads) {
     const int m = min(kScatterThreads, hi - c0);
     if (tid < m) {
@@ -109,44 +113,55 @@ __device__ __forceinline__ void scatter_segment(const ScatterArgs& a, int bin, i
         first = 2 * (l2 * a.PS + l1 * a.SX + l0) + (l2 & 1);
       }
       gi.w = __int_as_float(first);
-      float b[4];
+      float b[4], by4[4];
       qbasis(t[0], b);
-      R.bx[tid] = make_float4(b[0], b[1], b[2], b[3]);
-      qbasis(t[1], b);
-      R.by[tid] = make_float4(b[0], b[1], b[2], b[3]);
+      qbasis(t[1], by4);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        R.wxy[tid][j] = make_float4(b[0] * by4[j], b[1] * by4[j], b[2] * by4[j], b[3] * by4[j]);
       qbasis(t[2], b);
       R.bz[tid] = make_float4(__fmul_rn(b[0], kZScale), __fmul_rn(b[2], kZScale),
                               __fmul_rn(b[1], kZScale), __fmul_rn(b[3], kZScale));
       R.gi[tid] = gi;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) R.cell[d][tid] = cell[d];
     }
     __syncthreads();
     // the records of one particle ahead of the sums
     float4 gn = R.gi[0];
-    float wxy = wx[0] * wy[0];
+    float wn = wxy[0];
+#pragma unroll 2
     for (int i = 0; i < m; ++i) {
       const float4 g = gn;
-      const float wp = wxy;
-      const int first = __float_as_int(g.w), nxt = min(i + 1, m - 1);
+      const float wp = wn;
+      const int first = __float_as_int(g.w);
       if (first >= 0) {  // (uniform over the warp)
         const int row0 = (first & 1) ^ warp;  // the stencil's first plane of this warp
-        float4* q = mine + (first >> 1) + row0 * a.PS;
+        float4* q = mine + ((first >> 1) + row0 * a.PS);
         float4 v = *q;
         const float w = wp * wz[4 * i + 2 * row0];
-        gn = R.gi[nxt];
-        wxy = wx[4 * nxt] * wy[4 * nxt];
+        if (i + 1 < m) {
+          gn = R.gi[i + 1];
+          wn = wxy[16 * (i + 1)];
+        }
         v.x = fmaf(w, g.x, v.x);
         v.y = fmaf(w, g.y, v.y);
         v.z = fmaf(w, g.z, v.z);
         *q = v;
         __syncwarp();  // the next stencil's nodes may be other lanes'
       } else {
-        if (first == -1)  // planes warp and warp + 2 of the stencil
-          add_global(a, R.cell[0][i] + li, R.cell[1][i] + lj, R.cell[2][i] + warp + 2 * lk,
+        if (first == -1) {  // planes warp and warp + 2 of the stencil
+          const int64_t p = a.perm ? a.perm[c0 + i] : (int64_t)(c0 + i);
+          int cell[3];
+          float t;
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+            locate(a.pos[d * a.np + p], a.g.inv_h[d], a.g.n[d], cell[d], t);
+          add_global(a, cell[0] + li, cell[1] + lj, cell[2] + warp + 2 * lk,
                      wp * wz[4 * i + 2 * warp], g);
-        gn = R.gi[nxt];
-        wxy = wx[4 * nxt] * wy[4 * nxt];
+        }
+        if (i + 1 < m) {
+          gn = R.gi[i + 1];
+          wn = wxy[16 * (i + 1)];
+        }
       }
     }
     __syncthreads();  // the records are refilled, or the sums are complete
@@ -221,7 +236,8 @@ __global__ void __launch_bounds__(kScatterThreads) scatter_bricks(const __grid_c
 // gfield += the bricks' sums.  Node i of an axis lies in the halo of the bricks
 // b with b B - 1 <= i <= b B + B + 1 (mod n): floor((i + 1) / B), and the one
 // before where i + 1 - b B <= 2.  A block per (z, y) row (the bricks along y
-// and z and their offsets are the block's), blockIdx.y the component.
+// and z and their offsets are the block's), a thread per node and all three
+// components.
 struct Reach {
   int brick[2], l[2];
   bool two;
@@ -240,29 +256,34 @@ __global__ void __launch_bounds__(128) gather_sums(const __grid_constant__ Scatt
   const int nx = a.g.n[0], ny = a.g.n[1], z = blockIdx.x / ny, y = blockIdx.x - z * ny;
   const int e1 = a.PS * a.S[2];
   const Reach rz = reach(z, a.b.B[2], a.b.nb[2]), ry = reach(y, a.b.B[1], a.b.nb[1]);
-  float* o = a.gfield + ((int64_t)blockIdx.y * a.g.n[2] * ny + blockIdx.x) * nx;
+  const int64_t vol = (int64_t)a.g.n[2] * ny * nx;
+  float* o = a.gfield + (int64_t)blockIdx.x * nx;
   const float* base[2][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      base[i][j] = a.sums +
-                   (((int64_t)rz.brick[i] * a.b.nb[1] + ry.brick[j]) * a.b.nb[0] * 3 + blockIdx.y) *
-                       e1 + rz.l[i] * a.PS + ry.l[j] * a.SX;
+      base[i][j] = a.sums + ((int64_t)rz.brick[i] * a.b.nb[1] + ry.brick[j]) * a.b.nb[0] * 3 * e1 +
+                   rz.l[i] * a.PS + ry.l[j] * a.SX;
   for (int x = threadIdx.x; x < nx; x += blockDim.x) {
     const Reach rx = reach(x, a.b.B[0], a.b.nb[0]);
-    const int64_t x0 = (int64_t)rx.brick[0] * 3 * e1 + rx.l[0];
-    const int64_t x1 = (int64_t)rx.brick[1] * 3 * e1 + rx.l[1];
-    float s = o[x];
+    const int x0 = rx.brick[0] * 3 * e1 + rx.l[0], x1 = rx.brick[1] * 3 * e1 + rx.l[1];
+    float s[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s[c] = o[c * vol + x];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 2; ++j)
         if ((i == 0 || rz.two) && (j == 0 || ry.two)) {
-          s += __ldg(base[i][j] + x0);
-          if (rx.two) s += __ldg(base[i][j] + x1);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            s[c] += __ldg(base[i][j] + c * e1 + x0);
+            if (rx.two) s[c] += __ldg(base[i][j] + c * e1 + x1);
+          }
         }
-    o[x] = s;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) o[c * vol + x] = s[c];
   }
 }
 
@@ -319,7 +340,7 @@ ps_status scatter_bricks_launch(const ps_grid* grid, const int32_t brick[3], int
   const int64_t blocks = a.b.nbins + (np + kSegment - 1) / kSegment;
   scatter_bricks<<<(unsigned)blocks, kScatterThreads, smem, st>>>(a);
   if ((rc = check_launch("scatter_bricks")) || !a.sums) return rc;
-  gather_sums<<<dim3((unsigned)(a.g.n[1] * a.g.n[2]), 3), 128, 0, st>>>(a);
+  gather_sums<<<(unsigned)(a.g.n[1] * a.g.n[2]), 128, 0, st>>>(a);
   return check_launch("gather_sums");
 }
 

@@ -110,6 +110,20 @@ def test_results_by_way_of_bin_order(dtype):
                                                      scale_np1=sf.scale, vel=o[:3], ws=ws, **kw))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64, torch.int64])
+@pytest.mark.parametrize("np_,rows", [(1, 1), (1023, 3), (1025, 18), (70000, 5)])
+def test_permute_rows(dtype, np_, rows):
+    g = torch.Generator(DEV).manual_seed(np_)
+    perm = torch.randperm(np_, device=DEV, generator=g)
+    src = torch.randint(-2**20, 2**20, (rows, np_), device=DEV, generator=g).to(dtype)
+    dst = torch.empty_like(src)
+    ps.ps_permute_rows(src, perm, dst, to_bins=True)
+    assert torch.equal(dst, src[:, perm])
+    back = torch.empty_like(src)
+    ps.ps_permute_rows(dst, perm, back, to_bins=False)
+    assert torch.equal(back, src)
+
+
 @pytest.mark.parametrize("n,brick", [((24, 16, 40), (8, 8, 8)), ((9, 21, 5), (8, 8, 8)),
                                      ((3, 4, 5), (8, 8, 8)), ((20, 18, 12), (5, 7, 3)),
                                      ((40, 8, 8), (20, 4, 4)), ((32, 16, 24), (8, 8, 8))])
@@ -148,7 +162,9 @@ def test_binned_adjoint(n, brick, crowd):
         assert np.abs(gf - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
 
 
-def test_autograd_bins_enough_particles():
+@pytest.mark.parametrize("least", [0, 10**6])
+def test_autograd_bins_enough_particles(least, monkeypatch):
+    monkeypatch.setattr(ps, "_FN_MIN_IN_L2", least)  # binned, and in the particles' order
     n = (32, 24, 16)
     field = synth.random_field(n, ncomp=3, seed=35).astype(np.float32)
     cref = oracle.spline_coeffs(field.astype(np.float64))
