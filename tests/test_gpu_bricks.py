@@ -212,3 +212,12 @@ def test_streamed_solve_of_any_row(n):
     ps.ps_interp_backward(p32.coef, n, torch.from_numpy(pos).to(DEV), torch.from_numpy(w).to(DEV),
                           None, gf)
     assert np.abs(gf.cpu().numpy() - gf_ref).max() <= 1e-5 * np.abs(gf_ref).max() + 1e-6
+
+
+@pytest.mark.parametrize("n", [(4, 4, 4), (16, 16, 15), (16, 16, 16), (17, 16, 16)])
+def test_offsets_of_few_and_many_bins(n):
+    # one-cell bins: 64, 3840 and 4096 are scanned by one block, 4352 in three phases
+    pos = synth.uniform_particles(30_000, seed=41)
+    bins = ps.bin_particles(n, 1, torch.from_numpy(pos).to(DEV))
+    np.testing.assert_array_equal(bins.offsets.cpu().numpy(),
+                                  oracle.bin_particles(n, (1, 1, 1), pos)[1])
