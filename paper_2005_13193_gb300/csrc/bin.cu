@@ -3,8 +3,10 @@
 // (Sec. 3) and of its per-step particle migration (Sec. 4.3).
 //
 // count:   bin of every particle; a warp-aggregated atomicAdd on the bin's
-//          counter returns the particle's rank inside its bin.
-// scan:    exclusive prefix sum of the counters -> bin_offsets (3 phases).
+//          counter returns the particle's rank inside its bin (few bins: first
+//          in shared memory, then one atomicAdd per block and bin).
+// scan:    exclusive prefix sum of the counters -> bin_offsets (3 phases, one
+//          block for few counters).
 // scatter: slot = bin_offsets[bin] + rank; writes perm / sorted copies.
 // The count may instead come from the kernel that wrote the positions (it
 // counts each particle's new bin as it stores it, without ranks); bin_run
@@ -75,6 +77,71 @@ __global__ void bin_count_kernel(GridArgs g, BrickArgs b, int64_t np,
         bin_of[p] = key;
         rank[p] = basev + within;
       }
+    }
+  }
+}
+
+// The count for few bins, where the particles' atomics on few counters wait
+// for one another: a block counts kFewThreads * kFewItems particles in shared
+// memory, then adds each of its bins to the global counter once.  A whole sort
+// of particles in random order, an atomic per run of particles / per block and
+// bin: 4 M in 64 bins 1012 / 82 us, 512 bins 575 / 88, 1000 bins 398 / 92;
+// 500 k 133 / 19, 79 / 20, 51 / 21.  With more bins or fewer particles it
+// still pays for random orders (4 M in 1728 bins 258 / 92 us), but positions
+// already in bin order, whose runs need few atomics, lose by the block's
+// barriers (58 / 65 us there, 50 k in 512 bins 12.6 / 14.6); below the limits
+// they do not (4 M in 512 bins 72 / 64, in 1000 bins 64 / 66).  512 threads of
+// 8 particles spilled and took 97 us at 512 bins.
+constexpr int kFewThreads = 1024, kFewItems = 4, kFewBins = 1024;
+constexpr int64_t kFewMinParticles = 1 << 17;
+__global__ void __launch_bounds__(kFewThreads)
+    bin_count_few(GridArgs g, BrickArgs b, int64_t np, const double* __restrict__ pos,
+                  int32_t* __restrict__ bin_of, int32_t* __restrict__ rank,
+                  int32_t* __restrict__ counts, int32_t* status) {
+  __shared__ int32_t cnt[kFewBins];
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, nbins = (int)b.nbins;
+  for (int i = threadIdx.x; i < nbins; i += kFewThreads) cnt[i] = 0;
+  const int64_t p0 = (int64_t)blockIdx.x * (kFewThreads * kFewItems) + threadIdx.x;
+  double x[kFewItems], y[kFewItems], z[kFewItems];
+#pragma unroll
+  for (int u = 0; u < kFewItems; ++u) {
+    const int64_t p = p0 + u * kFewThreads;
+    x[u] = y[u] = z[u] = 0.0;
+    if (p < np) {
+      x[u] = pos[p];
+      y[u] = pos[np + p];
+      z[u] = pos[2 * np + p];
+    }
+  }
+  __syncthreads();
+  int key[kFewItems], mine[kFewItems];
+#pragma unroll
+  for (int u = 0; u < kFewItems; ++u) {
+    const int64_t p = p0 + u * kFewThreads;
+    key[u] = -1 - lane;  // unique per lane when invalid
+    if (p < np) {
+      bool ok;
+      key[u] = bin_of_position(g, b, x[u], y[u], z[u], ok);
+      if (!ok) flag_status(status, PS_DEV_NONFINITE_POS, p);
+    }
+    int first, within, len, basev = 0;
+    run_ranks(key[u], lane, first, within, len);
+    if (p < np && lane == first) basev = atomicAdd(&cnt[key[u]], len);
+    mine[u] = __shfl_sync(FULL, basev, first) + within;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nbins; i += kFewThreads) {
+    const int32_t c = cnt[i];
+    if (c) cnt[i] = atomicAdd(&counts[i], c);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kFewItems; ++u) {
+    const int64_t p = p0 + u * kFewThreads;
+    if (p < np) {
+      bin_of[p] = key[u];
+      rank[p] = cnt[key[u]] + mine[u];
     }
   }
 }
@@ -233,7 +300,12 @@ ps_status bin_run(const GridArgs& ga, const BrickArgs& ba, int64_t np, const dou
       (rc = check_cuda(cudaMemsetAsync(counts, 0, sizeof(int32_t) * (ba.nbins + 1), st),
                        "bin counts memset")))
     return rc;
-  if (np > 0 && !counted) {
+  if (!counted && np >= kFewMinParticles && ba.nbins <= kFewBins) {
+    const int64_t per = kFewThreads * kFewItems;
+    bin_count_few<<<(unsigned)((np + per - 1) / per), kFewThreads, 0, st>>>(
+        ga, ba, np, pos, bin_of, rank, counts, status);
+    if ((rc = check_launch("bin_count_few"))) return rc;
+  } else if (np > 0 && !counted) {
     bin_count_kernel<<<persistent_blocks(np, 256), 256, 0, st>>>(ga, ba, np, pos, bin_of,
                                                                  rank, counts, status);
     if ((rc = check_launch("bin_count"))) return rc;

@@ -221,3 +221,22 @@ def test_offsets_of_few_and_many_bins(n):
     bins = ps.bin_particles(n, 1, torch.from_numpy(pos).to(DEV))
     np.testing.assert_array_equal(bins.offsets.cpu().numpy(),
                                   oracle.bin_particles(n, (1, 1, 1), pos)[1])
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (24, 16, 9), (64, 64, 128), (64, 72, 128)])
+@pytest.mark.parametrize("np_", [(1 << 17) - 1, 1 << 17, 135_001])
+def test_sort_of_many_particles_into_few_bins(n, np_):
+    # counted in shared memory from 2^17 particles on in up to 1024 bins (1152: not)
+    pos = synth.uniform_particles(np_, seed=43) * 1.4 - 0.8
+    pos[:, np_ - 1] = 0.0  # where the bin of a position that is not finite is, too
+    pg = torch.from_numpy(pos).to(DEV)
+    pg[1, np_ - 1] = math.nan
+    st = torch.zeros(4, dtype=torch.int32, device=DEV)
+    bins = ps.bin_particles(n, 8, pg, status=st)
+    assert ps.ps_status_read(st) == [ps._abi.PS_DEV_NONFINITE_POS, np_ - 1, 0, 1]
+    ref_bin, ref_off, _ = oracle.bin_particles(n, (8, 8, 8), pos)
+    np.testing.assert_array_equal(bins.bin_of.cpu().numpy(), ref_bin)
+    np.testing.assert_array_equal(bins.offsets.cpu().numpy(), ref_off)
+    perm = bins.perm.cpu().numpy()
+    np.testing.assert_array_equal(np.sort(perm), np.arange(np_))
+    np.testing.assert_array_equal(ref_bin[perm], np.sort(ref_bin))
