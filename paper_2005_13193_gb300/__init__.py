@@ -12,6 +12,7 @@ torch and call the same entry points.
 from __future__ import annotations
 
 import ctypes
+import functools
 import math
 from typing import Optional, Sequence
 
@@ -81,9 +82,7 @@ def _check(rc: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _nbytes(t: Optional[torch.Tensor]) -> int:
@@ -105,10 +104,24 @@ def _dev(t: Optional[torch.Tensor], name: str, dtype=None, numel=None):
 
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the current device's current stream, without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
+
+
+# The geometry arguments of a call as C structures, kept by value; the C side
+# only reads them.  Building them, and pointer and stream objects, was a
+# quarter of a small step's time (solve and Heun step of 4096 particles on 32^3:
+# 164 -> 119 us).
+@functools.lru_cache(maxsize=256)
+def _grid_of(n, L) -> PsGrid:
+    return make_grid(n, L)
+
+
+def _grid(n, L) -> PsGrid:
+    return _grid_of(tuple(int(v) for v in n), tuple(float(v) for v in L))
 
 
 def make_grid(n: Sequence[int], L: Sequence[float] = DEFAULT_L) -> PsGrid:
@@ -120,18 +133,28 @@ def make_grid(n: Sequence[int], L: Sequence[float] = DEFAULT_L) -> PsGrid:
     return g
 
 
+@functools.lru_cache(maxsize=256)
+def _brick_of(brick):
+    return (ctypes.c_int32 * 3)(*brick)
+
+
 def _brick_arr(brick):
     if brick is None:
         return None
     if isinstance(brick, int):
         brick = (brick, brick, brick)
-    return (ctypes.c_int32 * 3)(*[int(b) for b in brick])
+    return _brick_of(tuple(int(b) for b in brick))
+
+
+@functools.lru_cache(maxsize=1024)
+def _row_pitch(nx: int, code: int) -> int:
+    return int(_lib().ps_coef_row_pitch(nx, code))
 
 
 def coef_row_pitch(nx: int, dtype: torch.dtype) -> int:
     """Row pitch (elements) of a padded coefficient array: nx+3 rounded up to
     16 bytes (ps_coef_row_pitch)."""
-    return int(_lib().ps_coef_row_pitch(int(nx), _dt_code(dtype)))
+    return _row_pitch(int(nx), _dt_code(dtype))
 
 
 def coef_shape(n, ncomp: int, dtype):
@@ -202,7 +225,7 @@ def ps_status_read(status: torch.Tensor, stream=None, raise_on_error: bool = Fal
 
 def ps_spline_coeffs_workspace_size(n, ncomp: int, coef_dtype: torch.dtype,
                                     L=DEFAULT_L) -> int:
-    g = make_grid(n, L)
+    g = _grid(n, L)
     return int(_lib().ps_spline_coeffs_workspace_size(ctypes.byref(g), ncomp,
                                                        _dt_code(coef_dtype)))
 
@@ -219,7 +242,7 @@ def ps_spline_coeffs(field: torch.Tensor, coef: torch.Tensor, scale: Optional[to
     _dev(coef, "coef")
     _dev(scale, "scale", torch.float32)
     _dev(ws, "ws")
-    g = make_grid(n, L)
+    g = _grid(n, L)
     ws_bytes = ws.numel() * ws.element_size() if ws is not None else 0
     call = _lib().ps_spline_coeffs_rows3 if rows3 else _lib().ps_spline_coeffs
     _check(call(ctypes.byref(g), ncomp, _DT[field.dtype], _ptr(field), _coef_type(coef),
@@ -227,7 +250,7 @@ def ps_spline_coeffs(field: torch.Tensor, coef: torch.Tensor, scale: Optional[to
 
 
 def ps_bin_workspace_size(n, brick, np_: int, L=DEFAULT_L) -> int:
-    g = make_grid(n, L)
+    g = _grid(n, L)
     return int(_lib().ps_bin_workspace_size(ctypes.byref(g), _brick_arr(brick), int(np_)))
 
 
@@ -244,7 +267,7 @@ def ps_bin_particles(n, brick, pos: torch.Tensor, bin_of: torch.Tensor, bin_offs
     _dev(pos_sorted, "pos_sorted", torch.float64, 3 * np_)
     _dev(ws, "ws")
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     ws_bytes = ws.numel() * ws.element_size() if ws is not None else 0
     _check(_lib().ps_bin_particles(ctypes.byref(g), _brick_arr(brick), np_, _ptr(pos),
                                    _ptr(bin_of), _ptr(bin_offsets), _ptr(perm), _ptr(pos_sorted),
@@ -252,7 +275,7 @@ def ps_bin_particles(n, brick, pos: torch.Tensor, bin_of: torch.Tensor, bin_offs
 
 
 def ps_spline_truncated_workspace_size(n, ncomp: int, L=DEFAULT_L) -> int:
-    g = make_grid(n, L)
+    g = _grid(n, L)
     return int(_lib().ps_spline_truncated_workspace_size(ctypes.byref(g), ncomp))
 
 
@@ -269,7 +292,7 @@ def ps_spline_coeffs_truncated(field: torch.Tensor, coef: torch.Tensor, K: int =
     if ws is None:
         ws = workspace(ps_spline_truncated_workspace_size(n, ncomp, L), field.device)
     _dev(ws, "ws")
-    g = make_grid(n, L)
+    g = _grid(n, L)
     _check(_lib().ps_spline_coeffs_truncated(ctypes.byref(g), ncomp, _ptr(field), int(K),
                                              _ptr(coef), _ptr(ws), ws.numel() * ws.element_size(),
                                              _stream(stream)))
@@ -295,7 +318,7 @@ def ps_interp(coef: torch.Tensor, n, pos: torch.Tensor, vel: torch.Tensor,
     _dev(grad, "grad", torch.float32, ncomp * 3 * np_)
     _dev(status, "status", torch.int32, 4)
     _dev(ws, "ws")
-    g = make_grid(n, L)
+    g = _grid(n, L)
     _check(_lib().ps_interp_ws(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef), _ptr(scale),
                                np_, _ptr(pos), _ptr(perm), _ptr(bin_offsets), _brick_arr(brick),
                                _ptr(vel), _ptr(grad), _ptr(ws), _nbytes(ws), _ptr(status),
@@ -320,7 +343,7 @@ def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Te
     _dev(g_pos, "g_pos", torch.float64, 3 * np_)
     _dev(g_field, "g_field", torch.float32, ncomp * n[0] * n[1] * n[2])
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     if bin_offsets is not None:
         _dev(perm, "perm", torch.int64, np_)
         _dev(bin_offsets, "bin_offsets", torch.int32)
@@ -369,7 +392,7 @@ def ps_interp_hessian(coef: torch.Tensor, n, pos: torch.Tensor, hess: torch.Tens
     _dev(perm, "perm", torch.int64, np_)
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     _dev(ws, "ws")
     _check(_lib().ps_interp_hessian_ws(ctypes.byref(g), ncomp, _coef_type(coef), _ptr(coef),
                                        _ptr(scale), np_, _ptr(pos), _ptr(perm),
@@ -400,7 +423,7 @@ def ps_lagrangian_accel(coef_n: torch.Tensor, n, pos: torch.Tensor, acc: torch.T
     _dev(perm, "perm", torch.int64, np_)
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     _dev(ws, "ws")
     _check(_lib().ps_lagrangian_accel_ws(ctypes.byref(g), _coef_type(coef_n), _ptr(coef_n),
                                          _ptr(scale_n), _ptr(coef_np1), _ptr(scale_np1),
@@ -411,7 +434,7 @@ def ps_lagrangian_accel(coef_n: torch.Tensor, n, pos: torch.Tensor, acc: torch.T
 
 
 def ps_rk2_workspace_size(n, brick, np_: int, L=DEFAULT_L) -> int:
-    g = make_grid(n, L)
+    g = _grid(n, L)
     return int(_lib().ps_rk2_workspace_size(ctypes.byref(g), _brick_arr(brick), int(np_)))
 
 
@@ -438,7 +461,7 @@ def ps_rk2_step(coef_n: torch.Tensor, n, pos: torch.Tensor, dt: float,
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(ws, "ws")
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     ws_bytes = ws.numel() * ws.element_size() if ws is not None else 0
     if coef_np1 is not None and _coef_type(coef_np1) != _coef_type(coef_n):
         raise ValueError("coef_np1 must have the storage of coef_n")
@@ -464,7 +487,7 @@ def ps_rk2_sort(n, brick, pos: torch.Tensor, pos_sorted: torch.Tensor,
     _dev(bin_offsets, "bin_offsets", torch.int32)
     _dev(ws, "ws")
     _dev(status, "status", torch.int32, 4)
-    g = make_grid(n, L)
+    g = _grid(n, L)
     _check(_lib().ps_rk2_sort(ctypes.byref(g), _brick_arr(brick), np_, _ptr(pos), _ptr(ids),
                               1 if counted else 0, _ptr(pos_sorted), _ptr(ids_sorted),
                               _ptr(bin_offsets), _ptr(ws), ws.numel() * ws.element_size(),
