@@ -40,11 +40,11 @@ POS_SEED = 2001
 WORKLOAD = ("mid: 512^3 FP32 u,v,w (k^-5/3, 1<=|k|<=170, unit rms), 16,777,216 uniform FP64 "
             "particles; spline solve + 10 Heun RK2 steps (dt 1e-3) with re-binning into 8^3 "
             "bricks every step")
-# kernels of libps launched per bench step: 3 solve passes + 10 x (3 scan passes, 1 scatter
-# and the RK2 step, which also counts the next sort's bins)
-LAUNCHES_PER_STEP = 3 + RK_STEPS * 5
-DOMINANT = "interp_staged<float4,3,RK2> (fused binned Heun step, halo by tensor copy)"
-SOURCE_FOR_TRAFFIC = os.path.join(ROOT, "paper_2005_13193_gb300", "csrc", "interp.cu")
+# kernels of libps launched per bench step: 2 solve passes and 2 copies of the periodic images
+# + 10 x (3 scan passes, 1 scatter and the RK2 step, which also counts the next sort's bins)
+LAUNCHES_PER_STEP = 4 + RK_STEPS * 5
+DOMINANT = "quad_kernel<float4,RK2> (fused binned Heun step, halo by tensor copy)"
+SOURCE_FOR_TRAFFIC = os.path.join(ROOT, "paper_2005_13193_gb300", "csrc", "brick.cuh")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.txt")
 
 
@@ -72,16 +72,19 @@ def parse():
         NP = args.particles or NP
         RK_STEPS = args.rk_steps or RK_STEPS
         KMAX = N // 3
-        LAUNCHES_PER_STEP = 3 + RK_STEPS * 5
+        # (one scan kernel for up to 4096 bricks)
+        scans = 1 if (-(-N // BRICK[0])) ** 3 <= 4096 else 3
+        LAUNCHES_PER_STEP = 4 + RK_STEPS * (scans + 2)
         WORKLOAD = (f"reduced case: {N}^3 FP32 u,v,w (k^-5/3, 1<=|k|<={KMAX}), {NP} particles, "
                     f"solve + {RK_STEPS} RK2 steps, 8^3 bricks")
     return args
 
 
-# Shared-memory wavefronts (128 B) per particle of the binned Heun step: two
-# 64-point float4 gathers (16) plus the particle records, as counted by ncu
-# (l1tex__data_pipe_lsu_wavefronts_mem_shared_op_{ld,st}) for the node form.
-SMEM_WAVEFRONTS = 24.5
+# Shared-memory wavefronts (128 B) per particle of the binned Heun step: the
+# 64-point float4 gathers (8, and 8 more where the predictor leaves its cell),
+# the shuffles and the particle records, as counted by ncu
+# (l1tex__data_pipe_lsu_wavefronts_mem_shared) for the node form.
+SMEM_WAVEFRONTS = 14.8
 
 
 def smem_bound_ms(np_: int, sms: int = 152, clock_ghz: float = 2.07) -> float:

@@ -7,7 +7,8 @@ per particle but hold fewer blocks per SM; the best shape depends on the grid,
 the particle density and the coefficient type, so it is measured, on the
 caller's own data, by timing the real step for each candidate.
 
-`tune_tracker` picks (brick kernel, brick shape) for single-field Heun steps
+`tune_tracker` picks (brick kernel, brick shape; for three components the
+kernels 0 and 5 are the same) for single-field Heun steps
 and applies the kernel choice with ps_tune_set; `tune_batch` picks the brick
 shape of a many-field plan.  Both can write the choice to a small text cache,
 one "key values" pair per line, which ps_batch_plan reads back ("brick bx by

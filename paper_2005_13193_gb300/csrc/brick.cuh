@@ -1,5 +1,5 @@
 // One brick of particles by the warps of a block, each on its own: the body of
-// the single-field kernels (quad.cu).
+// the single-field kernels (quad.cu) and of the many-field ones (batch_step.cu).
 //
 // The brick's coefficient halo (the union of the stencils of its cells,
 // (B+3)^3 nodes) is brought into shared memory by one tensor copy (nodes,

@@ -8,10 +8,11 @@
 //    any particle order (the "unsorted" path).
 //  * staged: particles stored in brick order (Sec. 3's dynamic mapping read as
 //    a bin sort); one CTA per brick copies the brick's coefficient halo once
-//    into shared memory as float4 (u, v, w, 0), and 8 lanes per particle read
-//    it with conflict-free 128-bit loads.  This is the GPU form
-//    of the paper's "fetch only the coefficients a particle needs": the halo
-//    is the union of the stencils of the brick's particles.
+//    into shared memory.  This is the GPU form of the paper's "fetch only the
+//    coefficients a particle needs": the halo is the union of the stencils of
+//    the brick's particles.  Three components: brick.cuh and quad.cu.  Here:
+//    one component, as float4 in shared memory and 8 lanes per particle, and
+//    the thread-per-particle form of both.
 //
 // FP64 work per particle is one multiply per axis (done by three lanes in
 // parallel); floor and fraction come from the bits of the product, the RK2
