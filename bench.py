@@ -589,7 +589,7 @@ def batch_extras(ps, torch, dev):
     pos = pos0.clone()
     ids = torch.arange(plan.np_total, dtype=torch.int64, device=dev)
     # the 48 solves and the 20 steps in one graph: the steps as one cooperative
-    # persistent launch (default), and as a launch per phase and step
+    # persistent launch, and as a launch per phase and step (default)
     timings = {}
     old = ps.ps_tune_get("batch_persistent")
     try:
@@ -599,13 +599,13 @@ def batch_extras(ps, torch, dev):
             timings[name] = _event_ms(torch, lambda: plan.run(flds, pos, nsteps, dt, solve=True,
                                                               ids=ids, use_graph=True), 3,
                                       warmup=1)
-        ps.ps_tune_set("batch_persistent", 1)
+        ps.ps_tune_set("batch_persistent", 0)
         plan.run(flds, pos, nsteps, dt, solve=False, ids=ids, use_graph=True)
         t_steps = _event_ms(torch, lambda: plan.run(flds, pos, nsteps, dt, solve=False, ids=ids,
                                                     use_graph=True), 3, warmup=1)
     finally:
         ps.ps_tune_set("batch_persistent", old)
-    t_graph = timings["persistent"]
+    t_graph = timings["launch_per_step"]
     trackers = []
     for f, (n, v) in enumerate(zip(sizes, nps)):
         b = plan.base[f]
@@ -624,8 +624,8 @@ def batch_extras(ps, torch, dev):
             "autotune_ms_per_step": {"x".join(map(str, k)): v for k, v in table.items()},
             "graph": "48 solves + 20 Heun steps",
             "batched_graph_ms": t_graph, "batched_particles_per_s": units / (t_graph * 1e-3),
-            "launch_per_step_graph_ms": timings["launch_per_step"],
-            "steps_only_persistent_ms": t_steps,
+            "persistent_graph_ms": timings["persistent"],
+            "steps_only_ms": t_steps,
             "steps_only_particles_per_s": units / (t_steps * 1e-3),
             "per_field_loop_ms": t_loop, "loop_particles_per_s": units / (t_loop * 1e-3),
             "loop_note": "per-field Tracker steps without the solves"}

@@ -139,8 +139,9 @@ int64_t ps_coef_row_pitch(int nx, ps_dtype coef_t);
  *  "batch_run_below" in [0, 2^20] (default 16): ps_batch_plan bins a field
  *     whose bricks would hold fewer particles on average in runs of about
  *     128 neighbouring particles (stencils from global memory), not bricks.
- *  "batch_persistent" 0 or 1 (default 1): ps_batch_run runs all steps in one
- *     cooperative persistent launch (1) or a launch per phase and step (0).
+ *  "batch_persistent" 0 or 1 (default 0): ps_batch_run runs all steps in one
+ *     cooperative persistent launch (1) or a launch per phase and step (0; a
+ *     graph of more than 1024 steps holds the one launch instead).
  *  "wait_probe" in [0, 2^30] (default 0), a test knob: > 0 makes every
  *     staged brick wait, after its halo copy has landed, on a barrier that
  *     nothing completes, for that many clocks; the wait gives up, the status
@@ -466,9 +467,9 @@ ps_status ps_rk2_sort(const ps_grid* grid, const int32_t brick[3], int64_t np,
 /* bin sort over all particles (global bin = first bin of the field + bin   */
 /* in the field) and one pass over the bricks of all fields, which counts  */
 /* the next step's bins as it writes the positions (the first step counts   */
-/* from the positions), all steps in one cooperative persistent launch      */
-/* whose phases meet at grid-wide barriers (tune "batch_persistent" 0: a    */
-/* launch per phase and step).  A                                           */
+/* from the positions), in a launch per phase and step, or (tune            */
+/* "batch_persistent" 1, graphs of more than 1024 steps) all steps in one   */
+/* cooperative launch whose phases meet at grid-wide barriers.  A           */
 /* barrier wait that runs out (about 2^31 clocks) stops every block and     */
 /* sets PS_DEV_TIMEOUT in *status; positions are then unspecified.          */
 /* Particles end in bin order per field, as with ps_rk2_step(rebin=1); ids  */

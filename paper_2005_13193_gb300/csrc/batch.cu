@@ -295,6 +295,17 @@ ps_status enqueue_step(ps_plan* p, double* pos, int64_t* ids, void* ws, int32_t*
 
 }  // namespace
 
+// A launch per phase and step, or all steps in one cooperative launch.  The
+// grid-wide barriers of the one launch take about 17 us each, five a step, and
+// its streaming phases run with the brick kernel's 16 warps an SM, so separate
+// launches were faster at every size measured, replayed from a graph or not.
+// Four steps, one launch -> a launch per phase, us: 3 fields of 64^3 with 10 k
+// particles 326 -> 116 (without a graph 344 -> 157), 3 M 2456 -> 1601; 48 fields
+// of 64^3, 100 k 586 -> 291, 3 M 1920 -> 1487; 16 fields of 64^3 to 256^3, 1 M
+// 1346 -> 1130, 3 M 2418 -> 1959; nodes alike.  A graph of very many steps would
+// hold some seven nodes for each: past kGraphSteps it takes the one launch.
+constexpr int kGraphSteps = 1024;
+
 extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int solve,
                                   double* pos, int64_t* ids, float* vel_out, int nsteps,
                                   double dt, int use_graph, void* ws, size_t ws_bytes,
@@ -313,7 +324,7 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
   }
   cudaStream_t st = as_stream(stream);
   ps_status rc;
-  const bool persistent = tuning().batch_persistent != 0;
+  const bool persistent = tuning().batch_persistent != 0 || (use_graph && nsteps > kGraphSteps);
   // the solves of all fields (into the workspace's quantisation area when the
   // storage needs an intermediate)
   auto enqueue_solves = [&](cudaStream_t s) -> ps_status {
@@ -342,6 +353,10 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
     if (!steps) return PS_OK;
     if ((rc = build_tables(p, fields, pos, ids, vel_out, dt, ws, status))) return rc;
     if ((rc = upload_tables(p, ws, st))) return rc;
+    if (!persistent &&
+        (rc = staged_batch_launch(p->coef_t, cube(p), nullptr, nullptr, nullptr, nullptr, 0, 0,
+                                  p->smem, true, st)))
+      return rc;
     return enqueue_steps(st);
   }
   if (!solve && !steps) return PS_OK;

@@ -82,7 +82,7 @@ struct Tuning {
   int wait_probe = 0;         // test knob: clocks of a wait that cannot complete
   int batch_run_below = 16;   // batched fields with fewer particles per brick on
                               // average are binned in runs, not bricks
-  int batch_persistent = 1;   // batched steps: one cooperative launch (1) or a launch
+  int batch_persistent = 0;   // batched steps: one cooperative launch (1) or a launch
                               // per phase and step (0)
 };
 Tuning& tuning();

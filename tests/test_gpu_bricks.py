@@ -240,3 +240,49 @@ def test_sort_of_many_particles_into_few_bins(n, np_):
     perm = bins.perm.cpu().numpy()
     np.testing.assert_array_equal(np.sort(perm), np.arange(np_))
     np.testing.assert_array_equal(ref_bin[perm], np.sort(ref_bin))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, ps.F32X4, ps.F16X4])
+@pytest.mark.parametrize("brick", [(8, 8, 8), (16, 16, 8)])
+def test_batch_launch_per_step_equals_one_launch(dtype, brick):
+    # the default (a launch per phase and step; bricks whose halo needs more than
+    # 48 KB too) against all steps in one launch, which a graph of more than 1024
+    # steps takes by itself
+    sizes, nps = [32, 48, 24], [3000, 9000, 700]
+    assert ps.ps_tune_get("batch_persistent") == 0
+    flds = [(None, ps.SplineField.from_field(
+        torch.from_numpy(synth.random_field((e,) * 3, ncomp=3, seed=50 + e).astype(np.float32))
+        .to(DEV), dtype)) for e in sizes]
+    pos0 = torch.from_numpy(synth.uniform_particles(sum(nps), seed=51)).to(DEV)
+    for nsteps, forms in ((3, ((0, False), (0, True), (1, False))), (1025, ((0, True), (1, True)))):
+        out = []
+        for persistent, use_graph in forms:
+            ps.ps_tune_set("batch_persistent", persistent)
+            try:
+                plan = ps.BatchPlan([(e,) * 3 for e in sizes], nps, coef_dtype=dtype, brick=brick)
+                pos, ids = pos0.clone(), torch.arange(sum(nps), device=DEV)
+                st = torch.zeros(4, dtype=torch.int32, device=DEV)
+                plan.run(flds, pos, nsteps, 1e-4, solve=False, ids=ids, use_graph=use_graph,
+                         status=st)
+                assert ps.ps_status_read(st)[0] == 0
+            finally:
+                ps.ps_tune_set("batch_persistent", 0)
+            out.append(torch.empty_like(pos).index_copy_(1, ids, pos))
+        assert all(torch.equal(o, out[0]) for o in out[1:])
+
+
+def test_one_launch_barrier_wait_gives_up():
+    # as wait_probe does in the staged bricks: after the first grid barrier every
+    # block waits on a word that nothing sets, gives up and leaves
+    sf = ps.SplineField.from_field(torch.randn((3, 24, 24, 24), device=DEV))
+    pos = torch.from_numpy(synth.uniform_particles(5000, seed=53)).to(DEV)
+    plan = ps.BatchPlan([(24, 24, 24)], [5000])
+    st = torch.zeros(4, dtype=torch.int32, device=DEV)
+    ps.ps_tune_set("batch_persistent", 1)
+    ps.ps_tune_set("wait_probe", 20000)
+    try:
+        plan.run([(None, sf)], pos, 3, 1e-3, solve=False, use_graph=False, status=st)
+        assert ps.ps_status_read(st)[0] == ps._abi.PS_DEV_TIMEOUT
+    finally:
+        ps.ps_tune_set("wait_probe", 0)
+        ps.ps_tune_set("batch_persistent", 0)
