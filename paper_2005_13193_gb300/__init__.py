@@ -505,8 +505,8 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 
 # Result rows from this size on go through bin order (see ps_interp_ws): beyond a good
 # half of the L2, scattered 4-byte stores reach DRAM one by one.  Stored directly / by
-# way of bin order, us: 34 MiB 86 / 133, 46 MiB 386 / 392, 69 MiB 159 / 247,
-# 92 MiB 594 / 390 and 1011 / 742, 183 MiB 1668 / 741, 549 MiB 5697 / 1934.
+# way of bin order, us: 34 MiB 86 / 112, 46 MiB 384 / 390, 69 MiB 160 / 191,
+# 92 MiB 594 / 310 and 1011 / 740, 183 MiB 1668 / 582, 549 MiB 5695 / 1490.
 _UNSORT_BYTES = 80 << 20
 
 

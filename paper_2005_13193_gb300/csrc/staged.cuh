@@ -94,7 +94,7 @@ ps_status with_quad_type(ps_dtype t, F&& f) {
 }
 // Rows in bin order -> rows in the particles' order (unsort.cu): n0 rows to
 // d0, the next n1 to d1.
-ps_status unsort_launch(int64_t np, const int64_t* perm, const float* src, float* d0, int n0,
+ps_status unsort_launch(int64_t np, const int64_t* perm, float* src, float* d0, int n0,
                         float* d1, int n1, cudaStream_t st);
 
 // The scatter of a binned cotangent onto a cleared field (adjoint.cu).
