@@ -36,10 +36,12 @@ struct ps_plan {
          off_sync = 0, ws_bytes = 0;
   std::vector<unsigned char> h_args;
   std::vector<BinField> h_bintab;
-  // captured step sequence and what it was captured for
+  // captured step sequence, what it was captured for, and whether the tables in
+  // the workspace are still the ones it was captured with
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
   std::vector<uintptr_t> key;
+  bool graph_tables = false;
 };
 
 namespace {
@@ -351,6 +353,7 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
   if (!use_graph) {
     if (solve && (rc = enqueue_solves(st))) return rc;
     if (!steps) return PS_OK;
+    p->graph_tables = false;
     if ((rc = build_tables(p, fields, pos, ids, vel_out, dt, ws, status))) return rc;
     if ((rc = upload_tables(p, ws, st))) return rc;
     if (!persistent &&
@@ -372,7 +375,24 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
     key.push_back((uintptr_t)fields[f].scale);
     key.push_back((uintptr_t)(solve ? fields[f].field : nullptr));
   }
-  if (p->exec && key == p->key) return check_cuda(cudaGraphLaunch(p->exec, st), "graph launch");
+  // the launches captured the tuning values too
+  static_assert(sizeof(Tuning) % sizeof(int) == 0, "Tuning holds ints only");
+  int tune[sizeof(Tuning) / sizeof(int)];
+  memcpy(tune, &tuning(), sizeof(tune));
+  for (int v : tune) key.push_back((uintptr_t)v);
+  if (p->exec && key == p->key) {
+    // the one launch, and a launch per step over more fields than go by value,
+    // read the per-field table from the workspace, where a run without the
+    // graph has put its own since
+    const bool reads_table = persistent || p->nfields > kBatchParamFields;
+    if (steps && reads_table && !p->graph_tables) {
+      if ((rc = build_tables(p, fields, pos, ids, vel_out, dt, ws, status))) return rc;
+      if ((rc = upload_tables(p, ws, st))) return rc;
+      p->graph_tables = true;
+    }
+    return check_cuda(cudaGraphLaunch(p->exec, st), "graph launch");
+  }
+  p->graph_tables = false;
   if (steps) {
     if ((rc = build_tables(p, fields, pos, ids, vel_out, dt, ws, status))) return rc;
     if ((rc = upload_tables(p, ws, st))) return rc;
@@ -403,6 +423,7 @@ extern "C" ps_status ps_batch_run(ps_plan* p, const ps_batch_field* fields, int 
   cudaGraphDestroy(graph);
   if (rc) return rc;
   p->key = key;
+  p->graph_tables = true;
   return check_cuda(cudaGraphLaunch(p->exec, st), "graph launch");
 }
 

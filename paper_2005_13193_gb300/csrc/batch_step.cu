@@ -81,15 +81,15 @@ __global__ void __launch_bounds__(kThreads, 8)
   batch_brick<Tc, CT>(tab, bin_base, nfields, blockIdx.x, smem_b128, sa, cur);
 }
 
-constexpr int kParamFields = 48;  // 48 x 640 bytes of arguments: within the 32 KB of parameters
+// (48 x 640 bytes of arguments: within the 32 KB of parameters)
 struct BatchParams {
-  StagedArgs a[kParamFields];
-  int bin_base[kParamFields + 1];
+  StagedArgs a[kBatchParamFields];
+  int bin_base[kBatchParamFields + 1];
   int nfields;
 };
 static_assert(sizeof(BatchParams) <= 32764, "kernel parameters are limited to 32764 bytes");
 
-// A batch of at most kParamFields fields passes its argument table as one
+// A batch of at most kBatchParamFields fields passes its argument table as one
 // kernel parameter: the brick body then reads each field's arguments from the
 // constant bank, as the single-field kernel does, and the tensor maps are named
 // in parameter space like the single-field kernel's.
@@ -325,7 +325,7 @@ ps_status staged_batch_launch(ps_dtype coef_t, bool cube, const void* d_tab, con
         return rc;
       }
       if (total_bins <= 0) return PS_OK;
-      if (h_tab && h_bin_base && nfields <= kParamFields) {
+      if (h_tab && h_bin_base && nfields <= kBatchParamFields) {
         // the table by value (a graph captures it with the launch)
         BatchParams tab;
         memcpy(tab.a, h_tab, (size_t)nfields * sizeof(StagedArgs));

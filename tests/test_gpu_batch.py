@@ -240,3 +240,57 @@ def test_autotune_tracker_and_batch(tmp_path):
         plan.run(fields, p, 3, 2e-3, solve=False, ids=ids, use_graph=False)
         outs.append(_by_label(p.cpu().numpy(), ids.cpu().numpy()))
     np.testing.assert_array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("nfields,persistent", [(3, 0), (49, 0), (3, 1)])
+def test_graph_replay_after_a_run_without_it(nfields, persistent):
+    # graph(A), a run without the graph on other positions with another dt, and
+    # graph(A) again on the same plan: the replay takes A's arguments, whether
+    # its steps hold the per-field table by value or read it from the workspace
+    sizes, nps = [(16, 20, 24)[f % 3] for f in range(nfields)], [300 + 11 * f for f in
+                                                                 range(nfields)]
+    flds = _fields(sizes, 1000)
+    pos0 = torch.from_numpy(_positions(nps, 1100)).to(DEV)
+    grids = [(n,) * 3 for n in sizes]
+    old = ps.ps_tune_get("batch_persistent")
+
+    def run(plan, pos, dt, use_graph):
+        ids = ids_of[id(pos)]
+        ids.copy_(torch.arange(plan.np_total, device=DEV))
+        pos.copy_(pos0)
+        plan.run(flds, pos, 2, dt, solve=False, ids=ids, use_graph=use_graph)
+        return torch.empty_like(pos).index_copy_(1, ids, pos)
+
+    try:
+        ps.ps_tune_set("batch_persistent", persistent)
+        plan = ps.BatchPlan(grids, nps)
+        a, b = torch.empty_like(pos0), torch.empty_like(pos0)
+        ids_of = {id(t): torch.empty(plan.np_total, dtype=torch.int64, device=DEV) for t in (a, b)}
+        first = run(plan, a, 4e-3, True)
+        other = run(plan, b, 8e-3, False)
+        kept = b.clone()
+        again = run(plan, a, 4e-3, True)
+        assert not torch.equal(first, other)
+        assert torch.equal(again, first) and torch.equal(b, kept)
+        assert torch.equal(run(plan, a, 4e-3, True), first)
+    finally:
+        ps.ps_tune_set("batch_persistent", old)
+
+
+def test_graph_follows_the_tuning_values():
+    # what a captured launch was given (here the test knob of the bounded wait)
+    # is captured anew after ps_tune_set
+    sizes, nps = [16, 32], [3000, 20000]
+    flds = _fields(sizes, 1200)
+    pos = torch.from_numpy(_positions(nps, 1300)).to(DEV)
+    plan = ps.BatchPlan([(n,) * 3 for n in sizes], nps)
+    st = torch.zeros(4, dtype=torch.int32, device=DEV)
+    old = ps.ps_tune_get("wait_probe")
+    try:
+        for probe, code in ((0, 0), (20000, ps._abi.PS_DEV_TIMEOUT), (0, 0)):
+            ps.ps_tune_set("wait_probe", probe)
+            st.zero_()
+            plan.run(flds, pos, 1, 1e-3, solve=False, use_graph=True, status=st)
+            assert ps.ps_status_read(st)[0] == code
+    finally:
+        ps.ps_tune_set("wait_probe", old)
