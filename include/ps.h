@@ -470,8 +470,9 @@ ps_status ps_rk2_sort(const ps_grid* grid, const int32_t brick[3], int64_t np,
 /* from the positions), in a launch per phase and step, or (tune            */
 /* "batch_persistent" 1, graphs of more than 1024 steps) all steps in one   */
 /* cooperative launch whose phases meet at grid-wide barriers.  A           */
-/* barrier wait that runs out (about 2^31 clocks) stops every block and     */
-/* sets PS_DEV_TIMEOUT in *status; positions are then unspecified.          */
+/* barrier wait that runs out (about 2^31 clocks), or a halo copy that has  */
+/* not landed after twice that, stops every block and sets PS_DEV_TIMEOUT   */
+/* in *status; positions are then unspecified.                              */
 /* Particles end in bin order per field, as with ps_rk2_step(rebin=1); ids  */
 /* (optional, int64 [np_total]) and vel_out (optional, [3][np_total] = u at */
 /* the start of the last step) follow them.  use_graph = 1 captures the     */

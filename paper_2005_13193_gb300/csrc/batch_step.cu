@@ -17,12 +17,13 @@ namespace {
 constexpr int kThreads = 64;  // per block, as the single-field kernel
 
 // The brick (or run of particles) `b` of one field by the block.
-template <typename Tc, int CT>
-__device__ __forceinline__ void field_brick(const StagedArgs& a, int b, unsigned char* smem,
-                                            const StagedArgs* maps) {
+template <typename Tc, int CT, bool ONCE = true>
+__device__ __forceinline__ bool field_brick(const StagedArgs& a, int b, unsigned char* smem,
+                                            const StagedArgs* maps, CopyBarriers& mb,
+                                            unsigned& phase) {
   const int nbx = a.b.nb[0], nby = a.b.nb[1];
   const int z = b / (nbx * nby), rem = b - z * nbx * nby, y = rem / nbx, x = rem - y * nbx;
-  warp_brick<Tc, 2, CT>(a, b, x, y, z, smem, maps);
+  return warp_brick<Tc, 2, CT, ONCE>(a, b, x, y, z, smem, maps, mb, phase);
 }
 
 // The field of global brick b: the last f with bin_base[f] <= b.
@@ -39,14 +40,15 @@ __device__ __forceinline__ int field_of(const int* __restrict__ bin_base, int nf
 // Global brick b of a many-field batch: the field's arguments are copied to
 // shared memory (sa; `cur` the field it holds), its tensor maps stay in the
 // global table.  Empty bins return at once.  Every thread of the block calls,
-// between block barriers.
-template <typename Tc, int CT>
-__device__ __forceinline__ void batch_brick(const StagedArgs* __restrict__ tab,
+// between block barriers.  Returns what warp_brick does.
+template <typename Tc, int CT, bool ONCE = true>
+__device__ __forceinline__ bool batch_brick(const StagedArgs* __restrict__ tab,
                                             const int* __restrict__ bin_base, int nfields,
-                                            int b, unsigned char* smem, StagedArgs& sa, int& cur) {
+                                            int b, unsigned char* smem, StagedArgs& sa, int& cur,
+                                            CopyBarriers& mb, unsigned& phase) {
   // field 0's offsets are the global offsets: empty bins leave at once
   const int32_t* goffs = tab[0].offs;
-  if (goffs[b] >= goffs[b + 1]) return;
+  if (goffs[b] >= goffs[b + 1]) return true;
   const int f = field_of(bin_base, nfields, b);
   if (f != cur) {
     cur = f;
@@ -67,7 +69,7 @@ __device__ __forceinline__ void batch_brick(const StagedArgs* __restrict__ tab,
     }
     __syncthreads();
   }
-  field_brick<Tc, CT>(sa, b - bin_base[f], smem, tab + f);
+  return field_brick<Tc, CT, ONCE>(sa, b - bin_base[f], smem, tab + f, mb, phase);
 }
 
 // Many fields in one launch: block b handles global brick b.
@@ -77,8 +79,10 @@ __global__ void __launch_bounds__(kThreads, 8)
                      int nfields) {
   extern __shared__ __align__(128) unsigned char smem_b128[];
   __shared__ StagedArgs sa;
+  __shared__ CopyBarriers mb;
   int cur = -1;
-  batch_brick<Tc, CT>(tab, bin_base, nfields, blockIdx.x, smem_b128, sa, cur);
+  unsigned phase = 0;
+  batch_brick<Tc, CT>(tab, bin_base, nfields, blockIdx.x, smem_b128, sa, cur, mb, phase);
 }
 
 // (48 x 640 bytes of arguments: within the 32 KB of parameters)
@@ -97,12 +101,14 @@ template <typename Tc, int CT>
 __global__ void __launch_bounds__(kThreads, 8)
     batch_param_step(const __grid_constant__ BatchParams tab) {
   extern __shared__ __align__(128) unsigned char smem_bp128[];
+  __shared__ CopyBarriers mb;
+  unsigned phase = 0;
   const int b = blockIdx.x;
   // field 0's offsets are the global offsets: empty bins leave at once
   const int32_t* goffs = tab.a[0].offs;
   if (goffs[b] >= goffs[b + 1]) return;
   const int f = field_of(tab.bin_base, tab.nfields, b);
-  field_brick<Tc, CT>(tab.a[f], b - tab.bin_base[f], smem_bp128, &tab.a[f]);
+  field_brick<Tc, CT>(tab.a[f], b - tab.bin_base[f], smem_bp128, &tab.a[f], mb, phase);
 }
 
 // ----------------------------------------------------- persistent batch ----
@@ -190,6 +196,13 @@ __global__ void __launch_bounds__(kThreads, 8) batch_persistent(const __grid_con
   __shared__ StagedArgs sa;
   __shared__ int32_t scan_sh[kThreads / 32];
   __shared__ unsigned claim[2];
+  __shared__ CopyBarriers mb;
+  __shared__ int lost;  // 1: a halo copy of this block did not land
+  unsigned phase = 0;
+  if (threadIdx.x == 0) {
+    init_copy_barriers(mb);
+    lost = 0;
+  }  // (published by the first grid barrier)
   int nbar = 0, cur = -1;  // cur: the field whose arguments sa holds
   const int lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,9 +245,15 @@ __global__ void __launch_bounds__(kThreads, 8) batch_persistent(const __grid_con
       if (threadIdx.x == 0) claim[it] = c;
       __syncthreads();  // the claim; and the last brick is done with sa and the shared memory
       const unsigned b = claim[it];
+      if (lost) {  // the copy may yet write to the halo: the run ends here
+        if (threadIdx.x == 0) atomicExch(&r.sync[2], 1u);
+        break;
+      }
       if (b >= r.total_bins) break;
       if (threadIdx.x == 0) c = atomicAdd(&r.sync[4], 1u);
-      batch_brick<Tc, CT>(r.tab, r.bin_base, r.nfields, (int)b, smem_bp, sa, cur);
+      if (!batch_brick<Tc, CT, false>(r.tab, r.bin_base, r.nfields, (int)b, smem_bp, sa, cur, mb,
+                                      phase))
+        lost = 1;  // (after the brick's block barrier, so behind every thread's read above)
     }
     if (!grid_barrier(r, nbar)) return;
   }

@@ -389,11 +389,28 @@ template <> struct WPack<0> {
   static __device__ __forceinline__ int l2(int w) { return (w >> 15) & 1023; }
 };
 
-template <typename Tc, int MODE, int CT>
-__device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi, int byi,
-                                           int bzi, unsigned char* smem, const StagedArgs* maps) {
+// The mbarriers of a block's halo copies: the halo, a second field's halo, the
+// test knob's (which nothing completes).  A block that takes one brick
+// initialises them in warp_brick (ONCE); one that takes brick after brick
+// initialises them once, by one thread, with a block barrier before the first
+// brick, and each copy completes the next phase, whose parity every thread
+// keeps in `phase` (bit i: barrier i).
+struct CopyBarriers {
+  unsigned long long b[3];
+};
+__device__ __forceinline__ void init_copy_barriers(CopyBarriers& mb) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) tma_init_barrier(&mb.b[i]);
+}
+
+// Returns whether this thread saw every copy of the brick land (false: the
+// block's shared memory must not be used again).
+template <typename Tc, int MODE, int CT, bool ONCE = true>
+__device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi, int byi,
+                                           int bzi, unsigned char* smem, const StagedArgs* maps,
+                                           CopyBarriers& mb, unsigned& phase) {
   const int beg = a.offs[bin], end = a.offs[bin + 1];
-  if (beg >= end) return;
+  if (beg >= end) return true;
   const QGeo<CT> geo(a);
   const GridArgs& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -422,7 +439,8 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
   const int hbytes = halo_bytes<Tc>(geo.Sz, geo.Sy, geo.PS);
   unsigned char* halo = smem;
   unsigned char* halo2 = smem + hbytes;
-  __shared__ __align__(8) unsigned long long mbar[3];
+  unsigned long long* mbar = mb.b;
+  const unsigned par = ONCE ? 0 : phase & 1, par2 = ONCE ? 0 : phase >> 1 & 1;
   __shared__ unsigned char slot_lane[4][32];
 
   // use1, use2: the halos of coef and coef2 hold the brick's nodes
@@ -432,8 +450,12 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
   const bool tma2 = tma && use2 && a.tma == 2;
   if (use1) {
     if (tid == 0 && tma) {
-      if (a.wait_probe > 0) tma_init_barrier(&mbar[2]);
-      tma_init_barrier(&mbar[0]);
+      if (ONCE) {
+        if (a.wait_probe > 0) tma_init_barrier(&mbar[2]);
+        tma_init_barrier(&mbar[0]);
+      } else {  // the last brick's accesses to the halo before this one's copy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
       if constexpr (IsNode16<Tc>::value) {
         // the nodes and the rows' scales, both on one barrier
         tma_copy_node16(&maps->tmap, &maps->tmap2, halo,
@@ -444,7 +466,7 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
             (unsigned)((IsPlanar<Tc>::value ? 12 : 16) * geo.SX * geo.Sy * geo.Sz);
         tma_copy<IsPlanar<Tc>::value>(&maps->tmap, halo, &mbar[0], P0, bytes);
         if (tma2) {
-          tma_init_barrier(&mbar[1]);
+          if (ONCE) tma_init_barrier(&mbar[1]);
           tma_copy<IsPlanar<Tc>::value>(&maps->tmap2, halo2, &mbar[1], P0, bytes);
         }
       }
@@ -531,11 +553,11 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
       // a copy that does not complete in time is reported and the particles
       // read global memory
       waited = true;
-      landed = tma_wait(&mbar[0], 0);
+      landed = tma_wait(&mbar[0], par);
       bool done = landed;
       if (done && a.wait_probe > 0) done = tma_wait(&mbar[2], 0, a.wait_probe);
       if (tma2) {
-        landed2 = tma_wait(&mbar[1], 0);
+        landed2 = tma_wait(&mbar[1], par2);
         done = done && landed2;
       }
       if (!__all_sync(FULL, done)) {
@@ -732,8 +754,10 @@ __device__ __forceinline__ void warp_brick(const StagedArgs& a, int bin, int bxi
   }
   if (MODE == 2 && a.next_counts && lane == 0 && stays) atomicAdd(&a.next_counts[bin], stays);
   // a copy still in flight must land before the block's memory is released
-  if (tma && !(waited && landed)) tma_wait(&mbar[0], 0);
-  if (tma2 && !(waited && landed2)) tma_wait(&mbar[1], 0);
+  if (tma && !(waited && landed)) landed = tma_wait(&mbar[0], par);
+  if (tma2 && !(waited && landed2)) landed2 = tma_wait(&mbar[1], par2);
+  if (!ONCE) phase ^= (tma ? 1u : 0u) | (tma2 ? 2u : 0u);
+  return landed && landed2;
 }
 
 }  // namespace

@@ -41,8 +41,11 @@ template <typename Tc, int MODE, int CT>
 __global__ void __launch_bounds__(kMaxThreads, 4)
     quad_kernel(const __grid_constant__ StagedArgs a) {
   extern __shared__ __align__(128) unsigned char smem_q[];
+  __shared__ CopyBarriers mb;
+  unsigned phase = 0;
   const int bin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  warp_brick<Tc, MODE, CT>(a, bin, blockIdx.x, blockIdx.y, blockIdx.z, smem_q, &a);
+  warp_brick<Tc, MODE, CT>(a, bin, blockIdx.x, blockIdx.y, blockIdx.z, smem_q, &a, mb,
+                           phase);
 }
 
 // Row length SX >= S[0] of a halo.  float4 nodes: SX even with SX * S[1] = 2 or

@@ -294,3 +294,32 @@ def test_graph_follows_the_tuning_values():
             assert ps.ps_status_read(st)[0] == code
     finally:
         ps.ps_tune_set("wait_probe", old)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, ps.F32X4, ps.F16X4])
+@pytest.mark.parametrize("per_brick", [9, 30])
+def test_one_launch_over_many_bricks_per_block(dtype, per_brick):
+    # more bricks than the device holds blocks, so that every block takes several
+    # (each halo copy completing the next phase of its barrier), of which at 9
+    # particles on average some are staged and some read global memory
+    sizes = [96, 64, 96]
+    nps = [per_brick * (n // 8) ** 3 for n in sizes]
+    assert sum((n // 8) ** 3 for n in sizes) > 3 * 1216  # (8 blocks on each of 152 SMs)
+    flds = _fields(sizes, 1400, dtype)
+    pos0 = torch.from_numpy(_positions(nps, 1500)).to(DEV)
+    old = {k: ps.ps_tune_get(k) for k in ("batch_persistent", "batch_run_below")}
+    out = []
+    try:
+        ps.ps_tune_set("batch_run_below", 0)  # bricks, not runs
+        for persistent in (0, 1):
+            ps.ps_tune_set("batch_persistent", persistent)
+            plan = ps.BatchPlan([(n,) * 3 for n in sizes], nps, coef_dtype=dtype)
+            pos, ids = pos0.clone(), torch.arange(plan.np_total, device=DEV)
+            st = torch.zeros(4, dtype=torch.int32, device=DEV)
+            plan.run(flds, pos, 3, 4e-3, solve=False, ids=ids, use_graph=False, status=st)
+            assert ps.ps_status_read(st)[0] == 0
+            out.append(torch.empty_like(pos).index_copy_(1, ids, pos))
+    finally:
+        for k, v in old.items():
+            ps.ps_tune_set(k, v)
+    assert torch.equal(*out)
