@@ -361,7 +361,8 @@ ps_status ps_lagrangian_accel(const ps_grid* grid, ps_dtype coef_t,
 /* the results of a permuted call (bin_offsets and perm given).  Storing     */
 /* every particle's values at its own place writes one DRAM sector per value */
 /* once the result rows outgrow the L2; with ws the values are stored in bin */
-/* order and the rows put in place afterwards.  The same results.            */
+/* order and the rows put in place afterwards.  The same results; particles  */
+/* that no slot of the bins names keep what their rows held, as without ws.  */
 /*   ws: ps_unsort_workspace_size(np, rows) bytes, 256-byte aligned, rows =  */
 /*   3 (vel), 12 (vel and grad), 18 (hess), 3 or 6 (acc, acc and vel); NULL  */
 /*   or too small, or without perm: as the calls above.                      */

@@ -159,7 +159,8 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, float* rows_ws) {
       a);
   ps_status rc = check_launch("quad_kernel");
   if (rc || !unsort) return rc;
-  return unsort_launch(a.np, a.perm, rows_ws, a0.vel, a0.vel ? 3 : 0, a0.grad, rows, st);
+  return unsort_launch(a.np, a.perm, a.offs, a.b.nbins, rows_ws, a0.vel, a0.vel ? 3 : 0, a0.grad,
+                       rows, st);
 }
 
 }  // namespace

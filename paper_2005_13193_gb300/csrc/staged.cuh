@@ -93,9 +93,10 @@ ps_status with_quad_type(ps_dtype t, F&& f) {
   }
 }
 // Rows in bin order -> rows in the particles' order (unsort.cu): n0 rows to
-// d0, the next n1 to d1.
-ps_status unsort_launch(int64_t np, const int64_t* perm, float* src, float* d0, int n0,
-                        float* d1, int n1, cudaStream_t st);
+// d0, the next n1 to d1.  Rows of particles that no slot of the bins (offs:
+// nbins + 1 bounds) names stay as they are.
+ps_status unsort_launch(int64_t np, const int64_t* perm, const int32_t* offs, int64_t nbins,
+                        float* src, float* d0, int n0, float* d1, int n1, cudaStream_t st);
 
 // The scatter of a binned cotangent onto a cleared field (adjoint.cu).
 ps_status scatter_bricks_launch(const ps_grid* grid, const int32_t brick[3], int64_t np,

@@ -286,3 +286,38 @@ def test_one_launch_barrier_wait_gives_up():
     finally:
         ps.ps_tune_set("wait_probe", 0)
         ps.ps_tune_set("batch_persistent", 0)
+
+
+@pytest.mark.parametrize("rows", [3, 6, 12, 18])
+def test_rows_that_no_slot_names_are_left_alone(rows):
+    # slots beyond the last offset, and particles whose slot names another one:
+    # by way of bin order too, their rows keep what they held
+    n, brick, np_ = (24, 16, 16), (8, 8, 8), 3000
+    sf = ps.SplineField.from_field(torch.from_numpy(
+        synth.random_field(n, ncomp=3, seed=61).astype(np.float32)).to(DEV))
+    pg = torch.from_numpy(synth.uniform_particles(np_, seed=62)).to(DEV)
+    bins = ps.bin_particles(n, brick, pg)
+    offsets = bins.offsets.clone()
+    offsets[-3:] = offsets[-4]  # the last bricks' particles are in no bin
+    perm = bins.perm.clone()
+    perm[100:200] = perm[:100].clone()
+    covered = perm[:int(offsets[-1])]
+    left = torch.ones(np_, dtype=torch.bool, device=DEV).index_fill_(0, covered, False)
+    assert left.sum() > 150
+    outs = []
+    for ws in (None, ps.workspace(ps._lib().ps_unsort_workspace_size(np_, rows))):
+        if ws is not None:
+            ws.fill_(0x55)
+        o = torch.full((rows, np_), 7.0, device=DEV)
+        kw = dict(perm=perm, bin_offsets=offsets, brick=brick, ws=ws)
+        if rows == 3:
+            ps.ps_interp(sf.coef, n, pg, o, **kw)
+        elif rows == 6:
+            ps.ps_lagrangian_accel(sf.coef, n, pg, o[3:], vel=o[:3], **kw)
+        elif rows == 12:
+            ps.ps_interp(sf.coef, n, pg, o[:3], grad=o[3:], **kw)
+        else:
+            ps.ps_interp_hessian(sf.coef, n, pg, o, **kw)
+        assert torch.all(o[:, left] == 7.0)
+        outs.append(o)
+    assert torch.equal(*outs)
