@@ -510,13 +510,15 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 _UNSORT_BYTES = 80 << 20
 
 
-def _unsort_ws(bins: Optional["Bins"], np_: int, rows: int, device):
+def _unsort_ws(sf: "SplineField", bins: Optional["Bins"], np_: int, rows: int):
     """A workspace for the rows of a permuted call, or None where it would not help or
     does not fit."""
     if bins is None or bins.perm is None or 4 * rows * np_ < _UNSORT_BYTES:
         return None
+    if sf.ncomp != 3 or sf.coef.dtype == torch.float64 or ps_tune_get("brick_kernel") == 2:
+        return None  # kernels that store each value at its own place
     try:
-        return workspace(int(_lib().ps_unsort_workspace_size(np_, rows)), device)
+        return workspace(int(_lib().ps_unsort_workspace_size(np_, rows)), sf.coef.device)
     except torch.cuda.OutOfMemoryError:
         return None
 
@@ -571,7 +573,7 @@ class SplineField:
         """Second derivatives at pos: [ncomp][6][np] (xx, yy, zz, xy, xz, yz); with
         `bins` of these positions, from each brick's staged halo."""
         h = torch.empty((self.ncomp, 6, pos.shape[1]), dtype=torch.float32, device=pos.device)
-        ws = _unsort_ws(bins, pos.shape[1], 18, pos.device)
+        ws = _unsort_ws(self, bins, pos.shape[1], 18)
         ps_interp_hessian(self.coef, self.n, pos, h, scale=self.scale,
                           perm=bins.perm if bins is not None else None,
                           bin_offsets=bins.offsets if bins is not None else None,
@@ -587,7 +589,7 @@ class SplineField:
         `later` (the field dt_field later) when given; with `bins` of these positions,
         from each brick's staged halo."""
         a = torch.empty((3, pos.shape[1]), dtype=torch.float32, device=pos.device)
-        ws = _unsort_ws(bins, pos.shape[1], 3, pos.device)
+        ws = _unsort_ws(self, bins, pos.shape[1], 3)
         ps_lagrangian_accel(self.coef, self.n, pos, a,
                             coef_np1=later.coef if later is not None else None,
                             dt_field=dt_field, scale_n=self.scale,
@@ -605,7 +607,7 @@ class SplineField:
         vel = torch.empty((self.ncomp, np_), dtype=torch.float32, device=pos.device)
         g = (torch.empty((self.ncomp, 3, np_), dtype=torch.float32, device=pos.device)
              if grad else None)
-        ws = _unsort_ws(bins, np_, 12 if grad else 3, pos.device)
+        ws = _unsort_ws(self, bins, np_, 12 if grad else 3)
         ps_interp(self.coef, self.n, pos, vel, scale=self.scale,
                   perm=bins.perm if bins is not None else None,
                   bin_offsets=bins.offsets if bins is not None else None,

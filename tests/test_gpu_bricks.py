@@ -321,3 +321,31 @@ def test_rows_that_no_slot_names_are_left_alone(rows):
         assert torch.all(o[:, left] == 7.0)
         outs.append(o)
     assert torch.equal(*outs)
+
+
+def test_scratch_only_for_rows_that_can_use_it(monkeypatch):
+    # one component, FP64 coefficients and the thread-per-particle kernel store
+    # each value at its own place
+    n, np_ = (24, 16, 16), 2000
+    pg = torch.from_numpy(synth.uniform_particles(np_, seed=63)).to(DEV)
+    bins = ps.bin_particles(n, 8, pg)
+    f = torch.from_numpy(synth.random_field(n, ncomp=3, seed=64).astype(np.float32)).to(DEV)
+    three = ps.SplineField.from_field(f)
+    asked = []
+    real = ps.workspace
+    monkeypatch.setattr(ps, "_UNSORT_BYTES", 0)
+    monkeypatch.setattr(ps, "workspace", lambda *a: asked.append(a) or real(*a))
+    others = [ps.SplineField.from_field(f[:1].contiguous()),
+              ps.SplineField.from_field(f, torch.float64)]
+    del asked[:]
+    for sf in others:
+        sf.interp(pg, grad=True, bins=bins)
+        sf.hessian(pg, bins=bins)
+    ps.ps_tune_set("brick_kernel", 2)
+    try:
+        three.interp(pg, grad=True, bins=bins)
+    finally:
+        ps.ps_tune_set("brick_kernel", -1)
+    assert not asked
+    three.hessian(pg, bins=bins)
+    assert len(asked) == 1
