@@ -11,6 +11,7 @@ torch and call the same entry points.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import functools
 import math
@@ -290,7 +291,8 @@ def ps_spline_coeffs_truncated(field: torch.Tensor, coef: torch.Tensor, K: int =
     if tuple(coef.shape) != coef_shape(n, ncomp, torch.float32):
         raise ValueError(f"coef shape {tuple(coef.shape)} != {coef_shape(n, ncomp, torch.float32)}")
     if ws is None:
-        ws = workspace(ps_spline_truncated_workspace_size(n, ncomp, L), field.device)
+        with _of_stream(stream):
+            ws = workspace(ps_spline_truncated_workspace_size(n, ncomp, L), field.device)
     _dev(ws, "ws")
     g = _grid(n, L)
     _check(_lib().ps_spline_coeffs_truncated(ctypes.byref(g), ncomp, _ptr(field), int(K),
@@ -510,7 +512,20 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 _UNSORT_BYTES = 80 << 20
 
 
-def _unsort_ws(sf: "SplineField", bins: Optional["Bins"], np_: int, rows: int):
+def _of_stream(stream):
+    """The context whose allocations belong to the stream of a call, so that scratch freed
+    when the call returns is reused behind the call's work, and is not memory that work
+    queued on the current stream still uses."""
+    if stream is None:
+        return contextlib.nullcontext()
+    if not isinstance(stream, torch.cuda.Stream):
+        # (handles 0 and 1 name the legacy default stream)
+        stream = (torch.cuda.default_stream() if int(stream) in (0, 1)
+                  else torch.cuda.ExternalStream(int(stream)))
+    return torch.cuda.stream(stream)
+
+
+def _unsort_ws(sf: "SplineField", bins: Optional["Bins"], np_: int, rows: int, stream):
     """A workspace for the rows of a permuted call, or None where it would not help or
     does not fit."""
     if bins is None or bins.perm is None or 4 * rows * np_ < _UNSORT_BYTES:
@@ -518,16 +533,10 @@ def _unsort_ws(sf: "SplineField", bins: Optional["Bins"], np_: int, rows: int):
     if sf.ncomp != 3 or sf.coef.dtype == torch.float64 or ps_tune_get("brick_kernel") == 2:
         return None  # kernels that store each value at its own place
     try:
-        return workspace(int(_lib().ps_unsort_workspace_size(np_, rows)), sf.coef.device)
+        with _of_stream(stream):
+            return workspace(int(_lib().ps_unsort_workspace_size(np_, rows)), sf.coef.device)
     except torch.cuda.OutOfMemoryError:
         return None
-
-
-def _on_stream(ws: Optional[torch.Tensor], stream):
-    """Keep a scratch tensor's memory until the work queued on `stream` is done."""
-    if ws is not None and stream is not None:
-        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream)
-                         else torch.cuda.ExternalStream(int(stream)))
 
 
 class SplineField:
@@ -563,7 +572,8 @@ class SplineField:
             out = cls(coef, scale, n, L)
         need = ps_spline_coeffs_workspace_size(n, ncomp, coef_kind(out.coef), L)
         if need and (ws is None or ws.numel() < need):
-            ws = workspace(need, field.device)
+            with _of_stream(stream):
+                ws = workspace(need, field.device)
         ps_spline_coeffs(field, out.coef, out.scale, ws if need else None, L=L, stream=stream,
                          rows3=rows3)
         return out
@@ -573,13 +583,12 @@ class SplineField:
         """Second derivatives at pos: [ncomp][6][np] (xx, yy, zz, xy, xz, yz); with
         `bins` of these positions, from each brick's staged halo."""
         h = torch.empty((self.ncomp, 6, pos.shape[1]), dtype=torch.float32, device=pos.device)
-        ws = _unsort_ws(self, bins, pos.shape[1], 18)
+        ws = _unsort_ws(self, bins, pos.shape[1], 18, stream)
         ps_interp_hessian(self.coef, self.n, pos, h, scale=self.scale,
                           perm=bins.perm if bins is not None else None,
                           bin_offsets=bins.offsets if bins is not None else None,
                           brick=bins.brick if bins is not None else None, status=status,
                           L=self.L, stream=stream, ws=ws)
-        _on_stream(ws, stream)
         return h
 
     def acceleration(self, pos: torch.Tensor, later: Optional["SplineField"] = None,
@@ -589,7 +598,7 @@ class SplineField:
         `later` (the field dt_field later) when given; with `bins` of these positions,
         from each brick's staged halo."""
         a = torch.empty((3, pos.shape[1]), dtype=torch.float32, device=pos.device)
-        ws = _unsort_ws(self, bins, pos.shape[1], 3)
+        ws = _unsort_ws(self, bins, pos.shape[1], 3, stream)
         ps_lagrangian_accel(self.coef, self.n, pos, a,
                             coef_np1=later.coef if later is not None else None,
                             dt_field=dt_field, scale_n=self.scale,
@@ -598,7 +607,6 @@ class SplineField:
                             bin_offsets=bins.offsets if bins is not None else None,
                             brick=bins.brick if bins is not None else None,
                             status=status, L=self.L, stream=stream, ws=ws)
-        _on_stream(ws, stream)
         return a
 
     def interp(self, pos: torch.Tensor, grad: bool = False, bins: Optional["Bins"] = None,
@@ -607,13 +615,12 @@ class SplineField:
         vel = torch.empty((self.ncomp, np_), dtype=torch.float32, device=pos.device)
         g = (torch.empty((self.ncomp, 3, np_), dtype=torch.float32, device=pos.device)
              if grad else None)
-        ws = _unsort_ws(self, bins, np_, 12 if grad else 3)
+        ws = _unsort_ws(self, bins, np_, 12 if grad else 3, stream)
         ps_interp(self.coef, self.n, pos, vel, scale=self.scale,
                   perm=bins.perm if bins is not None else None,
                   bin_offsets=bins.offsets if bins is not None else None,
                   brick=bins.brick if bins is not None else None, grad=g, status=status,
                   L=self.L, stream=stream, ws=ws)
-        _on_stream(ws, stream)
         return (vel, g) if grad else vel
 
 
@@ -638,7 +645,8 @@ def bin_particles(n, brick, pos: torch.Tensor, L=DEFAULT_L, want_perm=True,
     offsets = torch.empty(nb[0] * nb[1] * nb[2] + 1, dtype=torch.int32, device=dev)
     perm = torch.empty(np_, dtype=torch.int64, device=dev) if want_perm else None
     pos_sorted = torch.empty_like(pos) if want_sorted else None
-    ws = workspace(ps_bin_workspace_size(n, brick, np_, L), dev)
+    with _of_stream(stream):
+        ws = workspace(ps_bin_workspace_size(n, brick, np_, L), dev)
     ps_bin_particles(n, brick, pos, bin_of, offsets, perm, pos_sorted, ws, status, L, stream)
     b = Bins(tuple(brick), offsets, bin_of, perm)
     return (b, pos_sorted) if want_sorted else b

@@ -349,3 +349,32 @@ def test_scratch_only_for_rows_that_can_use_it(monkeypatch):
     assert not asked
     three.hessian(pg, bins=bins)
     assert len(asked) == 1
+
+
+@pytest.mark.parametrize("handle", [False, True])
+def test_scratch_belongs_to_the_stream_of_the_call(handle, monkeypatch):
+    # freed when the call returns, it must come back to that stream only
+    n, np_ = (65, 40, 33), 2000
+    f = torch.from_numpy(synth.random_field(n, ncomp=3, seed=65).astype(np.float32)).to(DEV)
+    pg = torch.from_numpy(synth.uniform_particles(np_, seed=66)).to(DEV)
+    monkeypatch.setattr(ps, "_UNSORT_BYTES", 0)
+    ref = ps.SplineField.from_field(f)
+    bins = ps.bin_particles(n, 8, pg)
+    grad_ref = ref.interp(pg, grad=True, bins=bins)[1]
+    seen = []
+    real = ps.workspace
+    monkeypatch.setattr(ps, "workspace", lambda *a: (
+        seen.append(torch.cuda.current_stream().cuda_stream), real(*a))[1])
+    side = torch.cuda.Stream()
+    for s in (side, torch.cuda.default_stream()):
+        del seen[:]
+        torch.cuda.synchronize()
+        arg = s.cuda_stream if handle else s
+        sf = ps.SplineField.from_field(f, stream=arg)
+        bins = ps.bin_particles(n, 8, pg, stream=arg)
+        grad = sf.interp(pg, grad=True, bins=bins, stream=arg)[1]
+        sf.hessian(pg, bins=bins, stream=arg)
+        sf.acceleration(pg, bins=bins, stream=arg)
+        torch.cuda.synchronize()
+        assert len(seen) == 5 and set(seen) == {s.cuda_stream}
+        assert torch.equal(grad, grad_ref)
