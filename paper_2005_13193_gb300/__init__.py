@@ -572,8 +572,13 @@ class SplineField:
             out = cls(coef, scale, n, L)
         need = ps_spline_coeffs_workspace_size(n, ncomp, coef_kind(out.coef), L)
         if need and (ws is None or ws.numel() < need):
-            with _of_stream(stream):
-                ws = workspace(need, field.device)
+            try:
+                with _of_stream(stream):
+                    ws = workspace(need, field.device)
+            except torch.cuda.OutOfMemoryError:
+                if coef_kind(out.coef) != torch.float32:
+                    raise
+                ws = None  # planar FP32 coefficients can be solved in place
         ps_spline_coeffs(field, out.coef, out.scale, ws if need else None, L=L, stream=stream,
                          rows3=rows3)
         return out

@@ -378,3 +378,20 @@ def test_scratch_belongs_to_the_stream_of_the_call(handle, monkeypatch):
         torch.cuda.synchronize()
         assert len(seen) == 5 and set(seen) == {s.cuda_stream}
         assert torch.equal(grad, grad_ref)
+
+
+def test_planar_solve_without_memory_for_its_scratch(monkeypatch):
+    # planar FP32 coefficients need none: they are solved in place; nodes do
+    n = (65, 40, 33)
+    field = synth.random_field(n, ncomp=3, seed=67).astype(np.float32)
+    f = torch.from_numpy(field).to(DEV)
+
+    def no_memory(*a):
+        raise torch.cuda.OutOfMemoryError("none left")
+
+    monkeypatch.setattr(ps, "workspace", no_memory)
+    sf = ps.SplineField.from_field(f)
+    ref = oracle.spline_coeffs(field.astype(np.float64))
+    assert np.abs(sf.padded().cpu().numpy() - ref).max() <= 2e-6 * np.abs(field).max()
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        ps.SplineField.from_field(f, ps.F32X4)
