@@ -578,7 +578,9 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
       const float tq[3] = {__shfl_sync(FULL, t[0], sj), __shfl_sync(FULL, t[1], sj),
                            __shfl_sync(FULL, t[2], sj)};
       int cq[3] = {0, 0, 0};
-      if (some_out) {
+      // (the cell of stencils read from global memory: outside the halo, or of a
+      // later field that is not staged)
+      if (some_out || (MODE == 4 && second && !use2)) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) cq[d] = __shfl_sync(FULL, cell[d], sj);
       }

@@ -395,3 +395,25 @@ def test_planar_solve_without_memory_for_its_scratch(monkeypatch):
     assert np.abs(sf.padded().cpu().numpy() - ref).max() <= 2e-6 * np.abs(field).max()
     with pytest.raises(torch.cuda.OutOfMemoryError):
         ps.SplineField.from_field(f, ps.F32X4)
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, torch.bfloat16, ps.BF16X4])
+@pytest.mark.parametrize("brick", [(8, 8, 8), (16, 16, 16), (20, 16, 12)])
+def test_acceleration_from_two_fields_in_large_bricks(dtype, brick):
+    # bricks whose two halos do not fit into shared memory side by side: the later
+    # field's nodes come from global memory, at each particle's own cell
+    n, np_ = (48, 40, 33), 6000
+    fields = [synth.random_field(n, ncomp=3, seed=s).astype(np.float32) for s in (70, 71)]
+    a, b = (ps.SplineField.from_field(torch.from_numpy(f).to(DEV), dtype) for f in fields)
+    pos = synth.uniform_particles(np_, seed=72)
+    pg = torch.from_numpy(pos).to(DEV)
+    got = a.acceleration(pg, later=b, dt_field=0.1, bins=ps.bin_particles(n, brick, pg))
+    ref = a.acceleration(pg, later=b, dt_field=0.1)  # the unbinned kernel
+    # both evaluate the same coefficients: velocities 1e-5 of their rms, gradients
+    # 3e-5 max|c| n/L, as above (each side once)
+    u, grad = a.interp(pg, grad=True)
+    cmax = 3 * max(np.abs(f).max() for f in fields)
+    tol = 2 * (3 * float(grad.abs().max()) * 1e-5 * cmax +
+               3 * float(u.abs().max()) * 3e-5 * cmax * max(n) / TWO_PI + 2 * 1e-5 * cmax / 0.1)
+    assert float((got - ref).abs().max()) <= tol
+    assert float((b.interp(pg) - u).abs().max()) / 0.1 > 100 * tol  # the later field counts
