@@ -360,10 +360,11 @@ __device__ __forceinline__ void stage_loads(const StagedArgs& a, const QGeo<CT>&
 
 // Values a lane keeps per particle until it finishes it: MODE 0 velocities; 1
 // and the gradient tensor; 2 the velocities of both stages of a Heun step; 3
-// second derivatives; 4 Lagrangian acceleration (u, its gradient, the later
-// field's u).
+// second derivatives; 4 Lagrangian acceleration from two fields (u, its
+// gradient, the later field's u); 5 from one (u, its gradient).
 template <int MODE> struct NOut {
-  static constexpr int v = MODE == 0 ? 3 : MODE == 1 ? 12 : MODE == 2 ? 6 : MODE == 3 ? 18 : 15;
+  static constexpr int v =
+      MODE == 0 ? 3 : MODE == 1 || MODE == 5 ? 12 : MODE == 2 ? 6 : MODE == 3 ? 18 : 15;
 };
 
 // A particle's stencil start in the halo in one word (negative: outside): the
@@ -418,7 +419,7 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
   const int k = lane & 3, quad = lane >> 2;
   const int64_t np = a.np;
   const Tc* coef = static_cast<const Tc*>(a.coef);
-  const bool second = (MODE == 2 || MODE == 4) && a.coef2 != nullptr;
+  const bool second = MODE == 4 || (MODE == 2 && a.coef2 != nullptr);
   const Tc* coef2 = second ? static_cast<const Tc*>(a.coef2) : coef;
   const float* scale2 = second ? a.scale2 : a.scale;
 
@@ -580,7 +581,7 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
       int cq[3] = {0, 0, 0};
       // (the cell of stencils read from global memory: outside the halo, or of a
       // later field that is not staged)
-      if (some_out || (MODE == 4 && second && !use2)) {
+      if (some_out || (MODE == 4 && !use2)) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) cq[d] = __shfl_sync(FULL, cell[d], sj);
       }
@@ -591,18 +592,13 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
       if (wq >= 0) fetch_halo<Tc, CT>(vq, halo, node, hrow, geo);
       else fetch_global<Tc>(vq, cq, k, g, coef, a.scale);
       if constexpr (MODE == 0) quad_sum<false>(vq, tq, k, out);
-      if constexpr (MODE == 1) quad_sum<true>(vq, tq, k, out);
+      if constexpr (MODE == 1 || MODE == 5) quad_sum<true>(vq, tq, k, out);
       if constexpr (MODE == 3) quad_sum_hess(vq, tq, k, out);
       if constexpr (MODE == 4) {
         quad_sum<true>(vq, tq, k, out);
-        if (second) {
-          if (wq >= 0 && use2) fetch_halo<Tc, CT>(vq, halo2, node, hrow, geo);
-          else fetch_global<Tc>(vq, cq, k, g, coef2, scale2);
-          quad_sum<false>(vq, tq, k, out + 12);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) out[12 + c] = out[c];
-        }
+        if (wq >= 0 && use2) fetch_halo<Tc, CT>(vq, halo2, node, hrow, geo);
+        else fetch_global<Tc>(vq, cq, k, g, coef2, scale2);
+        quad_sum<false>(vq, tq, k, out + 12);
       }
       if constexpr (MODE == 2) {
         quad_sum<false>(vq, tq, k, out);
@@ -686,15 +682,16 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
             a.grad[(c * 6 + e) * np + oo] = ok ? __fmul_rn(res[3 * e + c], sc[e]) : nanf_;
       }
     }
-    if constexpr (MODE == 4) {
-      // a = (u . grad) u + (u(coef2) - u) / dt_field (a.dt = 1 / dt_field) -> a.grad [3][np]
+    if constexpr (MODE == 4 || MODE == 5) {
+      // a = (u . grad) u [+ (u(coef2) - u) / dt_field] (a.dt = 1 / dt_field) -> a.grad [3][np]
       if (v) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           float acc = __fmul_rn(__fmul_rn(res[3 + c], g.inv_hf[0]), res[0]);
           acc = __fmaf_rn(__fmul_rn(res[6 + c], g.inv_hf[1]), res[1], acc);
           acc = __fmaf_rn(__fmul_rn(res[9 + c], g.inv_hf[2]), res[2], acc);
-          if (second) acc = __fmaf_rn(__fsub_rn(res[12 + c], res[c]), (float)a.dt, acc);
+          if (MODE == 4)
+            acc = __fmaf_rn(__fsub_rn(res[MODE == 4 ? 12 + c : 0], res[c]), (float)a.dt, acc);
           a.grad[c * np + oo] = ok ? acc : nanf_;
           if (a.vel) a.vel[c * np + oo] = ok ? res[c] : nanf_;
         }

@@ -417,3 +417,26 @@ def test_acceleration_from_two_fields_in_large_bricks(dtype, brick):
                3 * float(u.abs().max()) * 3e-5 * cmax * max(n) / TWO_PI + 2 * 1e-5 * cmax / 0.1)
     assert float((got - ref).abs().max()) <= tol
     assert float((b.interp(pg) - u).abs().max()) / 0.1 > 100 * tol  # the later field counts
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, ps.F16X4, torch.bfloat16])
+def test_acceleration_from_one_field(dtype):
+    # the convective part alone, bricks staged and not, a ragged last brick; bars as
+    # above: velocities 1e-5 of their rms, gradients 3e-5 max|c| n/L, 16-bit values
+    # compared with the unbinned kernel of the same coefficients
+    n, brick, np_ = (40, 24, 17), (8, 8, 8), 1500
+    field = synth.random_field(n, ncomp=3, seed=68).astype(np.float32)
+    sf = ps.SplineField.from_field(torch.from_numpy(field).to(DEV), dtype)
+    pos = synth.uniform_particles(np_, seed=69)
+    pg = torch.from_numpy(pos).to(DEV)
+    bins = ps.bin_particles(n, brick, pg)
+    got = sf.acceleration(pg, bins=bins)
+    vel, grad = (t.cpu().numpy().astype(np.float64) for t in sf.interp(pg, grad=True))
+    if dtype in (ps.F32X4, torch.float32):
+        vel, grad = oracle.interp(oracle.spline_coeffs(field.astype(np.float64)), pos, grad=True)
+    ref = (grad * vel[None]).sum(1)
+    gtol = 3e-5 * np.abs(field).max() * 3 * max(n) / TWO_PI
+    tol = 3 * (np.abs(grad).max() * 1e-5 * np.sqrt((vel ** 2).mean()) + np.abs(vel).max() * gtol)
+    assert np.abs(got.cpu().numpy() - ref).max() <= tol
+    # the time derivative of a field that does not change adds nothing
+    assert torch.equal(sf.acceleration(pg, later=sf, dt_field=0.5, bins=bins), got)
