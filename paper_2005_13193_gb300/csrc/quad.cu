@@ -91,6 +91,22 @@ bool halo_map(StagedArgs* a) {
   }
 }
 
+// Whether a step through two fields (or an acceleration from two) stages both
+// halos: from so many particles per brick on (of 11^3 halo nodes, others in
+// proportion).  Below, the later field's nodes are read from global memory: one
+// halo less to bring in, and twice the blocks.  256^3, one halo / both, us.  Heun
+// step: FP32 nodes, 12 particles per brick 267 / 288, 24 382 / 341, 64 680 / 411;
+// planar FP32 6 206 / 278, 12 250 / 238, 24 352 / 281; planar FP16 12 520 / 577, 24
+// 722 / 648; 16-bit nodes (whose later halo comes by plain loads) 24 300 / 347, 64
+// 440 / 457, 96 627 / 611.  Acceleration: 6 198 / 255, 12 246 / 235; 6 148 / 212,
+// 12 193 / 177; 12 448 / 519, 24 586 / 589; 24 232 / 278, 64 365 / 356.
+template <typename Tc>
+bool second_halo_pays(const StagedArgs& a) {
+  constexpr double least = IsNode16<Tc>::value ? 64.0 : IsQuant<Tc>::value ? 20.0 : 14.0;
+  const double nodes = (double)a.S[0] * a.S[1] * a.S[2];
+  return (double)a.np * 1331.0 >= least * nodes * (double)a.b.nbins;
+}
+
 // Geometry, shared memory and tensor maps of the quad form; *ct: the
 // compile-time geometry that applies (0: none).
 template <typename Tc>
@@ -116,7 +132,7 @@ void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
     return;
   }
   // a second field's halo beside the first where both fit
-  if (second && a->coef2 && 2 * *smem <= 226 * 1024) {
+  if (second && a->coef2 && 2 * *smem <= 226 * 1024 && second_halo_pays<Tc>(*a)) {
     a->two = 1;
     *smem *= 2;
     if constexpr (!n16) {

@@ -440,3 +440,44 @@ def test_acceleration_from_one_field(dtype):
     assert np.abs(got.cpu().numpy() - ref).max() <= tol
     # the time derivative of a field that does not change adds nothing
     assert torch.equal(sf.acceleration(pg, later=sf, dt_field=0.5, bins=bins), got)
+
+
+def _staged_and_not(n, brick, per, dtype, seed):
+    """Every brick call's results with halos staged as the dispatch has it, and with
+    every stencil from global memory."""
+    nbins = math.prod(-(-n[d] // brick[d]) for d in range(3))
+    pos = torch.from_numpy(synth.uniform_particles(per * nbins, seed=seed)).to(DEV)
+    a, b = (ps.SplineField.from_field(torch.from_numpy(
+        synth.random_field(n, ncomp=3, seed=seed + i).astype(np.float32)).to(DEV), dtype)
+        for i in (1, 2))
+    bins, xs = ps.bin_particles(n, brick, pos, want_sorted=True)
+    bins.perm = None
+    dt = 0.4 * TWO_PI / max(n)
+    out = []
+    try:
+        for least in (8, 1 << 20):
+            ps.ps_tune_set("brick_min_stage", least)
+            st = torch.zeros(4, dtype=torch.int32, device=DEV)
+            r = [*a.interp(xs, grad=True, bins=bins, status=st), a.interp(xs, bins=bins),
+                 a.hessian(xs, bins=bins), a.acceleration(xs, bins=bins),
+                 a.acceleration(xs, later=b, dt_field=0.1, bins=bins)]
+            for later in (None, b):
+                x, v = xs.clone(), torch.empty((3, xs.shape[1]), device=DEV)
+                ps.ps_rk2_step(a.coef, n, x, dt, coef_np1=later.coef if later else None,
+                               scale_n=a.scale, scale_np1=later.scale if later else None,
+                               vel_out=v, brick=brick, rebin=0, bin_offsets=bins.offsets,
+                               status=st)
+                r += [x, v]
+            assert ps.ps_status_read(st)[0] == 0
+            out.append(r)
+    finally:
+        ps.ps_tune_set("brick_min_stage", 8)
+    return out
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, ps.BF16X4, torch.float16])
+@pytest.mark.parametrize("per", [9, 13, 15, 21, 63, 65, 130])
+def test_halos_staged_or_not(per, dtype):
+    # around the densities from which a second field's halo is staged
+    staged, plain = _staged_and_not((32, 24, 16), (8, 8, 8), per, dtype, 80)
+    assert all(torch.equal(s, p) for s, p in zip(staged, plain))
