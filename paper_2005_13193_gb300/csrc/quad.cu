@@ -147,6 +147,24 @@ void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
   }
 }
 
+// Threads of a brick's block.  64 (two warps) where eight blocks share an SM; the
+// registers hold four blocks of 128.  So where the halos' size (as many as fit
+// into 227 KB) or the number of bricks leaves at most four blocks on an SM, 128
+// take twice the particles at a time.  64^3 FP32 nodes, 64 / 128 threads, us: 512
+// particles per brick, interpolation 25 / 20, gradient 33 / 27, Heun step 57 / 46;
+// 2048, 78 / 60, 111 / 84, 171 / 127 (32: alike); 72^3, with five blocks on an SM,
+// 88 / 91, 130 / 130, 200 / 205.  Bricks of 16^3, 128^3, 1.5 M particles: 348 /
+// 189, 503 / 271, 790 / 434.  With five to seven blocks that fit, 128 pay for dense
+// bricks (two planar halos, six blocks, Heun step at 256^3: 64 particles per brick
+// 404 / 452, 96 565 / 518, 256 1252 / 1189).
+int brick_threads(const StagedArgs& a, size_t smem) {
+  const int64_t fit = std::min<int64_t>(8, 227 * 1024 / ((int64_t)smem + 1024));
+  const int64_t sms = sm_count(), waiting = (a.b.nbins + sms - 1) / sms;
+  if (fit <= 4) return 128;
+  if (waiting <= 4) return a.np >= 64 * a.b.nbins ? 128 : 64;
+  return fit < 8 && a.np >= 96 * a.b.nbins ? 128 : 64;
+}
+
 template <typename Tc, int MODE>
 ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, float* rows_ws) {
   StagedArgs a = a0;
@@ -163,7 +181,7 @@ ps_status launch_quad_t(const StagedArgs& a0, cudaStream_t st, float* rows_ws) {
         "quad smem attribute");
     if (rc) return rc;
   }
-  const int threads = a.two ? 128 : 64;
+  const int threads = brick_threads(a, smem);
   // results by way of bin order: vel, then the gradient's or the second
   // derivatives' rows
   constexpr int rows = MODE == 1 ? 9 : MODE == 3 ? 18 : MODE >= 4 ? 3 : 0;
