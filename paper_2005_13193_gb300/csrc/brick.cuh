@@ -461,10 +461,10 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
         // the nodes and the rows' scales, both on one barrier
         tma_copy_node16(&maps->tmap, &maps->tmap2, halo,
                         halo + scale_off_bytes(geo.Sz, geo.PS), &mbar[0], P0,
-                        (unsigned)(geo.Sz * geo.Sy * (geo.SX * 8 + 16)));
+                        (unsigned)(geo.Sz * (geo.PS * 8 + geo.Sy * 16)));
       } else if constexpr (IsNode4<Tc>::value || IsPlanar<Tc>::value) {
         const unsigned bytes =
-            (unsigned)((IsPlanar<Tc>::value ? 12 : 16) * geo.SX * geo.Sy * geo.Sz);
+            (unsigned)((IsPlanar<Tc>::value ? 12 : 16) * geo.PS * geo.Sz);
         tma_copy<IsPlanar<Tc>::value>(&maps->tmap, halo, &mbar[0], P0, bytes);
         if (tma2) {
           if (ONCE) tma_init_barrier(&mbar[1]);

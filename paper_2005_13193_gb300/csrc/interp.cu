@@ -956,8 +956,8 @@ ps_status fill_staged(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[
   return PS_OK;
 }
 
-// Tensor map of the halo box over the coefficients (nodes: S[1] x S[2] rows of
-// SX nodes; planar FP32: rows of SX floats of the three components); the
+// Tensor map of the halo box over the coefficients (nodes: S[2] planes of PS / SX
+// rows of SX nodes; planar FP32: rows of SX floats of the three components); the
 // driver's encoder is looked up once.
 bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -982,12 +982,13 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
   const cuuint32_t unit[3] = {1, 1, 1};
   const cuuint64_t m1 = (cuuint64_t)g.m[1], m2 = (cuuint64_t)g.m[2], rx = (cuuint64_t)g.rx;
   // a box holds at most 256 values per axis
-  if (a->S[1] > 256 || a->S[2] > 256 || (coef_t == PS_F32 ? 1 : 4) * a->SX > 256) return false;
+  const cuuint32_t rows = (cuuint32_t)(a->PS / a->SX);
+  if (rows > 256 || a->S[2] > 256 || (coef_t == PS_F32 ? 1 : 4) * a->SX > 256) return false;
   if (coef_t == PS_F32) {
     // planar: [3][m2][m1][rx] floats, the box's three components one behind the other
     const cuuint64_t pd[4] = {rx, m1, m2, 3};
     const cuuint64_t ps[3] = {rx * 4, rx * m1 * 4, rx * m1 * m2 * 4};
-    const cuuint32_t pb[4] = {(cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2], 3};
+    const cuuint32_t pb[4] = {(cuuint32_t)a->SX, rows, (cuuint32_t)a->S[2], 3};
     const cuuint32_t pu[4] = {1, 1, 1, 1};
     return encode(&a->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(a->coef), pd, ps,
                   pb, pu, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -995,7 +996,7 @@ bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t) {
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   }
   const cuuint64_t dims[3] = {4 * rx, m1, m2};
-  const cuuint32_t box[3] = {4 * (cuuint32_t)a->SX, (cuuint32_t)a->S[1], (cuuint32_t)a->S[2]};
+  const cuuint32_t box[3] = {4 * (cuuint32_t)a->SX, rows, (cuuint32_t)a->S[2]};
   const cuuint64_t nb = coef_t == PS_F32X4 ? 16 : 8;  // bytes of a node
   const cuuint64_t strides[2] = {rx * nb, rx * m1 * nb};
   const CUtensorMapDataType t = coef_t == PS_F32X4    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32

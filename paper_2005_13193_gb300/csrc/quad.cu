@@ -50,22 +50,25 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
                            phase);
 }
 
-// Row length SX >= S[0] of a halo.  float4 nodes: SX even with SX * S[1] = 2 or
-// 6 (mod 8) where there is one (a quad's four z-rows on four bank groups of one
-// parity), else S[0].
-int quad_row(int sx, int sy) {
-  for (int r = sx; r < sx + 8; ++r)
-    if (((r * sy) & 3) == 2) return r;
-  return sx;
-}
-// 16-bit nodes and planar floats: rows of whole 16-byte units (node pairs,
-// four floats), SX a multiple of 4 with SX * S[1] an odd multiple of 4 where
-// there is one, so that the four z-rows of a quad read banks 4 apart.
-int quad_row4(int sx, int sy, int unit) {
-  const int r0 = (sx + unit - 1) / unit * unit;
-  for (int r = r0; r < r0 + 16; r += unit)
-    if ((r & 3) == 0 && ((r * sy) & 7) == 4) return r;
-  return r0;
+// The halo as it lies in shared memory: rows of SX >= S[0] nodes and planes of PS
+// nodes, PS / SX >= S[1] rows (the further ones are copied too and not read), the
+// smallest plane whose stride spreads a quad's four z-rows over the banks.  float4
+// nodes: PS = 2 (mod 4), four bank groups of one parity; 16-bit nodes and planar
+// floats: rows of whole 16-byte units (`unit` values), PS an odd multiple of 4, so
+// that the rows' banks are 4 apart.  Extents S[1] that are a multiple of 4 have
+// such planes with further rows only (bricks of 12 x 5 x 8, 128^3, 1.5 M particles,
+// interpolation without / with them, us: FP32 nodes 205 / 79, planar 227 / 102).
+void halo_plane(StagedArgs* a, int unit, bool words) {
+  const int r0 = (a->S[0] + unit - 1) / unit * unit;
+  int best = 0;
+  for (int sy = a->S[1]; sy < a->S[1] + 4; ++sy)
+    for (int r = r0; r < r0 + 16; r += unit) {
+      const bool ok = words ? (r & 3) == 0 && ((r * sy) & 7) == 4 : ((r * sy) & 3) == 2;
+      if (!ok || (best && r * sy >= best)) continue;
+      best = r * sy;
+      a->SX = r;
+    }
+  a->PS = best;
 }
 template <typename Tc> struct CoefDtype { static constexpr int v = -1; };
 template <> struct CoefDtype<float> { static constexpr int v = PS_F32; };
@@ -112,10 +115,7 @@ bool second_halo_pays(const StagedArgs& a) {
 template <typename Tc>
 void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
   constexpr bool n16 = IsNode16<Tc>::value, planar = IsPlanar<Tc>::value;
-  a->SX = n16      ? quad_row4(a->S[0], a->S[1], 2)
-          : planar ? quad_row4(a->S[0], a->S[1], 4)
-                   : quad_row(a->S[0], a->S[1]);
-  a->PS = a->SX * a->S[1];
+  halo_plane(a, n16 ? 2 : planar ? 4 : 1, n16 || planar);
   a->half_dt = 0.5 * a->dt;
   for (int d = 0; d < 3; ++d) a->ih32[d] = a->g.inv_h[d] * 4294967296.0;
   a->wait_probe = tuning().wait_probe;

@@ -16,8 +16,8 @@ struct StagedArgs {
   BrickArgs b;
   int E;        // extra halo cells on each side
   int S[3];     // staged extent per axis: B + 3 + 2E
-  int SX;       // row stride in float4 units (= S[0])
-  int PS;       // plane stride in float4 units: >= SX*S[1], = 4 (mod 8)
+  int SX;       // row stride in nodes (or planar values), >= S[0]
+  int PS;       // plane stride, >= SX * S[1] (phased kernel: = 4 mod 8; quad.cu)
   int vec;      // 1: halo rows are whole 16-byte vectors inside the array
   int min_stage;  // bricks with fewer particles gather from global memory
   int tma;        // 1: the node halo is one tensor copy described by tmap

@@ -481,3 +481,11 @@ def test_halos_staged_or_not(per, dtype):
     # around the densities from which a second field's halo is staged
     staged, plain = _staged_and_not((32, 24, 16), (8, 8, 8), per, dtype, 80)
     assert all(torch.equal(s, p) for s, p in zip(staged, plain))
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, ps.F16X4, torch.float16])
+@pytest.mark.parametrize("brick", [(8, 5, 8), (8, 1, 4), (4, 9, 4), (12, 5, 3), (7, 13, 2)])
+def test_halo_planes_with_further_rows(brick, dtype):
+    # halos of a multiple of 4 rows per plane lie with rows that no stencil uses
+    staged, plain = _staged_and_not((24, 26, 16), brick, 40, dtype, 90)
+    assert all(torch.equal(s, p) for s, p in zip(staged, plain))
