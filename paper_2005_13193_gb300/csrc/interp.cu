@@ -1311,6 +1311,26 @@ extern "C" ps_status ps_interp_backward_binned(
                             status, stream);
 }
 
+// Bricks whose halos are a multiple of four rows high bring further rows into
+// shared memory (quad.cu); with few particles each, the second derivatives and the
+// acceleration are faster unbinned: 128^3, second derivatives, staged / unbinned,
+// us: bricks of 8 x 1 x 8 with 4.6 particles FP32 nodes 86 / 32, planar 89 / 29,
+// planar FP16 99 / 33; 8 x 5 x 8 with 23 particles 37 / 33, 39 / 28, 104 / 35; 4 x 9
+// x 4 with 24, coefficients in the L2, 80 / 70, 83 / 60, 218 / 71; 256^3, beyond
+// the L2, 8 x 1 x 8 with 4, 753 / 208, 746 / 212, 818 / 257, with 8, 370 / 192,
+// 380 / 193 (4 x 9 x 4).
+static bool unbinned_pays(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3],
+                          int64_t np) {
+  StagedArgs a{};
+  size_t smem;
+  if ((brick[1] + 3) % 4 || fill_staged(grid, coef_t, brick, 0, false, &a, &smem))
+    return false;  // (what the staged form refuses stays refused)
+  const double nodes = (double)a.S[0] * a.S[1] * a.S[2];
+  const double bytes = (double)grid_volume(grid) * 3.0 * (double)dtype_size(coef_t);
+  const double least = bytes <= 64e6 ? 30.0 : 12.0;  // per 11^3 nodes
+  return (double)np * 1331.0 < least * nodes * (double)a.b.nbins;
+}
+
 // Brick-staged form of the second derivatives (mode 3) or the Lagrangian
 // acceleration (mode 4) by the quad kernel.
 static ps_status staged_extra(const ps_grid* grid, ps_dtype coef_t, const void* coef,
@@ -1365,7 +1385,7 @@ extern "C" ps_status ps_interp_hessian_ws(const ps_grid* grid, int ncomp, ps_dty
   if (perm && !bin_offsets) return fail(PS_ERR_INVALID_ARG, "perm needs bin_offsets");
   if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
   cudaStream_t st = as_stream(stream);
-  if (bin_offsets && ncomp == 3 && coef_t != PS_F64) {
+  if (bin_offsets && ncomp == 3 && coef_t != PS_F64 && !unbinned_pays(grid, coef_t, brick, np)) {
     return staged_extra(grid, coef_t, coef, scale, nullptr, nullptr, 0.0, np, pos, perm,
                         bin_offsets, brick, hess, nullptr, result_rows(perm, np, 18, ws, ws_bytes),
                         status, 3, st);
@@ -1417,7 +1437,7 @@ extern "C" ps_status ps_lagrangian_accel_ws(const ps_grid* grid, ps_dtype coef_t
   if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
   cudaStream_t st = as_stream(stream);
   const double inv_dt = coef_np1 ? 1.0 / dt_field : 0.0;
-  if (bin_offsets && coef_t != PS_F64) {
+  if (bin_offsets && coef_t != PS_F64 && !unbinned_pays(grid, coef_t, brick, np)) {
     return staged_extra(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, inv_dt, np, pos, perm,
                       bin_offsets, brick, acc, vel, result_rows(perm, np, vel ? 6 : 3, ws, ws_bytes),
                       status, 4, st);

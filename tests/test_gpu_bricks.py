@@ -489,3 +489,25 @@ def test_halo_planes_with_further_rows(brick, dtype):
     # halos of a multiple of 4 rows per plane lie with rows that no stencil uses
     staged, plain = _staged_and_not((24, 26, 16), brick, 40, dtype, 90)
     assert all(torch.equal(s, p) for s, p in zip(staged, plain))
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, torch.float16])
+@pytest.mark.parametrize("brick,per", [((8, 1, 8), 4), ((8, 5, 8), 20), ((8, 5, 8), 60)])
+def test_sparse_bricks_of_unfavourable_height(brick, per, dtype):
+    # with few particles second derivatives and accelerations take the unbinned
+    # kernels, with more the staged ones: both within the bars of the FP32 sums
+    n = (24, 25, 16)
+    np_ = per * math.prod(-(-n[d] // brick[d]) for d in range(3))
+    sf = ps.SplineField.from_field(torch.from_numpy(
+        synth.random_field(n, ncomp=3, seed=95).astype(np.float32)).to(DEV), dtype)
+    pg = torch.from_numpy(synth.uniform_particles(np_, seed=96)).to(DEV)
+    bins = ps.bin_particles(n, brick, pg)
+    for call, unit in ((sf.hessian, 6 * (max(n) / TWO_PI) ** 2),
+                       (sf.acceleration, 9 * max(n) / TWO_PI)):
+        got, ref = call(pg, bins=bins), call(pg)
+        assert torch.equal(got, ref) == (per < 30)
+        cmax = float(sf.padded().abs().max())
+        scale = cmax if call == sf.hessian else cmax ** 2
+        assert float((got - ref).abs().max()) <= 1e-5 * 8 * unit * scale
+    with pytest.raises(RuntimeError):  # a brick that the staged form refuses
+        sf.hessian(pg, bins=ps.Bins((30, 5, 8), bins.offsets, None, bins.perm))
