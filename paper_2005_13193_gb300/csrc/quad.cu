@@ -102,10 +102,12 @@ bool halo_map(StagedArgs* a) {
 // planar FP32 6 206 / 278, 12 250 / 238, 24 352 / 281; planar FP16 12 520 / 577, 24
 // 722 / 648; 16-bit nodes (whose later halo comes by plain loads) 24 300 / 347, 64
 // 440 / 457, 96 627 / 611.  Acceleration: 6 198 / 255, 12 246 / 235; 6 148 / 212,
-// 12 193 / 177; 12 448 / 519, 24 586 / 589; 24 232 / 278, 64 365 / 356.
+// 12 193 / 177; 12 448 / 519, 24 586 / 589; 24 232 / 278, 64 365 / 356.  Planar 16
+// bits in bricks that do not tile the grid, whose rows come value by value (250 x
+// 200 x 150, Heun step): 24 493 / 670, 48 644 / 708, 96 824 / 750.
 template <typename Tc>
 bool second_halo_pays(const StagedArgs& a) {
-  constexpr double least = IsNode16<Tc>::value ? 64.0 : IsQuant<Tc>::value ? 20.0 : 14.0;
+  const double least = IsNode16<Tc>::value ? 64.0 : !IsQuant<Tc>::value ? 14.0 : a.vec ? 20.0 : 80.0;
   const double nodes = (double)a.S[0] * a.S[1] * a.S[2];
   return (double)a.np * 1331.0 >= least * nodes * (double)a.b.nbins;
 }

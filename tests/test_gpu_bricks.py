@@ -511,3 +511,10 @@ def test_sparse_bricks_of_unfavourable_height(brick, per, dtype):
         assert float((got - ref).abs().max()) <= 1e-5 * 8 * unit * scale
     with pytest.raises(RuntimeError):  # a brick that the staged form refuses
         sf.hessian(pg, bins=ps.Bins((30, 5, 8), bins.offsets, None, bins.perm))
+
+
+@pytest.mark.parametrize("per", [30, 110])
+def test_planar_16_bit_halos_in_ragged_boxes(per):
+    # below and above the density from which both fields' halos are staged there
+    staged, plain = _staged_and_not((30, 21, 17), (8, 8, 8), per, torch.bfloat16, 100)
+    assert all(torch.equal(s, p) for s, p in zip(staged, plain))
