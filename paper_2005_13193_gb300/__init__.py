@@ -507,9 +507,24 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 
 # Result rows from this size on go through bin order (see ps_interp_ws): beyond a good
 # half of the L2, scattered 4-byte stores reach DRAM one by one.  Stored directly / by
-# way of bin order, us: 34 MiB 86 / 112, 46 MiB 384 / 390, 69 MiB 160 / 191,
-# 92 MiB 594 / 310 and 1011 / 740, 183 MiB 1668 / 582, 549 MiB 5695 / 1490.
-_UNSORT_BYTES = 80 << 20
+# way of bin order, us, 96^3: 46 MiB 123 / 160, 69 MiB 190 / 221, 92 MiB 336 / 309, 183
+# MiB 701 / 607; 256^3: 183 MiB 1668 / 582, 549 MiB 5695 / 1490.  Particles of a bin are
+# in about their own order, so that bricks that all run at once (up to 8 blocks on each
+# of 152 SMs) write near one another: 64^3, 512 bricks, 183 MiB 456 / 554, 275 MiB 767 /
+# 739; 72^3, 729, 549 MiB 1736 / 2020, 824 MiB 3322 / 2555.  Fewer than four rows are put
+# in place by words and gain less: three of 12 M particles, 96^3 1025 / 1150, 112^3 1129 /
+# 1196, 128^3 1281 / 1230, 160^3 1585 / 1320.
+_UNSORT_BYTES = 88 << 20
+_UNSORT_AT_ONCE = 8 * 152
+_UNSORT_BYTES_AT_ONCE = 600 << 20
+_UNSORT_BRICKS_OF_FEW_ROWS = 3000
+
+
+def _unsort_pays(np_: int, rows: int, bricks: int) -> bool:
+    if rows < 4 and bricks < _UNSORT_BRICKS_OF_FEW_ROWS:
+        return False
+    return 4 * rows * np_ >= (_UNSORT_BYTES_AT_ONCE if bricks <= _UNSORT_AT_ONCE
+                              else _UNSORT_BYTES)
 
 
 def _of_stream(stream):
@@ -528,7 +543,9 @@ def _of_stream(stream):
 def _unsort_ws(sf: "SplineField", bins: Optional["Bins"], np_: int, rows: int, stream):
     """A workspace for the rows of a permuted call, or None where it would not help or
     does not fit."""
-    if bins is None or bins.perm is None or 4 * rows * np_ < _UNSORT_BYTES:
+    if bins is None or bins.perm is None:
+        return None
+    if not _unsort_pays(np_, rows, bins.offsets.numel() - 1):
         return None
     if sf.ncomp != 3 or sf.coef.dtype == torch.float64 or ps_tune_get("brick_kernel") == 2:
         return None  # kernels that store each value at its own place

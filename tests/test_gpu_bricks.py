@@ -333,7 +333,7 @@ def test_scratch_only_for_rows_that_can_use_it(monkeypatch):
     three = ps.SplineField.from_field(f)
     asked = []
     real = ps.workspace
-    monkeypatch.setattr(ps, "_UNSORT_BYTES", 0)
+    monkeypatch.setattr(ps, "_unsort_pays", lambda *a: True)
     monkeypatch.setattr(ps, "workspace", lambda *a: asked.append(a) or real(*a))
     others = [ps.SplineField.from_field(f[:1].contiguous()),
               ps.SplineField.from_field(f, torch.float64)]
@@ -357,7 +357,7 @@ def test_scratch_belongs_to_the_stream_of_the_call(handle, monkeypatch):
     n, np_ = (65, 40, 33), 2000
     f = torch.from_numpy(synth.random_field(n, ncomp=3, seed=65).astype(np.float32)).to(DEV)
     pg = torch.from_numpy(synth.uniform_particles(np_, seed=66)).to(DEV)
-    monkeypatch.setattr(ps, "_UNSORT_BYTES", 0)
+    monkeypatch.setattr(ps, "_unsort_pays", lambda *a: True)
     ref = ps.SplineField.from_field(f)
     bins = ps.bin_particles(n, 8, pg)
     grad_ref = ref.interp(pg, grad=True, bins=bins)[1]

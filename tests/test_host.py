@@ -1,6 +1,7 @@
 """Host-side logic that needs no GPU: the autotuner's cache file and the
 plane-by-plane spectral generator."""
 import numpy as np
+import pytest
 import torch
 
 from paper_2005_13193_gb300 import autotune, synth
@@ -60,3 +61,13 @@ def test_tracker_rebin_modes(monkeypatch):
     full.step(1e-3)
     full.step(1e-3)
     assert seen == [1, 1]
+
+
+@pytest.mark.parametrize("np_,rows,bricks,pays", [
+    (2_000_000, 12, 4096, True), (1_000_000, 18, 4096, False), (4_000_000, 12, 512, False),
+    (4_000_000, 18, 729, False), (12_000_000, 18, 512, True), (2_000_000, 18, 1331, True),
+    (12_000_000, 3, 2744, False), (12_000_000, 3, 4096, True), (4_000_000, 3, 4096, False)])
+def test_rows_by_way_of_bin_order_where_it_pays(np_, rows, bricks, pays):
+    # few bricks write near one another as it is; few rows gain less
+    import paper_2005_13193_gb300 as ps
+    assert ps._unsort_pays(np_, rows, bricks) == pays
