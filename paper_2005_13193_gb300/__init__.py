@@ -725,22 +725,40 @@ class Tracker:
         self._counted = mode >= 2 and self.brick is not None
 
 
-# Particles of one differentiable call from which binning them first pays (forward and
-# both gradients go brick by brick).  Forward and backward in particle order / binned, us:
-#   256^3: 100 k particles 646 / 884, 200 k 902 / 910, 500 k 1667 / 995, 1 M 2950 / 1194
-#   128^3: 200 k 339 / 502, 500 k 468 / 511, 1 M 796 / 655;  64^3: 1 M 745 / 706
-# Coefficients that the L2 holds are gathered from it at any order, and the binned way has
-# more launches; beyond it, binning pays from some particles per brick.
+# Particles of one differentiable call from which binning them first pays: forward
+# and gradients then go brick by brick.  By what the call computes, in particle order
+# / binned, us:
+#                          velocity      position grad.  field grad.    both
+#   64^3  600 k           145 / 149      270 / 350      346 / 388      471 / 423
+#   64^3  800 k           184 / 150      349 / 355      444 / 400      608 / 483
+#   64^3  1.2 M           263 / 196      506 / 424      627 / 461      872 / 656
+#   96^3  800 k, 6 M      203 / 198, 1217 / 1413        469 / 398      635 / 516
+#   128^3 800 k, 6 M      220 / 205, 1236 / 1280        496 / 413      662 / 554
+#   192^3 200 k           210 / 227      276 / 370      428 / 506      494 / 558
+#   192^3 400 k           265 / 245      385 / 373      580 / 540      698 / 620
+#   256^3 300 k           387 / 315      594 / 402      953 / 851     1162 / 927
+#   256^3 1.5 M          1174 / 453     2174 / 767     3262 / 1107    4255 / 1401
+#   384^3 800 k          1753 / 1330    2542 / 1539    3856 / 3019    4634 / 3214
+# Coefficients that the L2 holds are gathered from it at any order, and the binned way
+# has more launches; beyond it, binning pays from some particles per brick.
 _FN_BRICK = (8, 8, 8)
 _FN_L2_BYTES = 64 << 20
 _FN_MIN_IN_L2 = 800_000
+_FN_MIN_BEYOND = 400_000
 _FN_MIN_PER_BRICK = 8
 
 
-def _fn_binned(n, np_: int) -> bool:
+def _fn_binned(n, np_: int, pos_grad: bool, field_grad: bool) -> bool:
+    if 12 * math.prod(n) > _FN_L2_BYTES:
+        least, most = _FN_MIN_BEYOND, 2**31 - 1
+    elif field_grad:
+        least, most = _FN_MIN_IN_L2, 2**31 - 1
+    elif pos_grad:
+        least, most = _FN_MIN_IN_L2 * 5 // 4, 2**31 - 1
+    else:
+        least, most = _FN_MIN_IN_L2, 4_000_000
     nbins = math.prod(-(-n[d] // _FN_BRICK[d]) for d in range(3))
-    least = _FN_MIN_IN_L2 if 12 * math.prod(n) <= _FN_L2_BYTES else 0
-    return max(least, _FN_MIN_PER_BRICK * nbins) <= np_ < 2**31
+    return max(least, _FN_MIN_PER_BRICK * nbins) <= np_ <= most
 
 
 class InterpFn(torch.autograd.Function):
@@ -752,8 +770,8 @@ class InterpFn(torch.autograd.Function):
     def forward(ctx, pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L):
         sf = SplineField.from_field(field.detach().float(), torch.float32, L, rows3=True)
         x = pos.detach()
-        order = None
-        if sf.ncomp == 3 and _fn_binned(sf.n, x.shape[1]):
+        order = (None, None, None)
+        if sf.ncomp == 3 and _fn_binned(sf.n, x.shape[1], *ctx.needs_input_grad[:2]):
             # positions in bin order serve the forward and both gradients; what
             # goes in or out in the particles' own order is moved by rows
             try:
@@ -763,18 +781,17 @@ class InterpFn(torch.autograd.Function):
                 ps_permute_rows(vs, bins.perm, vel, to_bins=False)
                 order = (bins.perm, bins.offsets, xs)
             except torch.cuda.OutOfMemoryError:
-                order = None  # the direct way needs no further memory
-        if order is None:
+                order = (None, None, None)  # the direct way needs no further memory
+        if order[0] is None:
             vel = sf.interp(x)
-        ctx.save_for_backward(pos)
+        ctx.save_for_backward(pos, *order)
         ctx.sf = sf
-        ctx.order = order
         ctx.field_dtype = field.dtype
         return vel
 
     @staticmethod
     def backward(ctx, g_vel):
-        (pos,) = ctx.saved_tensors
+        pos, *order = ctx.saved_tensors
         sf = ctx.sf
         g_vel = g_vel.contiguous().float()
         want_pos = ctx.needs_input_grad[0]
@@ -783,7 +800,7 @@ class InterpFn(torch.autograd.Function):
         g_field = (torch.empty((sf.ncomp, sf.n[2], sf.n[1], sf.n[0]), dtype=torch.float32,
                                device=pos.device) if want_field else None)
         if want_pos or want_field:
-            if ctx.order is None or not InterpFn._binned_backward(ctx, g_vel, g_pos, g_field):
+            if order[0] is None or not InterpFn._binned_backward(ctx.sf, order, g_vel, g_pos, g_field):
                 ps_interp_backward(sf.coef, sf.n, pos.detach(), g_vel, g_pos, g_field,
                                    scale=sf.scale, L=sf.L)
         if g_field is not None:
@@ -791,11 +808,10 @@ class InterpFn(torch.autograd.Function):
         return g_pos, g_field, None
 
     @staticmethod
-    def _binned_backward(ctx, g_vel, g_pos, g_field) -> bool:
+    def _binned_backward(sf, order, g_vel, g_pos, g_field) -> bool:
         """Both gradients over the particles in bin order; False where the memory for the
         reordered arrays is not there."""
-        sf = ctx.sf
-        perm, offsets, xs = ctx.order
+        perm, offsets, xs = order
         try:
             gs = torch.empty_like(g_vel)
             ps_sorted = torch.empty_like(xs) if g_pos is not None else None
@@ -881,4 +897,6 @@ class BatchPlan:
 
 
 def interp_autograd(pos: torch.Tensor, field: torch.Tensor, L=DEFAULT_L) -> torch.Tensor:
+    if not torch.is_grad_enabled():  # (so that the call knows that no gradient is needed)
+        pos, field = pos.detach(), field.detach()
     return InterpFn.apply(pos, field, L)

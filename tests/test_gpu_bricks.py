@@ -518,3 +518,41 @@ def test_planar_16_bit_halos_in_ragged_boxes(per):
     # below and above the density from which both fields' halos are staged there
     staged, plain = _staged_and_not((30, 21, 17), (8, 8, 8), per, torch.bfloat16, 100)
     assert all(torch.equal(s, p) for s, p in zip(staged, plain))
+
+
+def test_differentiable_call_bins_what_its_gradients_need(monkeypatch):
+    # the tensors kept for the backward pass are saved tensors: hooks see them and they
+    # are freed with the graph
+    n, np_ = (32, 24, 16), 60_000
+    f = torch.from_numpy(synth.random_field(n, ncomp=3, seed=97).astype(np.float32)).to(DEV)
+    x = torch.from_numpy(synth.uniform_particles(np_, seed=98)).to(DEV)
+    monkeypatch.setattr(ps, "_FN_MIN_IN_L2", 0)
+    sorts = []
+    real = ps.bin_particles
+    monkeypatch.setattr(ps, "bin_particles", lambda *a, **k: sorts.append(a) or real(*a, **k))
+    saved = []
+
+    def pack(t):
+        saved.append(t)
+        return t
+
+    xr, fr = x.clone().requires_grad_(), f.clone().requires_grad_()
+    with torch.autograd.graph.saved_tensors_hooks(pack, lambda t: t):
+        u = ps.interp_autograd(xr, fr)
+    assert len(sorts) == 1 and len(saved) == 4  # pos; permutation, offsets, sorted positions
+    assert {t.dtype for t in saved} == {torch.float64, torch.int64, torch.int32}
+    torch.autograd.grad(u, (xr, fr), torch.ones_like(u))
+    with pytest.raises(RuntimeError):  # freed
+        torch.autograd.grad(u, (xr, fr), torch.ones_like(u))
+    # what is asked of the limits: the gradients that the call will need
+    asked = []
+    monkeypatch.setattr(ps, "_fn_binned", lambda n, m, *want: asked.append(want) or False)
+    for a, b, want in ((x, f, (False, False)), (xr, f, (True, False)), (x, fr, (False, True)),
+                       (xr, fr, (True, True))):
+        v = ps.interp_autograd(a, b)
+        assert asked.pop() == want and v.requires_grad == any(want)
+        assert float((v - u).detach().abs().max()) <= 2e-5 * float(u.detach().abs().max())
+        with torch.no_grad():
+            v = ps.interp_autograd(a, b)
+        assert asked.pop() == (False, False) and not v.requires_grad
+    assert len(sorts) == 1

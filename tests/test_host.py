@@ -71,3 +71,15 @@ def test_rows_by_way_of_bin_order_where_it_pays(np_, rows, bricks, pays):
     # few bricks write near one another as it is; few rows gain less
     import paper_2005_13193_gb300 as ps
     assert ps._unsort_pays(np_, rows, bricks) == pays
+
+
+def test_differentiable_calls_binned_where_it_pays():
+    # (position gradient, field gradient) by particles; beyond the L2 from some particles
+    # per brick, within it by what is computed
+    import paper_2005_13193_gb300 as ps
+    for n, np_, want in [((64,) * 3, 700_000, (0, 0, 0, 0)), ((64,) * 3, 900_000, (1, 0, 1, 1)),
+                         ((64,) * 3, 1_100_000, (1, 1, 1, 1)), ((96,) * 3, 5_000_000, (0, 1, 1, 1)),
+                         ((192,) * 3, 300_000, (0, 0, 0, 0)), ((192,) * 3, 400_000, (1, 1, 1, 1)),
+                         ((384,) * 3, 800_000, (0, 0, 0, 0)), ((384,) * 3, 900_000, (1, 1, 1, 1))]:
+        got = [ps._fn_binned(n, np_, p, f) for p, f in ((0, 0), (1, 0), (0, 1), (1, 1))]
+        assert got == [bool(w) for w in want], (n, np_)
