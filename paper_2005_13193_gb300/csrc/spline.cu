@@ -1203,7 +1203,8 @@ ps_status launch_x_node4(const float* src, View sv, NodeT* dst, float* scale4, i
 // nodes) when a thread per value of a row fits a block (64 to 768 values; a
 // stage of 16 rows of 768 takes 55 KB, three of them one block per SM), every
 // streamed pencil holds two chunks and the planes are many or large enough
-// (tune "solve_stream" 0 keeps the three passes).  It needs the unpadded FP32 intermediate in the workspace.
+// (tune "solve_stream" 0 keeps the three passes).  It needs the unpadded FP32
+// intermediate in the workspace.
 bool stream_grid(const ps_grid* g) {
   const int nx = g->n[0];
   return nx >= 64 && nx <= 768 && g->n[1] >= 2 * kSB && g->n[2] >= 2 * kSB;
@@ -1232,8 +1233,28 @@ bool xy_stream_pays(const ps_grid* g, int ncomp) {
   const int64_t fit = (int64_t)sm_count() * std::max(1, 768 / (32 * warps));
   const double waves = (double)((planes + fit - 1) / fit);
   const double row = (0.5 + 0.1 * L) * (nx % L ? 1.7 : 1.0);
-  const double xy = waves * ((double)g->n[1] / kSB + 2) * ((kSB + warps - 1) / warps) * row;
-  return xy < 7.0 + 5e-6 * (double)ncomp * (double)grid_volume(g);
+  const double trips = waves * ((double)g->n[1] / kSB + 2) * ((kSB + warps - 1) / warps);
+  const double M = 1e-6 * ncomp * (double)grid_volume(g);
+  if (trips * row >= 7.0 + 5.0 * M) return false;
+  // Small boxes and rows with cut chunks, nearer: times fitted to 150 grids of 64 to
+  // 768 values per row with one and three components (us; within 12%).  The three
+  // passes have a part per row (the x pass takes a warp per row whatever its length)
+  // and write nodes with less than planar rows.  Both storages of three components
+  // take the same passes, so that they hold the same bits; two where planar rows gain
+  // and nodes lose little.  Kept at three by this part: 124 x 46 x 138 34 -> 39, nodes
+  // 31 -> 39; 188 x 359 x 316 413 -> 432, 358 -> 416; 739 x 48 x 238 187 -> 185, 173 ->
+  // 200; one component of 640 x 64 x 64 29 -> 33, of 767 x 100 x 100 69 -> 79.
+  constexpr double kWhole[7] = {0, 1.06, 0.81, 0.96, 1.35, 1.52, 2.04};  // [chunk / 4]
+  constexpr double kCut[7] = {0, 1.4, 2.2, 1.61, 1.98, 3.03, 3.5};
+  constexpr double kOdd[7] = {0, 1.75, 1.61, 1.48, 1.36, 2.59, 3.66};  // no multiple of 4
+  const double rows = 1e-3 * (double)planes * g->n[1];
+  const bool odd = nx % 4 != 0, wide = nx > 512;
+  const double two = 16.8 + (odd ? 3.6 : 2.1) * M +
+                     (odd ? kOdd : nx % L ? kCut : kWhole)[L / 4] * trips;
+  const double planar = 17.7 + (4.4 + (odd ? 1.0 : 0.0) + (wide ? 1.1 : 0.0)) * M + 0.56 * rows;
+  if (ncomp != 3) return two < 0.9 * planar;
+  const double nodes = 15.7 + (3.5 + (odd ? 1.0 : 0.0) + (wide ? 1.8 : 0.0)) * M + 0.5 * rows;
+  return two < 0.985 * planar && two + (odd ? 0.4 * M : 0.0) < 1.145 * nodes;
 }
 // `rows3` keeps the three passes on rows other than 128, 256 or 512 values.
 bool stream_solve_ok(const ps_grid* g, int ncomp, bool rows3 = false) {

@@ -556,3 +556,11 @@ def test_differentiable_call_bins_what_its_gradients_need(monkeypatch):
             v = ps.interp_autograd(a, b)
         assert asked.pop() == (False, False) and not v.requires_grad
     assert len(sorts) == 1
+
+
+@pytest.mark.parametrize("n", [(168, 33, 200), (236, 100, 150), (226, 200, 150), (225, 200, 150),
+                               (484, 150, 50), (612, 50, 50), (518, 100, 50), (519, 100, 50),
+                               (528, 33, 50), (88, 49, 393)])
+def test_streamed_solve_of_larger_boxes(n):
+    # two passes by the rule for whole chunks, chunks cut short, and odd rows
+    test_streamed_solve_of_any_row(n)
