@@ -120,8 +120,7 @@ __device__ __forceinline__ void scatter_segment(const ScatterArgs& a, int bin, i
       for (int j = 0; j < 4; ++j)
         R.wxy[tid][j] = make_float4(b[0] * by4[j], b[1] * by4[j], b[2] * by4[j], b[3] * by4[j]);
       qbasis(t[2], b);
-      R.bz[tid] = make_float4(__fmul_rn(b[0], kZScale), __fmul_rn(b[2], kZScale),
-                              __fmul_rn(b[1], kZScale), __fmul_rn(b[3], kZScale));
+      R.bz[tid] = make_float4(zscale(b[0]), zscale(b[2]), zscale(b[1]), zscale(b[3]));
       R.gi[tid] = gi;
     }
     __syncthreads();

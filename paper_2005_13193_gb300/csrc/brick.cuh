@@ -152,10 +152,10 @@ __device__ __forceinline__ void fetch_global(float v[16][3], const int cell[3], 
 // their derivatives, with every rounding explicit, so that each instantiation
 // evaluates them identically.  With s = 1 - t: s^3, 4 + t^2 (3t - 6), the same
 // in s, t^3.  The factors 1/6 of the three axes are applied once, on the z
-// weight, as 1/216 times 1 + 1.03e-7: the FP32 solves' pole and gain round so
-// that their coefficients come out 3.4e-8 low per axis (gain / (1 - z)^2).
-// Error of a velocity against 64 bits, 512^3: 6e-8 of the rms; 1.2e-7 with 1/216
-// itself, 7.9e-8 with a rounded 1/6 (3e-8 high) per axis.
+// weight, as the other kernels apply them: 1/6 rounded to FP32 on each axis, in
+// all 8.9e-8 above 1/216.  (The FP32 solves' pole and gain round so that their
+// coefficients come out about as much low, and a velocity's error against 64
+// bits is 7.9e-8 of the rms at 512^3; with 1/216 itself it is 1.2e-7.)
 __device__ __forceinline__ float b_outer(float r) { return __fmul_rn(__fmul_rn(r, r), r); }
 __device__ __forceinline__ float b_inner(float r) {
   return __fmaf_rn(__fmul_rn(r, r), __fmaf_rn(3.f, r, -6.f), 4.f);
@@ -183,16 +183,25 @@ __device__ __forceinline__ void qddbasis(float t, float d[4]) {
   d[2] = __fmaf_rn(-18.f, t, 6.f);
   d[3] = __fmul_rn(6.f, t);
 }
-// 1/216 (see above) times weight k of the z axis alone (a lane's z-row).
-constexpr float kZScale = (float)((1.0 + 1.03e-7) / 216.0);
+// (1/6)^3 as above, in two factors since no single float is that near.
+constexpr float kZScale0 = 0.08f;
+constexpr double kSixth3 = (double)(1.f / 6.f) * (double)(1.f / 6.f) * (double)(1.f / 6.f);
+constexpr float kZScale1 = (float)(kSixth3 / (double)kZScale0);
+static_assert((double)kZScale0 * (double)kZScale1 / kSixth3 - 1.0 < 1e-9 &&
+                  1.0 - (double)kZScale0 * (double)kZScale1 / kSixth3 < 1e-9,
+              "the two factors give (1/6)^3");
+__device__ __forceinline__ float zscale(float b) {
+  return __fmul_rn(__fmul_rn(b, kZScale0), kZScale1);
+}
+// Weight k of the z axis alone (a lane's z-row), scaled.
 __device__ __forceinline__ float zbasis(float t, int k) {
   const float r = (k & 1) ? t : __fsub_rn(1.f, t);  // s for even k, t for odd k
   const bool in = k == 1 || k == 2;
   const float b = __fmaf_rn(__fmul_rn(r, r), in ? __fmaf_rn(3.f, r, -6.f) : r, in ? 4.f : 0.f);
-  return __fmul_rn(b, kZScale);
+  return zscale(b);
 }
 __device__ __forceinline__ float zpick(const float d[4], int k) {
-  return __fmul_rn(pick4(d, k), kZScale);
+  return zscale(pick4(d, k));
 }
 
 // z sum over the quad of one value (xor butterfly: every lane ends with the

@@ -564,3 +564,24 @@ def test_differentiable_call_bins_what_its_gradients_need(monkeypatch):
 def test_streamed_solve_of_larger_boxes(n):
     # two passes by the rule for whole chunks, chunks cut short, and odd rows
     test_streamed_solve_of_any_row(n)
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32])
+def test_bricks_scale_as_the_unbinned_kernels(dtype):
+    # the constant factor of the sums, from a fit against 64 bits of the same
+    # coefficients (rounding noise 1e-7 / sqrt(600,000) = 2e-10): that of 1/6 rounded to
+    # FP32 on each axis, 8.94e-8, in bricks and out of them
+    n, np_ = (32, 24, 40), 200_000
+    field = synth.random_field(n, ncomp=3, seed=110).astype(np.float32)
+    f = torch.from_numpy(field).to(DEV)
+    sf = ps.SplineField.from_field(f, dtype)
+    pos = synth.uniform_particles(np_, seed=111)
+    pg = torch.from_numpy(pos).to(DEV)
+    bins = ps.bin_particles(n, 8, pg)
+    ref = torch.from_numpy(oracle.interp(sf.padded().cpu().numpy().astype(np.float64), pos)).to(DEV)
+
+    def factor(a, b):
+        return float((a.double() * b).sum() / (b * b).sum() - 1)
+
+    direct, binned = factor(sf.interp(pg), ref), factor(sf.interp(pg, bins=bins), ref)
+    assert abs(direct - 8.94e-8) <= 5e-9 and abs(binned - 8.94e-8) <= 5e-9
