@@ -83,8 +83,8 @@ __device__ __forceinline__ void scatter_segment(const ScatterArgs& a, int bin, i
   float4* mine = acc + 2 * lk * a.PS + lj * a.SX + li;  // + the warp's first plane of a stencil
   const float* wz = reinterpret_cast<const float*>(R.bz) + lk;
   const float* wxy = reinterpret_cast<const float*>(R.wxy) + (lane & 15);
-  for (int c0 = lo; c0 < hi; c0 += kScatterThreads) {
-    const int m = min(kScatterThreads, hi - c0);
+  for (unsigned c0 = lo; c0 < (unsigned)hi; c0 += kScatterThreads) {  // (to beyond 2^31)
+    const int m = (int)min((unsigned)kScatterThreads, (unsigned)hi - c0);
     if (tid < m) {
       const int64_t p = a.perm ? a.perm[c0 + tid] : (int64_t)(c0 + tid);
       float4 gi;

@@ -424,7 +424,7 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
   const QGeo<CT> geo(a);
   const GridArgs& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int per_trip = (int)blockDim.x;
+  const unsigned per_trip = blockDim.x;
   const int k = lane & 3, quad = lane >> 2;
   const int64_t np = a.np;
   const Tc* coef = static_cast<const Tc*>(a.coef);
@@ -432,13 +432,15 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
   const Tc* coef2 = second ? static_cast<const Tc*>(a.coef2) : coef;
   const float* scale2 = second ? a.scale2 : a.scale;
 
-  // the first particles' positions are on their way before anything else
-  int c0 = beg + 32 * warp;
+  // the first particles' positions are on their way before anything else (slots
+  // as unsigned: the trip after the last one lies beyond 2^31 in the largest sets)
+  const unsigned last = (unsigned)end;
+  unsigned c0 = (unsigned)beg + 32 * warp;
   int p = 0;
   double x[3] = {0.0, 0.0, 0.0};
-  auto load = [&](int c) {
-    if (c + lane < end) {
-      p = a.perm ? (int)a.perm[c + lane] : c + lane;
+  auto load = [&](unsigned c) {
+    if (c + lane < last) {
+      p = a.perm ? (int)a.perm[c + lane] : (int)(c + lane);
 #pragma unroll
       for (int d = 0; d < 3; ++d) x[d] = a.pos_in[d * np + p];
     }
@@ -492,8 +494,8 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
                        min(geo.Sz - 4, g.n[2] - 1 - P0[2])};
   int stays = 0;
 
-  for (; c0 < end; c0 += per_trip) {
-    const int m = min(32, end - c0);
+  for (; c0 < last; c0 += per_trip) {
+    const int m = (int)min(32u, last - c0);
     const bool v = lane < m;
     // -- 1: location, and the slot among the warp's particles
     const double xp[3] = {x[0], x[1], x[2]};
@@ -663,7 +665,7 @@ __device__ __forceinline__ bool warp_brick(const StagedArgs& a, int bin, int bxi
     // -- 3: lane i finishes particle i
     const float nanf_ = __int_as_float(0x7fc00000);
     if (v && !ok) flag_status(a.status, PS_DEV_NONFINITE_POS, pp);
-    const int oo = a.slot_out ? c0 + lane : pp;  // where the results go
+    const int oo = a.slot_out ? (int)(c0 + lane) : pp;  // where the results go
     if constexpr (MODE <= 1) {
       if (v) {
 #pragma unroll

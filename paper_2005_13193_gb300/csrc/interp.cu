@@ -577,8 +577,8 @@ __device__ __forceinline__ void process_brick(const StagedArgs& a, int beg, int 
   const float nanf_ = __int_as_float(0x7fc00000);
   const HaloGeo<KS> hg(a);
 
-  for (int cb = beg; cb < end; cb += kRecords) {
-    const int m = min(kRecords, end - cb);
+  for (unsigned cb = beg; cb < (unsigned)end; cb += kRecords) {  // (to beyond 2^31)
+    const int m = (int)min((unsigned)kRecords, (unsigned)end - cb);
     // phase A: tasks (particle i, axis d), task = d * m + i
     for (int task = tid; task < 3 * m; task += kThreads) {
       const int d = task < m ? 0 : (task < 2 * m ? 1 : 2), i = task - d * m;
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(64) interp_thread(StagedArgs a) {
   const GridArgs& g = a.g;
   const int64_t np = a.np;
   const float nanf_ = __int_as_float(0x7fc00000);
-  for (int s = beg + threadIdx.x; s < end; s += blockDim.x) {
+  for (unsigned s = beg + threadIdx.x; s < (unsigned)end; s += blockDim.x) {
     const int64_t p = a.perm ? a.perm[s] : (int64_t)s;
     double x[3];
     int cell[3];

@@ -585,3 +585,40 @@ def test_bricks_scale_as_the_unbinned_kernels(dtype):
 
     direct, binned = factor(sf.interp(pg), ref), factor(sf.interp(pg, bins=bins), ref)
     assert abs(direct - 8.94e-8) <= 5e-9 and abs(binned - 8.94e-8) <= 5e-9
+
+
+def test_slots_next_to_2_31():
+    # the last particles of the largest set: the trip after them begins beyond 2^31
+    np_, m, n = 2**31 - 1, 77, (16, 16, 16)
+    if torch.cuda.mem_get_info()[0] < 100e9:
+        pytest.skip("needs 100 GB")
+    f = torch.from_numpy(synth.random_field(n, ncomp=3, seed=120).astype(np.float32)).to(DEV)
+    last = (torch.from_numpy(synth.uniform_particles(m, seed=121)).to(DEV) + TWO_PI) / 2
+    pos = torch.empty((3, np_), dtype=torch.float64, device=DEV)
+    pos[:, np_ - m:] = last
+    offsets = torch.full((9,), np_ - m, dtype=torch.int32, device=DEV)
+    offsets[8] = np_  # all in the last brick
+    small = torch.zeros(9, dtype=torch.int32, device=DEV)
+    small[8] = m
+    buf = torch.empty((3, np_), dtype=torch.float32, device=DEV)
+    for field, dtype, kernel in ((f, torch.float32, -1), (f, ps.F16X4, -1), (f, torch.float32, 2),
+                                 (f[:1].contiguous(), torch.float32, -1)):
+        sf = ps.SplineField.from_field(field, dtype)
+        ref = torch.empty((sf.ncomp, m), device=DEV)
+        ps.ps_tune_set("brick_kernel", kernel)
+        try:
+            ps.ps_interp(sf.coef, n, last, ref, scale=sf.scale, bin_offsets=small, brick=8)
+            ps.ps_interp(sf.coef, n, pos, buf[:sf.ncomp], scale=sf.scale, bin_offsets=offsets,
+                         brick=8)
+        finally:
+            ps.ps_tune_set("brick_kernel", -1)
+        assert torch.equal(buf[:sf.ncomp, np_ - m:], ref)
+    sf = ps.SplineField.from_field(f)
+    out = []
+    for p, o, w in ((last, small, ref := torch.randn((3, m), device=DEV)), (pos, offsets, buf)):
+        buf[:, np_ - m:] = ref
+        g = torch.empty_like(f)
+        ps.ps_interp_backward(sf.coef, n, p, w, None, g, bin_offsets=o, brick=8,
+                              ws=ps.workspace(ps.ps_backward_workspace_size(n, 8)))
+        out.append(g)
+    assert torch.equal(*out)
