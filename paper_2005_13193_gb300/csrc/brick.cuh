@@ -183,25 +183,34 @@ __device__ __forceinline__ void qddbasis(float t, float d[4]) {
   d[2] = __fmaf_rn(-18.f, t, 6.f);
   d[3] = __fmul_rn(6.f, t);
 }
-// (1/6)^3 as above, in two factors since no single float is that near.
-constexpr float kZScale0 = 0.08f;
+// (1/6)^3 as above in two factors, since no single float is that near: the first one
+// short, so that its products with the constants of the derivatives are exact and cost
+// nothing, the second a multiplication.
+constexpr float kZ0 = 1365.f / 2048.f;
 constexpr double kSixth3 = (double)(1.f / 6.f) * (double)(1.f / 6.f) * (double)(1.f / 6.f);
-constexpr float kZScale1 = (float)(kSixth3 / (double)kZScale0);
-static_assert((double)kZScale0 * (double)kZScale1 / kSixth3 - 1.0 < 1e-9 &&
-                  1.0 - (double)kZScale0 * (double)kZScale1 / kSixth3 < 1e-9,
+constexpr float kZ1 = (float)(kSixth3 / (double)kZ0);
+static_assert((double)kZ0 * (double)kZ1 / kSixth3 - 1.0 < 1e-10 &&
+                  1.0 - (double)kZ0 * (double)kZ1 / kSixth3 < 1e-10,
               "the two factors give (1/6)^3");
-__device__ __forceinline__ float zscale(float b) {
-  return __fmul_rn(__fmul_rn(b, kZScale0), kZScale1);
-}
-// Weight k of the z axis alone (a lane's z-row), scaled.
+__device__ __forceinline__ float zscale(float b) { return __fmul_rn(__fmul_rn(b, kZ0), kZ1); }
+// Weight k of the z axis alone (a lane's z-row), scaled, and its first and second
+// derivative: in r = s for even k, t for odd k.
 __device__ __forceinline__ float zbasis(float t, int k) {
-  const float r = (k & 1) ? t : __fsub_rn(1.f, t);  // s for even k, t for odd k
+  const float r = (k & 1) ? t : __fsub_rn(1.f, t);
   const bool in = k == 1 || k == 2;
   const float b = __fmaf_rn(__fmul_rn(r, r), in ? __fmaf_rn(3.f, r, -6.f) : r, in ? 4.f : 0.f);
-  return zscale(b);
+  return zscale(b);  // (with kZ0 in the constants a Heun step took 4% longer)
 }
-__device__ __forceinline__ float zpick(const float d[4], int k) {
-  return zscale(pick4(d, k));
+__device__ __forceinline__ float zdbasis(float t, int k) {
+  const float r = (k & 1) ? t : __fsub_rn(1.f, t);
+  const bool in = k == 1 || k == 2;
+  const float q = __fmaf_rn(in ? 9.f * kZ0 : 3.f * kZ0, r, in ? -12.f * kZ0 : 0.f);
+  return __fmul_rn(__fmul_rn((k & 1) ? r : -r, q), kZ1);
+}
+__device__ __forceinline__ float zddbasis(float t, int k) {
+  const float r = (k & 1) ? t : __fsub_rn(1.f, t);
+  const bool in = k == 1 || k == 2;
+  return __fmul_rn(__fmaf_rn(in ? 18.f * kZ0 : 6.f * kZ0, r, in ? -12.f * kZ0 : 0.f), kZ1);
 }
 
 // z sum over the quad of one value (xor butterfly: every lane ends with the
@@ -224,11 +233,9 @@ __device__ __forceinline__ void quad_sum(const float v[16][3], const float t[3],
   const float bz = zbasis(t[2], k);
   float dbx[4], dby[4], dbz = 0.f;
   if (GRAD) {
-    float d4[4];
     qdbasis(t[0], dbx);
     qdbasis(t[1], dby);
-    qdbasis(t[2], d4);
-    dbz = zpick(d4, k);
+    dbz = zdbasis(t[2], k);
   }
   float A = 0.f, Bx = 0.f, By = 0.f;
   // u and v as packed pairs (two FP32 operations per instruction, each
@@ -279,7 +286,7 @@ __device__ __forceinline__ void quad_sum(const float v[16][3], const float t[3],
 // c], e = xx, yy, zz, xy, xz, yz; every lane of the quad returns them.
 __device__ __forceinline__ void quad_sum_hess(const float v[16][3], const float t[3], int k,
                                               float* out) {
-  float bx[4], by[4], dbx[4], dby[4], ddbx[4], ddby[4], z4[4];
+  float bx[4], by[4], dbx[4], dby[4], ddbx[4], ddby[4];
   qbasis(t[0], bx);
   qbasis(t[1], by);
   qdbasis(t[0], dbx);
@@ -287,10 +294,7 @@ __device__ __forceinline__ void quad_sum_hess(const float v[16][3], const float 
   qddbasis(t[0], ddbx);
   qddbasis(t[1], ddby);
   const float bz = zbasis(t[2], k);
-  qdbasis(t[2], z4);
-  const float dbz = zpick(z4, k);
-  qddbasis(t[2], z4);
-  const float ddbz = zpick(z4, k);
+  const float dbz = zdbasis(t[2], k), ddbz = zddbasis(t[2], k);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     // y sums of the x sums: A = by s0, Bx = by s1, By = dby s0, Cxx = by s2,
