@@ -1313,22 +1313,24 @@ extern "C" ps_status ps_interp_backward_binned(
 
 // Bricks whose halos are a multiple of four rows high bring further rows into
 // shared memory (quad.cu); with few particles each, the second derivatives and the
-// acceleration are faster unbinned: 128^3, second derivatives, staged / unbinned,
-// us: bricks of 8 x 1 x 8 with 4.6 particles FP32 nodes 86 / 32, planar 89 / 29,
-// planar FP16 99 / 33; 8 x 5 x 8 with 23 particles 37 / 33, 39 / 28, 104 / 35; 4 x 9
-// x 4 with 24, coefficients in the L2, 80 / 70, 83 / 60, 218 / 71; 256^3, beyond
-// the L2, 8 x 1 x 8 with 4, 753 / 208, 746 / 212, 818 / 257, with 8, 370 / 192,
-// 380 / 193 (4 x 9 x 4).
+// acceleration are faster unbinned.  Particles per brick, staged / unbinned, us,
+// bricks of 4 x 9 x 4.  128^3, coefficients in the L2, second derivatives: FP32 nodes
+// 24 80 / 70, 32 87 / 92; planar 32 91 / 84, 48 99 / 129; planar FP16 64 268 / 206;
+// acceleration from two fields: 8 64 / 48, 16 74 / 83; 24 87 / 87.  256^3, second
+// derivatives: 16 474 / 358, 492 / 354; at particles in no order (perm given), whose
+// unbinned stencils come from DRAM, 8 428 / 343, 435 / 639; acceleration: 8 464 / 305,
+// 16 520 / 582; 16 515 / 463; in no order 4 504 / 374, 2 401 / 402.
 static bool unbinned_pays(const ps_grid* grid, ps_dtype coef_t, const int32_t brick[3],
-                          int64_t np) {
+                          int64_t np, const int64_t* perm, bool accel) {
   StagedArgs a{};
   size_t smem;
   if ((brick[1] + 3) % 4 || fill_staged(grid, coef_t, brick, 0, false, &a, &smem))
     return false;  // (what the staged form refuses stays refused)
-  const double nodes = (double)a.S[0] * a.S[1] * a.S[2];
-  const double bytes = (double)grid_volume(grid) * 3.0 * (double)dtype_size(coef_t);
-  const double least = bytes <= 64e6 ? 30.0 : 12.0;  // per 11^3 nodes
-  return (double)np * 1331.0 < least * nodes * (double)a.b.nbins;
+  const bool nodes = coef_t == PS_F32X4 || coef_t == PS_BF16X4 || coef_t == PS_F16X4;
+  const bool in_l2 = (double)grid_volume(grid) * (double)dtype_size(coef_t) * (nodes ? 1 : 3) < 64e6;
+  double least = in_l2 ? (nodes ? 64.0 : 80.0) : !perm ? 36.0 : nodes ? 20.0 : 10.0;
+  if (accel) least *= 0.5;  // per 11^3 halo nodes
+  return (double)np * 1331.0 < least * (double)a.S[0] * a.S[1] * a.S[2] * (double)a.b.nbins;
 }
 
 // Brick-staged form of the second derivatives (mode 3) or the Lagrangian
@@ -1385,7 +1387,8 @@ extern "C" ps_status ps_interp_hessian_ws(const ps_grid* grid, int ncomp, ps_dty
   if (perm && !bin_offsets) return fail(PS_ERR_INVALID_ARG, "perm needs bin_offsets");
   if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
   cudaStream_t st = as_stream(stream);
-  if (bin_offsets && ncomp == 3 && coef_t != PS_F64 && !unbinned_pays(grid, coef_t, brick, np)) {
+  if (bin_offsets && ncomp == 3 && coef_t != PS_F64 &&
+      !unbinned_pays(grid, coef_t, brick, np, perm, false)) {
     return staged_extra(grid, coef_t, coef, scale, nullptr, nullptr, 0.0, np, pos, perm,
                         bin_offsets, brick, hess, nullptr, result_rows(perm, np, 18, ws, ws_bytes),
                         status, 3, st);
@@ -1437,7 +1440,8 @@ extern "C" ps_status ps_lagrangian_accel_ws(const ps_grid* grid, ps_dtype coef_t
   if (bin_offsets && !brick) return fail(PS_ERR_INVALID_ARG, "bin_offsets needs brick");
   cudaStream_t st = as_stream(stream);
   const double inv_dt = coef_np1 ? 1.0 / dt_field : 0.0;
-  if (bin_offsets && coef_t != PS_F64 && !unbinned_pays(grid, coef_t, brick, np)) {
+  if (bin_offsets && coef_t != PS_F64 &&
+      !unbinned_pays(grid, coef_t, brick, np, perm, true)) {
     return staged_extra(grid, coef_t, coef_n, scale_n, coef_np1, scale_np1, inv_dt, np, pos, perm,
                       bin_offsets, brick, acc, vel, result_rows(perm, np, vel ? 6 : 3, ws, ws_bytes),
                       status, 4, st);
