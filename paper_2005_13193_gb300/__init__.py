@@ -509,22 +509,24 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 # half of the L2, scattered 4-byte stores reach DRAM one by one.  Stored directly / by
 # way of bin order, us, 96^3: 46 MiB 123 / 160, 69 MiB 190 / 221, 92 MiB 336 / 309, 183
 # MiB 701 / 607; 256^3: 183 MiB 1668 / 582, 549 MiB 5695 / 1490.  Particles of a bin are
-# in about their own order, so that bricks that all run at once (up to 8 blocks on each
-# of 152 SMs) write near one another: 64^3, 512 bricks, 183 MiB 456 / 554, 275 MiB 767 /
-# 739; 72^3, 729, 549 MiB 1736 / 2020, 824 MiB 3322 / 2555.  Fewer than four rows are put
+# in about their own order, so that bricks that all run at once (up to 8 blocks of 64
+# threads on each of 152 SMs; up to 4 of 128, less so) write near one another: 64^3, 512
+# bricks, 183 MiB 456 / 554, 275 MiB 767 / 739; 72^3, 729, 275 MiB 708 / 806, 549 MiB
+# 1736 / 2020, 824 MiB 3322 / 2555.  Fewer than four rows are put
 # in place by words and gain less: three of 12 M particles, 96^3 1025 / 1150, 112^3 1129 /
 # 1196, 128^3 1281 / 1230, 160^3 1585 / 1320.
 _UNSORT_BYTES = 88 << 20
 _UNSORT_AT_ONCE = 8 * 152
-_UNSORT_BYTES_AT_ONCE = 600 << 20
+_UNSORT_BYTES_AT_ONCE = 600 << 20  # (of blocks of 64 threads; of 128: 256 MiB)
 _UNSORT_BRICKS_OF_FEW_ROWS = 3000
 
 
 def _unsort_pays(np_: int, rows: int, bricks: int) -> bool:
     if rows < 4 and bricks < _UNSORT_BRICKS_OF_FEW_ROWS:
         return False
-    return 4 * rows * np_ >= (_UNSORT_BYTES_AT_ONCE if bricks <= _UNSORT_AT_ONCE
-                              else _UNSORT_BYTES)
+    least = (_UNSORT_BYTES if bricks > _UNSORT_AT_ONCE else
+             _UNSORT_BYTES_AT_ONCE if 2 * bricks > _UNSORT_AT_ONCE else 256 << 20)
+    return 4 * rows * np_ >= least
 
 
 def _of_stream(stream):
@@ -749,7 +751,9 @@ _FN_MIN_PER_BRICK = 8
 
 
 def _fn_binned(n, np_: int, pos_grad: bool, field_grad: bool) -> bool:
-    if 12 * math.prod(n) > _FN_L2_BYTES:
+    if 12 * math.prod(n) > 2 * _FN_L2_BYTES:
+        least, most = 0, 2**31 - 1
+    elif 12 * math.prod(n) > _FN_L2_BYTES:
         least, most = _FN_MIN_BEYOND, 2**31 - 1
     elif field_grad:
         least, most = _FN_MIN_IN_L2, 2**31 - 1

@@ -65,7 +65,7 @@ def test_tracker_rebin_modes(monkeypatch):
 
 @pytest.mark.parametrize("np_,rows,bricks,pays", [
     (2_000_000, 12, 4096, True), (1_000_000, 18, 4096, False), (4_000_000, 12, 512, False),
-    (4_000_000, 18, 729, False), (12_000_000, 18, 512, True), (2_000_000, 18, 1331, True),
+    (4_000_000, 18, 729, False), (4_000_000, 18, 512, True), (12_000_000, 18, 512, True), (2_000_000, 18, 1331, True),
     (12_000_000, 3, 2744, False), (12_000_000, 3, 4096, True), (4_000_000, 3, 4096, False)])
 def test_rows_by_way_of_bin_order_where_it_pays(np_, rows, bricks, pays):
     # few bricks write near one another as it is; few rows gain less
@@ -80,6 +80,6 @@ def test_differentiable_calls_binned_where_it_pays():
     for n, np_, want in [((64,) * 3, 700_000, (0, 0, 0, 0)), ((64,) * 3, 900_000, (1, 0, 1, 1)),
                          ((64,) * 3, 1_100_000, (1, 1, 1, 1)), ((96,) * 3, 5_000_000, (0, 1, 1, 1)),
                          ((192,) * 3, 300_000, (0, 0, 0, 0)), ((192,) * 3, 400_000, (1, 1, 1, 1)),
-                         ((384,) * 3, 800_000, (0, 0, 0, 0)), ((384,) * 3, 900_000, (1, 1, 1, 1))]:
+                         ((256,) * 3, 262_144, (1, 1, 1, 1)), ((384,) * 3, 800_000, (0, 0, 0, 0)), ((384,) * 3, 900_000, (1, 1, 1, 1))]:
         got = [ps._fn_binned(n, np_, p, f) for p, f in ((0, 0), (1, 0), (0, 1), (1, 1))]
         assert got == [bool(w) for w in want], (n, np_)
