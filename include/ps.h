@@ -126,7 +126,9 @@ int64_t ps_coef_row_pitch(int nx, ps_dtype coef_t);
  *     brick, 8 lanes per particle, phases separated by block barriers (2: one
  *     thread per particle).
  *  "brick_min_stage" in [0, 2^20] (default 8): bricks holding fewer particles
- *     skip the halo staging and gather their stencils from global memory.
+ *     skip the halo staging and gather their stencils from global memory (planar
+ *     16-bit coefficients in bricks that do not tile the grid in 8 values along x:
+ *     at least a particle per four halo rows).
  *  "node_tma" 0 or 1 (default 1): halos of node coefficients by tensor copy.
  *  "solve_xw" 0, 8, 16 or 32 (0 = default 16): x extent of a block of the
  *     strided spline passes.

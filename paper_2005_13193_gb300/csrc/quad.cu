@@ -118,6 +118,13 @@ template <typename Tc>
 void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
   constexpr bool n16 = IsNode16<Tc>::value, planar = IsPlanar<Tc>::value;
   halo_plane(a, n16 ? 2 : planar ? 4 : 1, n16 || planar);
+  // planar 16-bit halos that do not come in whole vectors are widened value by value,
+  // 16 or 32 lanes a row: staged from a particle per four rows on.  128^3 boxes, FP16,
+  // interpolation staged / from global memory, us: bricks of 8 x 5 x 8 with 9 particles
+  // 68 / 25, 17 85 / 39, 35 89 / 64; 4 x 4 x 4 with 12 255 / 110; 12^3 with 61 56 / 37,
+  // 122 60 / 66; 250 x 200 x 150, 8^3 with 12 220 / 103, 24 243 / 205, 48 265 / 442.
+  if (IsQuant<Tc>::value && !n16 && !a->vec)
+    a->min_stage = std::max(a->min_stage, a->S[1] * a->S[2] * (a->S[0] > 16 ? 2 : 1) / 4);
   a->half_dt = 0.5 * a->dt;
   for (int d = 0; d < 3; ++d) a->ih32[d] = a->g.inv_h[d] * 4294967296.0;
   a->wait_probe = tuning().wait_probe;

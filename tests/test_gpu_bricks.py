@@ -622,3 +622,10 @@ def test_slots_next_to_2_31():
                               ws=ps.workspace(ps.ps_backward_workspace_size(n, 8)))
         out.append(g)
     assert torch.equal(*out)
+
+
+@pytest.mark.parametrize("brick,per", [((8, 5, 8), 20), ((8, 5, 8), 24), ((4, 4, 4), 11),
+                                       ((4, 4, 4), 14), ((20, 3, 3), 17), ((20, 3, 3), 20)])
+def test_planar_16_bit_halos_from_a_particle_per_four_rows(brick, per):
+    staged, plain = _staged_and_not((26, 22, 18), brick, per, torch.float16, 130)
+    assert all(torch.equal(s, p) for s, p in zip(staged, plain))
