@@ -1,4 +1,5 @@
 // Host-side plumbing of the C ABI: error strings, status words, validation.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -96,10 +97,13 @@ Tuning& tuning() {
 }
 
 int sm_count() {
+  static std::atomic<int> known[64];  // per device, 0: not asked yet
   int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 1;
+  if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
     return 1;
+  if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
   return n;
 }
 
