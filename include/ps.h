@@ -129,7 +129,8 @@ int64_t ps_coef_row_pitch(int nx, ps_dtype coef_t);
  *     skip the halo staging and gather their stencils from global memory (planar
  *     16-bit coefficients in bricks that do not tile the grid in 8 values along x:
  *     at least a particle per four halo rows).
- *  "node_tma" 0 or 1 (default 1): halos of node coefficients by tensor copy.
+ *  "node_tma" 0 or 1 (default 1): halos of node and planar FP32 coefficients by
+ *     tensor copy.
  *  "solve_xw" 0, 8, 16 or 32 (0 = default 16): x extent of a block of the
  *     strided spline passes.
  *  "solve_stream" 0 or 1 (default 1): FP32 solves in two streamed passes

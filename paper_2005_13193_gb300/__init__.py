@@ -334,8 +334,9 @@ def ps_interp_backward(coef: torch.Tensor, n, pos: torch.Tensor, g_vel: torch.Te
                        bin_offsets: Optional[torch.Tensor] = None, brick=None,
                        ws: Optional[torch.Tensor] = None):
     """Adjoint of ps_interp and of the coefficient solve.  With bin_offsets (and brick,
-    perm as for ps_interp) both gradients are formed brick by brick; ws
-    (ps_backward_workspace_size) holds the bricks' sums."""
+    perm as for ps_interp) the field gradient's scatter is summed brick by brick (ws,
+    ps_backward_workspace_size, holds the bricks' sums) and the position gradients are
+    gathered in bin order."""
     _check_coef_shape(coef, n)
     ncomp = _ncomp_of(coef)
     np_ = pos.shape[1]

@@ -7,8 +7,7 @@ per particle but hold fewer blocks per SM; the best shape depends on the grid,
 the particle density and the coefficient type, so it is measured, on the
 caller's own data, by timing the real step for each candidate.
 
-`tune_tracker` picks (brick kernel, brick shape; for three components the
-kernels 0 and 5 are the same) for single-field Heun steps
+`tune_tracker` picks (brick kernel, brick shape) for single-field Heun steps
 and applies the kernel choice with ps_tune_set; `tune_batch` picks the brick
 shape of a many-field plan.  Both can write the choice to a small text cache,
 one "key values" pair per line, which ps_batch_plan reads back ("brick bx by
@@ -28,7 +27,8 @@ from . import BatchPlan, PSError, SplineField, Tracker, ps_tune_get, ps_tune_set
 # within 32 nodes
 CANDIDATES = ((8, 8, 8), (8, 8, 4), (8, 4, 4), (4, 4, 4), (8, 8, 16), (16, 8, 8),
               (16, 8, 4), (16, 16, 8))
-KERNELS = (0, 2, 5)
+# kernels of a three-component step (5 and -1 name the same one as 0)
+KERNELS = (0, 2)
 
 
 def _time_ms(fn, warmup: int, reps: int, stream=None) -> float:

@@ -1,6 +1,6 @@
 // Adjoint of the binned interpolation (Sec. 2.2, Operations 2 and 3 transposed):
-// the cotangent's scatter onto the field by bricks of cells, and the position
-// gradient from each brick's staged halo.
+// the cotangent's scatter onto the field by bricks of cells.  (The position
+// gradients are the unbinned kernel's, over particles in bin order: interp.cu.)
 //
 // The scatter adds g_vel * basis weights to 64 nodes of three components per
 // particle.  Straight to global memory that is 192 atomics per particle, 8

@@ -1,9 +1,9 @@
 // Many periodic fields of uneven sizes and their particle sets advanced
 // together: one bin sort over the concatenated particles of all fields (global
 // bin = first bin of the field + bin in the field) and one pass over the
-// bricks of all fields per Heun step.  By default all steps run in one
-// cooperative persistent launch (the sort's phases and the brick pass
-// separated by grid-wide barriers); otherwise a launch per phase and step.
+// bricks of all fields per Heun step, in a launch per phase and step or (tune
+// "batch_persistent", graphs of very many steps) in one cooperative launch of all
+// steps, whose phases are separated by grid-wide barriers.
 // With use_graph the solves of all fields and the steps are captured once in a
 // CUDA graph and replayed.  Not part of the paper's method: a way of running
 // many of its problems at once on one device.

@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(kThreads, 8) batch_persistent(const __grid_con
 }  // namespace
 
 // ---------------------------------------------------------------- batch ----
-// Helpers of the many-field form (batch.cu); StagedArgs stays private to this
-// file and travels as opaque bytes.
+// Helpers of the many-field form (batch.cu, where a field's StagedArgs travel as
+// opaque bytes).
 
 size_t staged_args_size() { return sizeof(StagedArgs); }
 

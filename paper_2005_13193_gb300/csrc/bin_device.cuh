@@ -1,5 +1,5 @@
 // Device pieces of the bin sort shared by the sort kernels (bin.cu) and the
-// persistent many-field kernel (interp.cu): the bin of a position, the
+// persistent many-field kernel (batch_step.cu): the bin of a position, the
 // counting pass over many fields, the three phases of the exclusive scan of
 // the bin counters (tiles of kScanTile counters, blocks of any multiple of 32
 // threads), and the scatter into bin order.  Internal to libps.

@@ -74,7 +74,7 @@ struct Tuning {
   int brick_kernel = -1;      // 2 thread per particle; else (-1, 0, 5) quad
                               // (one component: phased)
   int brick_min_stage = 8;    // per-brick kernel: fewer particles skip the halo
-  int node_tma = 1;           // PS_F32X4 halos by tensor copy
+  int node_tma = 1;           // node and planar FP32 halos by tensor copy
   int solve_xw = 0;           // x extent of a strided-pass block (0: default)
   int solve_stream = 1;       // FP32 solves in two streamed passes (y-x, then z)
   int solve_zt = 0;           // columns per block of the streamed z pass (0: default)
@@ -245,27 +245,6 @@ __device__ __forceinline__ int brick_coord(const GridArgs& g, const BrickArgs& b
 // Bin of brick (bx, by, bz), x fastest; -1 if a coordinate is -1.
 __device__ __forceinline__ int bin_of_coords(const BrickArgs& b, int bx, int by, int bz) {
   return (bx | by | bz) < 0 ? -1 : (bz * b.nb[1] + by) * b.nb[0] + bx;
-}
-
-// Counting step of the bin sort for the particles a warp holds: lane l has
-// particle p (valid) whose bin is key (-1: position rejected; it is counted
-// in bin 0 and reported, as the counting pass does).  The bin goes to
-// bin_of[p]; lanes with equal keys add to the bin's counter with one atomic
-// whose result is not waited for (the scatter takes the ranks later).  All
-// 32 lanes must call.
-__device__ __forceinline__ void count_into_bin(int32_t* counts, int32_t* bin_of,
-                                               int32_t* status, bool valid, int64_t p,
-                                               int key, int key_base = 0) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  if (valid && key < 0) {
-    flag_status(status, PS_DEV_NONFINITE_POS, p);
-    key = 0;
-  }
-  const int k = valid ? key : -1 - lane;  // unique per lane when invalid
-  const unsigned peers = __match_any_sync(FULL, k);
-  if (valid && lane == __ffs(peers) - 1) atomicAdd(&counts[k], __popc(peers));
-  if (valid) bin_of[p] = key_base + k;
 }
 
 // FP64 variant for FP64 coefficients: t = s - floor(s) in FP64.

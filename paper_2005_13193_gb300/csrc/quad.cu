@@ -1,6 +1,6 @@
 // Brick-staged interpolation (Sec. 2.2, Operations 2 and 3) and the fused
 // second-order Runge-Kutta particle advance (Sec. 2.1, Sec. 4.3) for three
-// components: one block of two warps per brick of cells (brick.cuh).
+// components: one block of two or four warps per brick of cells (brick.cuh).
 //
 // What bounds it (512^3, 64 particles per brick, ncu at the same density): the
 // latency of each warp's chain at 13 warps per SM (41-52% of the issue slots,

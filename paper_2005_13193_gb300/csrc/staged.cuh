@@ -20,7 +20,7 @@ struct StagedArgs {
   int PS;       // plane stride, >= SX * S[1] (phased kernel: = 4 mod 8; quad.cu)
   int vec;      // 1: halo rows are whole 16-byte vectors inside the array
   int min_stage;  // bricks with fewer particles gather from global memory
-  int tma;        // 1: the node halo is one tensor copy described by tmap
+  int tma;        // 1: the halo is one tensor copy described by tmap
                   // (2: the second field's too, by tmap2)
   int two;        // 1: the second field's halo is staged beside the first
   int chunked;    // 1: bins are runs of particles (sparse field): no halo
@@ -55,12 +55,13 @@ struct StagedArgs {
   // (sign cleared) only if |x n/L| < 2^30, read without an FP64 operation
   int xguard_hi[3];
   int slot_out;       // 1: results at the particle's slot in bin order, not at perm[slot]
-  CUtensorMap tmap;   // node halo box (valid when tma == 1)
-  CUtensorMap tmap2;  // 16-bit nodes: the box of the halo rows' scales
+  CUtensorMap tmap;   // the halo's box (valid when tma > 0)
+  CUtensorMap tmap2;  // 16-bit nodes: the box of the halo rows' scales; others, with
+                      // tma == 2: the second field's halo
 };
 
-// Tensor map of the node halo box (4 floats x a.SX nodes x S[1] rows x S[2]
-// planes) over a node coefficient array (interp.cu).
+// Tensor map of the halo box (rows of a.SX nodes or planar floats, a.PS / a.SX rows
+// per plane, S[2] planes) over a node or planar FP32 coefficient array (interp.cu).
 bool encode_node_halo_map(StagedArgs* a, ps_dtype coef_t);
 
 // Geometry of the brick-staged kernels (interp.cu): extents, plain-load layout,
