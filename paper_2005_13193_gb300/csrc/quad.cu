@@ -3,22 +3,22 @@
 // components: one block of two or four warps per brick of cells (brick.cuh).
 //
 // What bounds it (512^3, 64 particles per brick, ncu at the same density): the
-// latency of each warp's chain at 13 warps per SM (41-52% of the issue slots,
-// 48-62% of the shared-memory wavefronts; HBM 24-39%).  Eight blocks of 27 KB
+// latency of each warp's chain at 13 warps per SM (37-49% of the issue slots,
+// 44-61% of the shared-memory wavefronts; HBM 24-39%).  Eight blocks of 27 KB
 // of halo and 64 threads of at most 128 registers fill both the shared memory
 // and the register file.  Against the form with (particle, axis) tasks and
-// block barriers between its phases: 32 warp instructions per particle instead
-// of 61 (interpolation) and 66 instead of 104 (Heun step), 12 and 16
+// block barriers between its phases: 29 warp instructions per particle instead
+// of 61 (interpolation) and 62 instead of 104 (Heun step), 12 and 16
 // shared-memory wavefronts instead of 13 and 30.  Measured there, one launch,
-// before -> after: interpolation 1427 -> 1013 us, gradient tensor 1938 ->
-// 1352, second derivatives 2345 -> 1812, acceleration from two fields 3007 ->
-// 2839, re-binned Heun step with its sort 2596 -> 2195.  256^3 with 1.4 M
+// before -> after: interpolation 1427 -> 1020 us, gradient tensor 1938 ->
+// 1339, second derivatives 2345 -> 1792, acceleration from two fields 3007 ->
+// 2655, re-binned Heun step with its sort 2596 -> 2195.  256^3 with 1.4 M
 // particles and FP16 nodes: Heun step with its sort 328 -> 254.  Planar FP32,
 // 256^3 with 4 M particles, halo by a planar tensor copy and gathered as three
 // planes instead of loaded and interleaved: interpolation 419 -> 257, Heun step
 // with its sort 683 -> 501; two snapshots of 180 x 150 x 132 with 500,000
 // particles, the second halo staged beside the first instead of gathered from
-// global memory: two steps 531 -> 316.  Tried and not faster: three warps of 24
+// global memory: two steps 531 -> 322.  Tried and not faster: three warps of 24
 // particles (spills at 96 registers: 1503), two bricks along x per block
 // (1055), blocks that walk over the bricks with the next bounds and positions
 // loaded ahead (1024, Heun step 2516).
