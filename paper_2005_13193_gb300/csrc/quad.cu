@@ -128,6 +128,11 @@ void setup_t(StagedArgs* a, bool second, size_t* smem, int* ct) {
   a->half_dt = 0.5 * a->dt;
   for (int d = 0; d < 3; ++d) a->ih32[d] = a->g.inv_h[d] * 4294967296.0;
   a->wait_probe = tuning().wait_probe;
+  if (halo_bytes<Tc>(a->S[2], a->S[1], a->PS) > 226 * 1024) {
+    // the largest halos: without the further rows and the padding
+    a->SX = (a->S[0] + (planar ? 3 : n16 ? 1 : 0)) & ~(planar ? 3 : n16 ? 1 : 0);
+    a->PS = a->SX * a->S[1];
+  }
   *ct = a->S[0] == 11 && a->S[1] == 11 && a->S[2] == 11 && a->SX == (n16 || planar ? 12 : 14)
             ? a->SX
             : 0;

@@ -622,10 +622,20 @@ def test_slots_next_to_2_31():
                               ws=ps.workspace(ps.ps_backward_workspace_size(n, 8)))
         out.append(g)
     assert torch.equal(*out)
+    del pos, buf, w
+    torch.cuda.empty_cache()
 
 
 @pytest.mark.parametrize("brick,per", [((8, 5, 8), 20), ((8, 5, 8), 24), ((4, 4, 4), 11),
                                        ((4, 4, 4), 14), ((20, 3, 3), 17), ((20, 3, 3), 20)])
 def test_planar_16_bit_halos_from_a_particle_per_four_rows(brick, per):
     staged, plain = _staged_and_not((26, 22, 18), brick, per, torch.float16, 130)
+    assert all(torch.equal(s, p) for s, p in zip(staged, plain))
+
+
+@pytest.mark.parametrize("dtype", [ps.F32X4, torch.float32, torch.bfloat16, ps.F16X4])
+@pytest.mark.parametrize("n,brick", [((32, 40, 34), (16, 16, 32)), ((32, 20, 34), (29, 17, 17))])
+def test_largest_halos(n, brick, dtype):
+    # nearly all of the shared memory: staged without padding where that alone fits
+    staged, plain = _staged_and_not(n, brick, 300, dtype, 140)
     assert all(torch.equal(s, p) for s, p in zip(staged, plain))
